@@ -9,8 +9,9 @@
 //              integers below 2^53 are order independent).
 //  FINALIZE    M1 = C/T, M2 = (alpha0+1) P/S2 - alpha0 M1 M1^T; top-D
 //              eigenpairs by randomised subspace iteration (FP32 products,
-//              FP64 CholeskyQR2), FP64 Rayleigh-Ritz with a cyclic Jacobi
-//              eigensolver in one block, W = U Lambda^-1/2, m1 = W^T M1.
+//              FP64 CholeskyQR), FP64 Rayleigh-Ritz with a cyclic Jacobi
+//              eigensolver over the grid, W = U Lambda^-1/2, m1 = W^T M1.
+//              FP64 products run on the tensor cores in exact slices (gemm64.cuh).
 //  unwhiten    mu_i = ||phi_i||^2 W (W^T W)^-1 phi_i, alpha_i ~ ||phi_i||^-6,
 //              clip at 0, normalise (FP64).
 #include <algorithm>
@@ -20,6 +21,7 @@
 #include <functional>
 #include <vector>
 
+#include "gemm64.cuh"
 #include "scan.cuh"
 #include "tlda_internal.h"
 
@@ -30,6 +32,8 @@ namespace {
 constexpr int kMaxFitV = 65536;
 
 // ------------------------------------------------------------------ scan + pairs
+// One warp per document.  Only the pairs on or below the diagonal of P are
+// added (the words ascend within a document); k_m2_mirror fills in the rest.
 __global__ void k_fit_accumulate(tlda_csr b, int V, double *P, unsigned long long *C,
                                  unsigned long long *TS, int *err) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -42,26 +46,33 @@ __global__ void k_fit_accumulate(tlda_csr b, int V, double *P, unsigned long lon
   const int u = hi - lo;
   bool bad = false;
   long long L = 0;
-  for (int j = lo; j < hi; ++j) {
+  for (int j = lo + lane; j < hi; j += 32) {
     const int m = b.indices[j], f = b.counts[j];
-    if (m < 0 || m >= V || f <= 0 || (j > lo && m <= b.indices[j - 1])) {
-      bad = true;
-      continue;
-    }
-    L += f;
+    if (m < 0 || m >= V || f <= 0 || (j > lo && m <= b.indices[j - 1])) bad = true;
+    else L += f;
   }
-  if (bad) {
+  if (__any_sync(0xffffffffu, bad)) {
     if (lane == 0) atomicOr(err, 1);
     return;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   if (lane == 0) {
     atomicAdd(TS + 0, (unsigned long long)L);
     atomicAdd(TS + 1, (unsigned long long)(L * (L - 1)));
     atomicAdd(TS + 2, (unsigned long long)(L * (L - 1) * (L - 2)));
   }
   for (int j = lo + lane; j < hi; j += 32) atomicAdd(C + b.indices[j], (unsigned long long)b.counts[j]);
-  for (int q = lane; q < u * u; q += 32) {
-    const int x = q / u, y = q % u;
+  // pair t of the lower triangle by rows: row x holds t = x(x+1)/2 .. x(x+1)/2 + x
+  const long long np = (long long)u * (u + 1) / 2;
+  int x = 0;
+  long long row = 0;  // first pair of row x
+  for (long long t = lane; t < np; t += 32) {
+    while (t > row + x) {
+      row += x + 1;
+      ++x;
+    }
+    const int y = (int)(t - row);
     const int ma = b.indices[lo + x], mb = b.indices[lo + y];
     const long long fa = b.counts[lo + x], fb = b.counts[lo + y];
     const long long v = fa * fb - (x == y ? fa : 0);
@@ -69,96 +80,259 @@ __global__ void k_fit_accumulate(tlda_csr b, int V, double *P, unsigned long lon
   }
 }
 
-// ------------------------------------------------------------------ generic GEMMs
-// C[M x N] = A[M x Kd] B[Kd x N] (row-major), 64 x 64 tiles, 4 x 4 per thread.
-template <class T>
-__global__ void __launch_bounds__(256) k_gemm_nn(const T *A, int lda, const T *B, int ldb, T *C, int ldc,
-                                                 int M, int N, int Kd) {
-  __shared__ T As[16][64 + 1];
-  __shared__ T Bs[16][64];
+// ------------------------------------------------------------------ products
+// FP32: C[M x N] = A[M x Kd] B[Kd x N] (row-major, any pitch), FFMA.  Tiles of
+// 128 rows x 16 TN columns, 8 x TN outputs a thread, so that N = 66 or 116
+// columns (D + 16) waste at most 15 of a tile; the next 16 terms are in flight
+// in registers while a slab is used.  Few row tiles leave SMs idle, so the terms
+// are split over blockIdx.z into partial products (sgemm_splits), summed in
+// order by k_sgemm_sum.
+template <int TN>
+__global__ void __launch_bounds__(256) k_sgemm(const float *__restrict__ A, int lda, const float *__restrict__ B, int ldb,
+                                               float *__restrict__ C, int ldc, int M, int N, int Kd, int chunk,
+                                               long long cstride) {
+  constexpr int BN = 16 * TN, BK = 16, NB = (BK * BN + 255) / 256;
+  __shared__ __align__(16) float As[2][BK][128 + 4];
+  __shared__ __align__(16) float Bs[2][BK][BN];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  T acc[4][4];
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-  for (int k0 = 0; k0 < Kd; k0 += 16) {
-    for (int e = tid; e < 16 * 64; e += 256) {
-      const int r = e >> 4, kk = e & 15;  // A: 64 rows x 16
-      const int gm = m0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < M && gk < Kd) ? A[(long long)gm * lda + gk] : T(0);
-      const int kb = e >> 6, nn = e & 63;  // B: 16 x 64
-      const int gkb = k0 + kb, gn = n0 + nn;
-      Bs[kb][nn] = (gkb < Kd && gn < N) ? B[(long long)gkb * ldb + gn] : T(0);
-    }
-    __syncthreads();
+  const int m0 = blockIdx.y * 128, n0 = blockIdx.x * BN;
+  const int kb = blockIdx.z * chunk, ke = min(Kd, kb + chunk);
+  float acc[8][TN], ra[8], rb[NB];
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      T ar[4], br[4];
-      for (int i = 0; i < 4; ++i) ar[i] = As[kk][ty * 4 + i];
-      for (int j = 0; j < 4; ++j) br[j] = Bs[kk][tx * 4 + j];
-      for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) acc[i][j] += ar[i] * br[j];
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = tid + i * 256, k = k0 + (e & 15), r = m0 + (e >> 4);
+      ra[i] = (k < ke && r < M) ? __ldg(A + (long long)r * lda + k) : 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + i * 256, k = k0 + e / BN, c = n0 + e % BN;
+      rb[i] = (e < BK * BN && k < ke && c < N) ? __ldg(B + (long long)k * ldb + c) : 0.f;
+    }
+  };
+  auto file = [&](int p) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = tid + i * 256;
+      As[p][e & 15][e >> 4] = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + i * 256;
+      if (e < BK * BN) Bs[p][e / BN][e % BN] = rb[i];
+    }
+  };
+  fetch(kb);
+  file(0);
+  __syncthreads();
+  int p = 0;
+  for (int k0 = kb; k0 < ke; k0 += BK, p ^= 1) {
+    const bool more = k0 + BK < ke;
+    if (more) fetch(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4 *>(&As[p][kk][ty * 8]);
+      const float4 a1 = *reinterpret_cast<const float4 *>(&As[p][kk][ty * 8 + 4]);
+      const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      float br[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) br[j] = Bs[p][kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
+    }
+    if (more) file(p ^ 1);
     __syncthreads();
   }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-      if (gm < M && gn < N) C[(long long)gm * ldc + gn] = acc[i][j];
-    }
-}
-
-// C[M x N] += A[Kd x M]^T B[Kd x N] in FP64, split over Kd (atomics into C).
-template <class TA, class TB>
-__global__ void __launch_bounds__(256) k_gemm_tn64(const TA *A, int lda, const TB *B, int ldb, double *C,
-                                                   int ldc, int M, int N, int Kd, int chunk) {
-  __shared__ double As[16][64 + 1];
-  __shared__ double Bs[16][64];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.z * 64;
-  const int kb = blockIdx.x * chunk, ke = min(Kd, kb + chunk);
-  double acc[4][4] = {};
-  for (int k0 = kb; k0 < ke; k0 += 16) {
-    for (int e = tid; e < 16 * 64; e += 256) {
-      const int kk = e >> 6, c = e & 63, gk = k0 + kk;
-      As[kk][c] = (gk < ke && m0 + c < M) ? (double)A[(long long)gk * lda + m0 + c] : 0.0;
-      Bs[kk][c] = (gk < ke && n0 + c < N) ? (double)B[(long long)gk * ldb + n0 + c] : 0.0;
-    }
-    __syncthreads();
+  float *c = C + blockIdx.z * cstride;
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk)
-      for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) acc[i][j] += As[kk][ty * 4 + i] * Bs[kk][tx * 4 + j];
-    __syncthreads();
-  }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-      if (gm < M && gn < N && acc[i][j] != 0.0) atomicAdd(C + (long long)gm * ldc + gn, acc[i][j]);
+  for (int i = 0; i < 8; ++i) {
+    const int r = m0 + ty * 8 + i;
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int n = n0 + tx + 16 * j;
+      if (r < M && n < N) c[(long long)r * ldc + n] = acc[i][j];
     }
+  }
 }
 
-template <class T>
-void gemm_nn(const T *A, int lda, const T *B, int ldb, T *C, int ldc, int M, int N, int Kd, cudaStream_t s) {
-  dim3 g((N + 63) / 64, (M + 63) / 64);
-  k_gemm_nn<T><<<g, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, Kd);
+__global__ void k_sgemm_sum(const float *part, int splits, long long n, float *C) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  float v = part[e];
+  for (int s = 1; s < splits; ++s) v += part[s * n + e];
+  C[e] = v;
 }
 
+// Splits of the terms: about two tiles per SM, at least 256 terms each.
+int sgemm_splits(int M, int N, int Kd, int sms) {
+  const int tiles = ((M + 127) / 128) * ((N + 127) / 128);
+  return std::max(1, std::min(2 * sms / tiles, Kd / 256));
+}
+
+// part: splits x M x N floats when there is more than one split (C then is M x N).
+void sgemm(const float *A, int lda, const float *B, int ldb, float *C, int M, int N, int Kd, float *part, int splits,
+           cudaStream_t s) {
+  const int nt = (N + 127) / 128, tn = (N + 16 * nt - 1) / (16 * nt);
+  const int chunk = ((Kd + splits - 1) / splits + 15) / 16 * 16;
+  splits = (Kd + chunk - 1) / chunk;
+  const dim3 g(nt, (M + 127) / 128, splits);
+  float *out = splits > 1 ? part : C;
+#define TLDA_SGEMM(TNv)                                                                                          \
+  case TNv: k_sgemm<TNv><<<g, 256, 0, s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N); break;
+  switch (tn) {
+    TLDA_SGEMM(1) TLDA_SGEMM(2) TLDA_SGEMM(3) TLDA_SGEMM(4) TLDA_SGEMM(5) TLDA_SGEMM(6) TLDA_SGEMM(7)
+    default: k_sgemm<8><<<g, 256, 0, s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N); break;
+  }
+#undef TLDA_SGEMM
+  if (splits > 1) {
+    const long long n = (long long)M * N;
+    k_sgemm_sum<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, splits, n, C);
+  }
+}
+
+// Exponents of the operands of the FP64 products (gemm64.cuh): V rows, V terms,
+// then two sets of up to 2 kMaxDim columns.
+constexpr int kExpCols = 2 * kMaxDim;
+
+template <bool FIN, class T>
+void col_exp(const T *x, int ld, int rows, int cols, const int *add, int *e, cudaStream_t s) {
+  const int slab = std::max(64, (rows + 63) / 64);
+  cudaMemsetAsync(e, 0x80, sizeof(int) * cols, s);
+  k_col_exp<FIN, T><<<dim3((cols + 31) / 32, (rows + slab - 1) / slab), 256, 0, s>>>(x, ld, rows, cols, slab, add, e);
+}
+
+// Splits of the terms of an FP64 product: one block per SM runs, so the time
+// goes with the waves of blocks over the splits.
+int gemm64_splits(int tiles, int Kd, int sms) {
+  const int folds = (Kd + kG64Fold - 1) / kG64Fold;
+  int best = 1;
+  double cost = 1e30;
+  for (int S = 1; S <= folds && S <= 64; ++S) {
+    const int waves = (tiles * S + sms - 1) / sms, per = (folds + S - 1) / S;
+    const double c = (double)waves * (per + 0.5);  // a block's start and its sums into C: about half a fold's time
+    if (c < cost) {
+      cost = c;
+      best = S;
+    }
+  }
+  return best;
+}
+
+// C[M x N] = A^T B (FP64), A: Kd x M, B: Kd x N.  exps: ctx->g64_exp.
 template <class TA, class TB>
-void gemm_tn64(const TA *A, int lda, const TB *B, int ldb, double *C, int ldc, int M, int N, int Kd,
-               cudaStream_t s) {
+void gemm_tn64(const TA *A, int lda, const TB *B, int ldb, double *C, int ldc, int M, int N, int Kd, int *exps, int V,
+               int sms, cudaStream_t s) {
   cudaMemsetAsync(C, 0, sizeof(double) * (size_t)M * ldc, s);
-  const int chunk = 512;
-  dim3 g((Kd + chunk - 1) / chunk, (M + 63) / 64, (N + 63) / 64);
-  k_gemm_tn64<TA, TB><<<g, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, Kd, chunk);
+  int *eA = exps + 2 * (size_t)V, *eB = eA + kExpCols;
+  const int tm = (M + kG64Tile - 1) / kG64Tile, tn = (N + kG64Tile - 1) / kG64Tile;
+  col_exp<false>(A, lda, Kd, M, nullptr, eA, s);
+  if (static_cast<const void *>(A) == static_cast<const void *>(B) && lda == ldb && M == N && sizeof(TA) == sizeof(TB)) {
+    g64_launch<true, true, true>(A, lda, B, ldb, C, ldc, M, N, Kd, gemm64_splits(tm * (tm + 1) / 2, Kd, sms), eA, eA,
+                                 nullptr, s);
+  } else {
+    col_exp<false>(B, ldb, Kd, N, nullptr, eB, s);
+    g64_launch<true, true, false>(A, lda, B, ldb, C, ldc, M, N, Kd, gemm64_splits(tm * tn, Kd, sms), eA, eB, nullptr, s);
+  }
+}
+
+// C[M x N] = A B (FP64), A: M x Kd (M, Kd <= V), B: Kd x N.
+template <class TA>
+void gemm_nn64(const TA *A, int lda, const double *B, int ldb, double *C, int ldc, int M, int N, int Kd, int *exps, int V,
+               int sms, cudaStream_t s) {
+  int *eA = exps, *ck = exps + V, *eB = exps + 2 * (size_t)V;
+  col_exp<true>(A, lda, M, Kd, nullptr, ck, s);
+  k_row_exp<TA><<<(M + 7) / 8, 256, 0, s>>>(A, lda, M, Kd, ck, eA);
+  col_exp<false>(B, ldb, Kd, N, ck, eB, s);
+  const int tiles = ((M + kG64Tile - 1) / kG64Tile) * ((N + kG64Tile - 1) / kG64Tile);
+  const int splits = gemm64_splits(tiles, Kd, sms);
+  if (splits > 1) {
+    cudaMemsetAsync(C, 0, sizeof(double) * (size_t)M * ldc, s);
+    g64_launch<false, true, false>(A, lda, B, ldb, C, ldc, M, N, Kd, splits, eA, eB, ck, s);
+  } else {
+    g64_launch<false, false, false>(A, lda, B, ldb, C, ldc, M, N, Kd, 1, eA, eB, ck, s);
+  }
+}
+
+// y[j] += sum over a slab of rows of x[m] Q[m][j] (FP64; y zeroed before): one
+// block per 32 columns and slab.
+__global__ void __launch_bounds__(256) k_vec_tn64(const double *x, const double *Q, int rows, int cols, int slab, double *y) {
+  __shared__ double red[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int r0 = blockIdx.y * slab, r1 = min(rows, r0 + slab);
+  double v = 0.0;
+  if (c < cols)
+    for (int r = r0 + w; r < r1; r += 8) v = fma(x[r], Q[(long long)r * cols + c], v);
+  red[w][lane] = v;
+  __syncthreads();
+  if (w == 0 && c < cols) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v += red[q][lane];
+    atomicAdd(y + c, v);
+  }
+}
+
+void vec_tn64(const double *x, const double *Q, int rows, int cols, double *y, cudaStream_t s) {
+  const int slab = std::max(32, (rows + 63) / 64);
+  cudaMemsetAsync(y, 0, sizeof(double) * cols, s);
+  k_vec_tn64<<<dim3((cols + 31) / 32, (rows + slab - 1) / slab), 256, 0, s>>>(x, Q, rows, cols, slab, y);
+}
+
+// out (D x K) = R X with R FP64 (D x D), plain FP64 sums, one block per row: the
+// products of small triangular factors, whose entries may differ in scale by
+// more than exact slices hold.  scale (K) multiplies the columns when given.
+template <class TX, class TO>
+__global__ void __launch_bounds__(256) k_small_nn(const double *R, const TX *X, int D, int K, const double *scale, TO *out) {
+  __shared__ double g[kMaxDim];
+  const int r = blockIdx.x;
+  for (int j = threadIdx.x; j < D; j += 256) g[j] = R[r * D + j];
+  __syncthreads();
+  for (int i = threadIdx.x; i < K; i += 256) {
+    double v = 0.0;
+#pragma unroll 8
+    for (int j = 0; j < D; ++j) v = fma(g[j], (double)X[j * K + i], v);
+    out[r * K + i] = (TO)(scale ? v * scale[i] : v);
+  }
 }
 
 // ------------------------------------------------------------------ elementwise helpers
-__global__ void k_m2_f32(const double *P, const double *M1, int V, double sP, double a0, float *M2) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)V * V) return;
-  const int i = (int)(e / V), j = (int)(e % V);
-  M2[e] = (float)(sP * P[e] - a0 * M1[i] * M1[j]);
+// The upper half of P (32 x 32 tiles, read below the diagonal) and the FP32
+// M2 = sP P - a0 M1 M1^T in both halves.
+__global__ void __launch_bounds__(256) k_m2_mirror(double *P, const double *M1, int V, double sP, double a0, float *M2) {
+  const int by = blockIdx.y, bx = blockIdx.x;
+  if (bx > by) return;
+  __shared__ double t[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = by * 32 + ty + 8 * q, j = bx * 32 + tx;
+    t[ty + 8 * q][tx] = (i < V && j < V) ? P[(long long)i * V + j] : 0.0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = ty + 8 * q;
+    int i = by * 32 + r, j = bx * 32 + tx;
+    const bool low = bx < by || tx <= r;  // the entry below the diagonal that this one equals
+    if (i < V && j < V) {
+      const double v = low ? t[r][tx] : t[tx][r];
+      M2[(long long)i * V + j] = (float)(sP * v - a0 * M1[i] * M1[j]);
+      if (!low) P[(long long)i * V + j] = v;
+    }
+    if (bx < by) {
+      i = bx * 32 + r, j = by * 32 + tx;
+      if (i < V && j < V) {
+        const double v = t[tx][r];
+        P[(long long)i * V + j] = v;
+        M2[(long long)i * V + j] = (float)(sP * v - a0 * M1[i] * M1[j]);
+      }
+    }
+  }
 }
 
 __global__ void k_m1(const unsigned long long *C, const unsigned long long *TS, int V, double *M1) {
@@ -181,11 +355,6 @@ __global__ void k_gauss(float *O, long long n, unsigned long long seed) {
   const double u1 = ((h1 >> 11) + 0.5) * (1.0 / 9007199254740992.0);
   const double u2 = (h2 >> 11) * (1.0 / 9007199254740992.0);
   O[e] = (float)(sqrt(-2.0 * log(u1)) * cos(6.283185307179586 * u2));
-}
-
-__global__ void k_f2d(const float *x, double *y, long long n) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n) y[e] = x[e];
 }
 
 __global__ void k_d2f(const double *x, float *y, long long n) {
@@ -231,7 +400,10 @@ __device__ bool jac_sync(JacCtl *ctl, unsigned target, int *s_ok) {
     int ok = 1;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar) : "memory");
     const long long t0 = clock64();
-    while (jac_ld_acquire(&ctl->bar) < target) {
+    // the abort flag and the bound are looked at every 16th poll: each look is
+    // a round trip to L2 of its own
+    for (int poll = 1; jac_ld_acquire(&ctl->bar) < target; ++poll) {
+      if (poll & 15) continue;
       if (*reinterpret_cast<volatile int *>(&ctl->abort)) {
         ok = 0;
         break;
@@ -248,6 +420,41 @@ __device__ bool jac_sync(JacCtl *ctl, unsigned target, int *s_ok) {
   return *reinterpret_cast<volatile int *>(s_ok) != 0;
 }
 
+// FP64 to FP32 and back on the integer units, toward zero: a conversion takes
+// the FP64 pipe 65 cycles.  Outside FP32's normal range: 0 below, infinity above.
+__device__ __forceinline__ float seed_f32(double x) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 896;  // FP32 exponent field
+  const uint32_t m = (uint32_t)(b >> 29) & 0x7fffffu, s = (uint32_t)(b >> 32) & 0x80000000u;
+  return __uint_as_float(s | (e <= 0 ? 0u : e >= 255 ? 0x7f800000u : ((uint32_t)e << 23) | m));
+}
+__device__ __forceinline__ double widen_f32(float x) {  // finite; below FP32's normal range: 0
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  const long long s = (long long)(b & 0x80000000u) << 32;
+  return __longlong_as_double(e == 0 ? s : s | ((long long)(e + 896) << 52) | ((long long)(b & 0x7fffffu) << 29));
+}
+
+// 1/d: FP32, then one third-order step (d in FP32's normal range, else divided).
+__device__ __forceinline__ double recip64(double d) {
+  const float f = __frcp_rn(seed_f32(d)), a = fabsf(f);
+  if (!(a > 1e-37f && a < 1e37f)) return 1.0 / d;
+  const double q = widen_f32(f), e = fma(-d, q, 1.0);
+  return fma(q, fma(e, e, e), q);
+}
+
+// Slot of the round-robin ordering: slot 0 holds index 0, the others rotate.
+__device__ __forceinline__ int jac_slot(int slot, int round, int r) {
+  const int x = slot - 1 + round;  // below 2 (r - 1)
+  return slot == 0 ? 0 : 1 + (x >= r - 1 ? x - (r - 1) : x);
+}
+
+// Indices p < q of pair k in a round.
+__device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q) {
+  const int a = jac_slot(k, round, r), b = jac_slot(r - 1 - k, round, r);
+  p = min(a, b);
+  q = max(a, b);
+}
+
 // Cyclic Jacobi for a symmetric r x r FP64 matrix A (r even, global memory,
 // overwritten), round-robin ordering so each round applies r/2 disjoint
 // rotations in parallel (Golub & Van Loan, "Matrix Computations", sec. 8.5,
@@ -256,22 +463,43 @@ __device__ bool jac_sync(JacCtl *ctl, unsigned target, int *s_ok) {
 // Because the rotations of one round are disjoint, A <- J^T A J is applied in
 // one pass over the 2 x 2 blocks (pair k rows, pair l columns), each block
 // rotated on the left by pair k and on the right by pair l; the eigenvectors
-// are kept as rows, Et <- J^T Et.  The rounds are spread over the whole grid
-// (FP64 arithmetic is scarce per SM), one grid barrier per round; every
-// block derives the round's rotations itself.  Et starts as I; on return
-// eval[i] = A_ii and row i of Et is its eigenvector.
-// Sweeps stop when the off-diagonal mass is below 1e-26 r^2 of the total,
-// i.e. entries near 1e-13 of the scale (or after max_sweeps).
+// are kept as rows, Et <- J^T Et.  Et starts as I; on return eval[i] = A_ii and
+// row i of Et is its eigenvector.  Sweeps stop when the off-diagonal mass is
+// below 1e-26 r^2 of the total, i.e. entries near 1e-13 of the scale (or after
+// max_sweeps).
+// A round is bound by its latency: one grid barrier, one L2 round trip, and the
+// FP64 pipe, which takes 2 operations a clock per SM.  So the 2 x 2 blocks are
+// dealt as tiles of bt x bt pairs over T x T thread blocks: a block needs the
+// rotations of its 2 bt pairs only, not of all r/2; its entries are requested
+// before the rotations are computed; and the angle is found in FP32, with c =
+// (1 - h^2)/(1 + h^2) and s = 2 h/(1 + h^2) in FP64 for the h that FP32 gives
+// (an FP64 division or square root takes 430 to 680 cycles here): the rotation
+// is orthogonal to FP64 rounding, and the annihilated entry keeps its computed
+// rest, 1e-7 of what it was.
 __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, int r, double *__restrict__ Et,
                                                        double *__restrict__ eval, int max_sweeps,
                                                        JacCtl *ctl) {
-  __shared__ double cs[kMaxDim / 2], sn[kMaxDim / 2];
-  __shared__ int pp[kMaxDim / 2], qq[kMaxDim / 2];
+  __shared__ double cs[2][kMaxDim / 2], sn[2][kMaxDim / 2];  // rows' pairs, columns' pairs of this block
   __shared__ double red_o[kJacThreads / 32], red_t[kJacThreads / 32];
   __shared__ int s_ok, s_done;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
   const int gt = blockIdx.x * nt + tid, gn = G * nt;
   const int h = r / 2, rr = r * r;
+  int T = 1;
+  while ((T + 1) * (T + 1) <= G) ++T;
+  const int bt = (h + T - 1) / T, ti = blockIdx.x / T, tj = blockIdx.x % T;
+  const int ka = min(h, ti * bt), kn = blockIdx.x < T * T ? min(h, ka + bt) - ka : 0;
+  const int la = min(h, tj * bt), ln = min(h, la + bt) - la;
+  const int ja = (int)((long long)r * tj / T), jn = (int)((long long)r * (tj + 1) / T) - ja;  // columns of Et
+  const int nb = kn * ln, ne = kn * jn;
+  // this thread's first two 2 x 2 blocks and four eigenvector pairs, in every round
+  int bk[2] = {}, bl[2] = {}, ek[4] = {}, ej[4] = {};
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (tid + u * nt < nb) bk[u] = (tid + u * nt) / ln, bl[u] = (tid + u * nt) % ln;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (tid + u * nt < ne) ek[u] = (tid + u * nt) / jn, ej[u] = (tid + u * nt) % jn;
   unsigned nbar = 0;
   for (int e = gt; e < rr; e += gn) {
     const int i = e / r, j = e % r;
@@ -310,97 +538,111 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
       ctl->part[sweep & 1][1][blockIdx.x] = st;
     }
     if (!jac_sync(ctl, ++nbar * G, &s_ok)) return;
-    if (tid == 0) {  // every block sums the partials in the same order
+    if (tid < 32) {  // every block sums the partials in the same order
       double so = 0.0, st = 0.0;
-      for (int g = 0; g < G; ++g) {
+      for (int g = tid; g < G; g += 32) {
         so += __ldcg(&ctl->part[sweep & 1][0][g]);
         st += __ldcg(&ctl->part[sweep & 1][1][g]);
       }
-      s_done = so <= 1e-26 * (double)r * r * st;
+      for (int m = 16; m > 0; m >>= 1) {
+        so += __shfl_xor_sync(0xffffffffu, so, m);
+        st += __shfl_xor_sync(0xffffffffu, st, m);
+      }
+      if (tid == 0) s_done = so <= 1e-26 * (double)r * r * st;
     }
     __syncthreads();
     if (s_done) break;
     for (int round = 0; round < r - 1; ++round) {
-      for (int k = tid; k < h; k += nt) {
-        // round-robin pairing: slot 0 holds index 0, the others rotate
-        const int sa = k, sb = r - 1 - k;
-        int p = sa == 0 ? 0 : 1 + (sa - 1 + round) % (r - 1);
-        int q = sb == 0 ? 0 : 1 + (sb - 1 + round) % (r - 1);
-        if (p > q) {
-          const int tmp = p;
-          p = q;
-          q = tmp;
+      double x[2][4], ev[4][2];
+      int bx[2][4], ei[4][2];
+      auto block_at = [&](int k, int l, int (&base)[4]) {
+        int pk, qk, pl, ql;
+        jac_pair(ka + k, round, r, pk, qk);
+        jac_pair(la + l, round, r, pl, ql);
+        base[0] = pk * r + pl;
+        base[1] = pk * r + ql;
+        base[2] = qk * r + pl;
+        base[3] = qk * r + ql;
+      };
+      auto pair_at = [&](int k, int j, int (&base)[2]) {
+        int p, q;
+        jac_pair(ka + k, round, r, p, q);
+        base[0] = p * r + ja + j;
+        base[1] = q * r + ja + j;
+      };
+      // the rotations' entries first: they are waited for first
+      const bool mine = tid < kn + ln;
+      int p = 0, q = 0;
+      if (mine) jac_pair(tid < kn ? ka + tid : la + tid - kn, round, r, p, q);
+      double apq = 0.0, app = 0.0, aqq = 0.0;
+      if (mine) {
+        apq = __ldcg(A + p * r + q);
+        app = __ldcg(A + p * r + p);
+        aqq = __ldcg(A + q * r + q);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (tid + u * nt < nb) {
+          block_at(bk[u], bl[u], bx[u]);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) x[u][v] = __ldcg(A + bx[u][v]);
         }
-        const double apq = __ldcg(A + p * r + q);
-        const double app = __ldcg(A + p * r + p), aqq = __ldcg(A + q * r + q);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (tid + u * nt < ne) {
+          pair_at(ek[u], ej[u], ei[u]);
+#pragma unroll
+          for (int v = 0; v < 2; ++v) ev[u][v] = __ldcg(Et + ei[u][v]);
+        }
+      if (mine) {
         double c = 1.0, sv = 0.0;
-        if (apq != 0.0) {
-          const double tau = (aqq - app) / (2.0 * apq);
-          const double tt = tau >= 0.0 ? 1.0 / (tau + sqrt(1.0 + tau * tau)) : -1.0 / (-tau + sqrt(1.0 + tau * tau));
-          c = 1.0 / sqrt(1.0 + tt * tt);
-          sv = tt * c;
+        const float fp = seed_f32(apq), fd = seed_f32(aqq - app);
+        if (fp != 0.f) {  // an entry below FP32's range is left as it is
+          const float tau = __fdividef(0.5f * fd, fp), f = fabsf(tau);
+          const float t = __frcp_rn(f + __fsqrt_rn(fmaf(f, f, 1.f)));
+          const float h1 = __fdividef(t, 1.f + __fsqrt_rn(fmaf(t, t, 1.f)));  // tan of half the angle, at most 0.42
+          const double hh = widen_f32(tau < 0.f ? -h1 : h1), w = fma(hh, hh, 1.0);
+          const double q = recip64(w);
+          c = fma(2.0, q, -1.0);
+          sv = 2.0 * hh * q;
         }
-        cs[k] = c;
-        sn[k] = sv;
-        pp[k] = p;
-        qq[k] = q;
+        const int side = tid < kn ? 0 : 1, at = tid < kn ? tid : tid - kn;
+        cs[side][at] = c;
+        sn[side][at] = sv;
       }
       __syncthreads();
-      // 2 x 2 blocks, two per thread per iteration (loads before stores)
-      const int nb = h * h;
-      for (int w0 = gt; w0 < nb; w0 += 2 * gn) {
-        double x[2][4];
-        int base[2][4];
-        bool ok[2];
+      auto rotate_block = [&](int k, int l, const double (&v)[4], const int (&base)[4]) {
+        const double ck = cs[0][k], sk = sn[0][k], cl = cs[1][l], sl = sn[1][l];
+        const double a1 = ck * v[0] - sk * v[2], b1 = ck * v[1] - sk * v[3];
+        const double c1 = sk * v[0] + ck * v[2], d1 = sk * v[1] + ck * v[3];
+        A[base[0]] = cl * a1 - sl * b1;
+        A[base[1]] = sl * a1 + cl * b1;
+        A[base[2]] = cl * c1 - sl * d1;
+        A[base[3]] = sl * c1 + cl * d1;
+      };
+      auto rotate_pair = [&](int k, const double (&v)[2], const int (&base)[2]) {
+        const double c = cs[0][k], sv = sn[0][k];
+        Et[base[0]] = c * v[0] - sv * v[1];
+        Et[base[1]] = sv * v[0] + c * v[1];
+      };
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int w = w0 + u * gn;
-          ok[u] = w < nb;
-          const int k = ok[u] ? w / h : 0, l = ok[u] ? w % h : 0;
-          const int pk = pp[k], qk = qq[k], pl = pp[l], ql = qq[l];
-          base[u][0] = pk * r + pl;
-          base[u][1] = pk * r + ql;
-          base[u][2] = qk * r + pl;
-          base[u][3] = qk * r + ql;
+      for (int u = 0; u < 2; ++u)
+        if (tid + u * nt < nb) rotate_block(bk[u], bl[u], x[u], bx[u]);
 #pragma unroll
-          for (int v = 0; v < 4; ++v) x[u][v] = ok[u] ? __ldcg(A + base[u][v]) : 0.0;
-        }
+      for (int u = 0; u < 4; ++u)
+        if (tid + u * nt < ne) rotate_pair(ek[u], ev[u], ei[u]);
+      // what a small grid leaves over
+      for (int w = tid + 2 * nt; w < nb; w += nt) {
+        block_at(w / ln, w % ln, bx[0]);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (!ok[u]) continue;
-          const int w = w0 + u * gn, k = w / h, l = w % h;
-          const double ck = cs[k], sk = sn[k], cl = cs[l], sl = sn[l];
-          const double a1 = ck * x[u][0] - sk * x[u][2], b1 = ck * x[u][1] - sk * x[u][3];
-          const double c1 = sk * x[u][0] + ck * x[u][2], d1 = sk * x[u][1] + ck * x[u][3];
-          A[base[u][0]] = cl * a1 - sl * b1;
-          A[base[u][1]] = (k == l) ? 0.0 : sl * a1 + cl * b1;
-          A[base[u][2]] = (k == l) ? 0.0 : cl * c1 - sl * d1;
-          A[base[u][3]] = sl * c1 + cl * d1;
-        }
+        for (int v = 0; v < 4; ++v) x[0][v] = __ldcg(A + bx[0][v]);
+        rotate_block(w / ln, w % ln, x[0], bx[0]);
       }
-      // eigenvector rows: Et[p] <- c Et[p] - s Et[q], Et[q] <- s Et[p] + c Et[q]
-      const int ne = h * r;
-      for (int w0 = gt; w0 < ne; w0 += 2 * gn) {
-        double ep[2], eq[2];
-        int ip[2], iq[2];
+      for (int w = tid + 4 * nt; w < ne; w += nt) {
+        pair_at(w / jn, w % jn, ei[0]);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int w = w0 + u * gn;
-          const int k = w < ne ? w / r : 0, j = w < ne ? w % r : 0;
-          ip[u] = pp[k] * r + j;
-          iq[u] = qq[k] * r + j;
-          ep[u] = w < ne ? __ldcg(Et + ip[u]) : 0.0;
-          eq[u] = w < ne ? __ldcg(Et + iq[u]) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int w = w0 + u * gn;
-          if (w >= ne) continue;
-          const int k = w / r;
-          const double c = cs[k], sv = sn[k];
-          Et[ip[u]] = c * ep[u] - sv * eq[u];
-          Et[iq[u]] = sv * ep[u] + c * eq[u];
-        }
+        for (int v = 0; v < 2; ++v) ev[0][v] = __ldcg(Et + ei[0][v]);
+        rotate_pair(w / jn, ev[0], ei[0]);
       }
       if (!jac_sync(ctl, ++nbar * G, &s_ok)) return;
     }
@@ -409,65 +651,184 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
   if (gt == 0) ctl->sweeps = sweep;
 }
 
-
 // Cholesky factor and inverse of a symmetric positive definite r x r FP64
-// matrix A (overwritten): A = L L^T by right-looking elimination (column j:
-// l_jj = sqrt(a_jj), l_ij = a_ij / l_jj, then a_ik -= l_ij l_kj for
-// j < k <= i), and X = L^-1 by right-looking forward substitution on
-// Z = diag(L) X (z_ic -= l_ik / l_kk z_kc for i > k, then x_ic = z_ic / l_ii).
-// Spread over the grid, one grid barrier per column of each phase.  L (lower,
-// zeros above) and the scratch Z are required; Linv, LinvT64 = L^-T and
-// LinvT32 (FP32) are written when given.  status: 1 if a pivot was not
-// positive (it is taken as 1), 2 if a grid barrier expired.
+// matrix A (overwritten), r <= 512: A = L L^T in panels of 32 columns, then
+// X = L^-1 column by column.  Per panel every block factors the 32 x 32
+// diagonal block for itself in shared memory (one block barrier a column: the
+// columns are scaled at the end), warps solve the rows below it, a grid
+// barrier, then the trailing entries take the panel's 32 terms, and another:
+// 2 r/32 grid barriers where one per column took 2 r, each about as long as a
+// panel's arithmetic.  The columns of X are independent: each block takes its
+// own by forward substitution from LT, with no grid barrier.
+// L (lower, zeros above) and LT (its transpose, scratch) are required; Linv,
+// LinvT64 = L^-T and LinvT32 (FP32) are written when given.  status: 1 if a
+// pivot was not positive (it is taken as 1), 2 if a grid barrier expired.
+constexpr int kCholNb = 32;
 __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A, int r, double *__restrict__ L,
-                                                         double *__restrict__ Z, double *Linv, double *LinvT64,
+                                                         double *__restrict__ LT, double *Linv, double *LinvT64,
                                                          float *LinvT32, int *status, JacCtl *ctl) {
+  __shared__ double Ds[kCholNb][kCholNb + 1], inv[kMaxDim];
+  __shared__ double sx[2][4];
   __shared__ int s_ok;
-  const int G = gridDim.x, gt = blockIdx.x * blockDim.x + threadIdx.x, gn = G * blockDim.x;
-  const int rr = r * r;
+  const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int gt = blockIdx.x * nt + tid, gn = G * nt, rr = r * r;
   unsigned nbar = 0;
-  for (int e = gt; e < rr; e += gn) {
-    const int i = e / r, k = e % r;
-    Z[e] = (i == k) ? 1.0 : 0.0;
-    if (k > i) L[e] = 0.0;
-  }
-  for (int j = 0; j < r; ++j) {
-    double d = __ldcg(A + j * r + j);
-    if (!(d > 0.0)) {
-      if (gt == 0) atomicMax(status, 1);
-      d = 1.0;
+  for (int e = gt; e < rr; e += gn)
+    if (e % r > e / r) L[e] = 0.0;
+  for (int j0 = 0; j0 < r; j0 += kCholNb) {
+    const int jb = min(kCholNb, r - j0), j1 = j0 + jb;
+    for (int e = tid; e < jb * jb; e += nt) Ds[e / jb][e % jb] = __ldcg(A + (j0 + e / jb) * r + j0 + e % jb);
+    __syncthreads();
+    // four warps factor, one per SM quarter: an FP64 operation takes a quarter
+    // 64 cycles a warp, so more warps would only repeat the pivot's reciprocal.
+    // Lane = column (kept in registers: rows w, w + 4, ...); the pivot's column
+    // passes through shared memory.  Entries keep a_ij - sum l_ik l_jk, the
+    // columns are scaled afterwards.
+    if (tid < 128) {
+      const int w = tid >> 5;
+      double a[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) a[u] = (w + 4 * u < jb && lane < jb) ? Ds[w + 4 * u][lane] : 0.0;
+      for (int j = 0; j < jb; ++j) {
+        double d = Ds[j][j];
+        if (!(d > 0.0)) {
+          if (gt == 0) atomicMax(status, 1);
+          d = 1.0;
+        }
+        const double f = -Ds[lane][j] * recip64(d);  // rows below j of column j are up to date
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = w + 4 * u;
+          if (i > j && i < jb) {
+            a[u] = fma(Ds[i][j], f, a[u]);
+            if (lane > j && lane <= i) Ds[i][lane] = a[u];
+          }
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
     }
-    d = sqrt(d);
-    const double inv = 1.0 / d;
-    const int m = r - j - 1;
-    for (int e = gt; e <= m; e += gn) L[(j + e) * r + j] = e == 0 ? d : __ldcg(A + (j + e) * r + j) * inv;
+    __syncthreads();
+    if (tid < jb) {
+      const double d = Ds[tid][tid];
+      inv[j0 + tid] = rsqrt(d > 0.0 ? d : 1.0);
+    }
+    __syncthreads();
+    for (int e = tid; e < jb * jb; e += nt) {
+      const int i = e / jb, k = e % jb;
+      if (k < i) Ds[i][k] *= inv[j0 + k];
+    }
+    if (tid < jb) {
+      const double d = Ds[tid][tid];
+      Ds[tid][tid] = (d > 0.0 ? d : 1.0) * inv[j0 + tid];
+    }
+    __syncthreads();
+    if (blockIdx.x == 0)
+      for (int e = tid; e < jb * jb; e += nt) {
+        const int i = e / jb, k = e % jb;
+        if (k <= i) {
+          L[(j0 + i) * r + j0 + k] = Ds[i][k];
+          LT[(j0 + k) * r + j0 + i] = Ds[i][k];
+        }
+      }
+    // rows below: x L11^T = a, lane k holds column k
+    for (int i = j1 + (gt >> 5); i < r; i += gn >> 5) {
+      double a = lane < jb ? __ldcg(A + i * r + j0 + lane) : 0.0;
+      for (int k = 0; k < jb; ++k) {
+        const double x = __shfl_sync(0xffffffffu, a, k) * inv[j0 + k];
+        if (lane == k) a = x;
+        else if (lane > k && lane < jb) a = fma(-x, Ds[lane][k], a);
+      }
+      if (lane < jb) {
+        L[i * r + j0 + lane] = a;
+        LT[(j0 + lane) * r + i] = a;
+      }
+    }
+    if (!jac_sync(ctl, ++nbar * G, &s_ok)) {
+      if (tid == 0) atomicMax(status, 2);
+      return;
+    }
+    if (j1 >= r) break;
+    const int m = r - j1;
     for (int e = gt; e < m * m; e += gn) {
-      const int i = j + 1 + e / m, k = j + 1 + e % m;
-      if (k <= i) A[i * r + k] = __ldcg(A + i * r + k) - (__ldcg(A + i * r + j) * inv) * (__ldcg(A + k * r + j) * inv);
+      const int i = j1 + e / m, k = j1 + e % m;
+      if (k > i) continue;
+      double v = __ldcg(A + i * r + k);
+#pragma unroll 8
+      for (int q = 0; q < kCholNb; ++q)  // a panel with columns after it is whole
+        v = fma(-__ldcg(LT + (j0 + q) * r + i), __ldcg(LT + (j0 + q) * r + k), v);
+      A[i * r + k] = v;
     }
     if (!jac_sync(ctl, ++nbar * G, &s_ok)) {
-      if (threadIdx.x == 0) atomicMax(status, 2);
+      if (tid == 0) atomicMax(status, 2);
       return;
     }
   }
-  for (int k = 0; k < r - 1; ++k) {
-    const double f = 1.0 / __ldcg(L + k * r + k);
-    const int m = r - k - 1, w = k + 1;  // rows k+1 .. r-1, columns 0 .. k
-    for (int e = gt; e < m * w; e += gn) {
-      const int i = k + 1 + e / w, c = e % w;
-      Z[i * r + c] = __ldcg(Z + i * r + c) - __ldcg(L + i * r + k) * f * __ldcg(Z + k * r + c);
+  if (!Linv && !LinvT64 && !LinvT32) return;
+  // columns blockIdx, blockIdx + G, ... of L^-1, four at a time; thread i holds
+  // rows i and i + 256.  Two FP64 operations and a block barrier a step, each row
+  // of x scaled by its own thread.
+  for (int c0 = blockIdx.x; c0 < r; c0 += 4 * G) {
+    const int nc = min(4, (r - c0 + G - 1) / G);
+    double z[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[u][q] = (tid + u * kJacThreads == c0 + q * G) ? 1.0 : 0.0;
+    double lv[4][2], nx[4][2];
+    auto rows = [&](int k, double (&v)[4][2]) {  // L rows tid, tid + 256 of columns k .. k + 3
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int i = tid + u * kJacThreads;
+          v[g][u] = (k + g < r && i < r && i > k + g) ? __ldcg(LT + (k + g) * r + i) : 0.0;
+        }
+    };
+    rows(c0, lv);
+    __syncthreads();  // sx of the columns before
+    for (int k0 = c0; k0 < r; k0 += 4) {
+      rows(k0 + 4, nx);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const int k = k0 + g;
+        if (k < r) {
+          if (tid == (k & (kJacThreads - 1))) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (q < nc) {
+                const double x = (k < kJacThreads ? z[0][q] : z[1][q]) * inv[k];
+                if (k < kJacThreads) z[0][q] = x;
+                else z[1][q] = x;
+                sx[k & 1][q] = x;
+              }
+          }
+          __syncthreads();
+          // FP64 issue is what a step costs: rows at or above k and columns past r are skipped
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < nc) {
+              const double x = sx[k & 1][q];
+              if ((tid | 31) > k) z[0][q] = fma(-lv[g][0], x, z[0][q]);
+              if (kJacThreads < r && (tid | 31) + kJacThreads > k) z[1][q] = fma(-lv[g][1], x, z[1][q]);
+            }
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) lv[g][u] = nx[g][u];
     }
-    if (!jac_sync(ctl, ++nbar * G, &s_ok)) {
-      if (threadIdx.x == 0) atomicMax(status, 2);
-      return;
-    }
-  }
-  for (int e = gt; e < rr; e += gn) {
-    const int i = e / r, c = e % r;
-    const double x = c <= i ? __ldcg(Z + e) / __ldcg(L + i * r + i) : 0.0;
-    if (Linv) Linv[e] = x;
-    if (LinvT64) LinvT64[c * r + i] = x;
-    if (LinvT32) LinvT32[c * r + i] = (float)x;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = tid + u * kJacThreads, c = c0 + q * G;
+        if (i >= r || c >= r) continue;
+        const double x = c <= i ? z[u][q] : 0.0;
+        if (Linv) Linv[i * r + c] = x;
+        if (LinvT64) LinvT64[c * r + i] = x;
+        if (LinvT32) LinvT32[c * r + i] = (float)x;
+      }
   }
 }
 
@@ -484,7 +845,7 @@ __global__ void __launch_bounds__(kJacThreads) k_solve_right(const double *__res
                                                             double *__restrict__ B, int *status, JacCtl *ctl) {
   __shared__ unsigned char used[kMaxDim];
   __shared__ int piv[kMaxDim];
-  __shared__ double red_v[kJacThreads / 32];
+  __shared__ unsigned long long red_v[kJacThreads / 32];
   __shared__ int red_i[kJacThreads / 32];
   __shared__ int s_ok, s_p;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
@@ -501,18 +862,21 @@ __global__ void __launch_bounds__(kJacThreads) k_solve_right(const double *__res
     return;
   }
   for (int j = 0; j < r; ++j) {
-    double bv = -1.0;
+    // largest |pivot|, lowest row on ties, as one key: magnitudes compare as
+    // their bits (integer units; an FP64 comparison takes 64 cycles), NaN is
+    // no candidate
+    unsigned long long bv = 0;  // bits + 1
     int bi = r;
     for (int i = tid; i < r; i += nt)
       if (!used[i]) {
-        const double v = fabs(__ldcg(M + i * r + j));
-        if (v > bv) {
-          bv = v;
+        const unsigned long long v = (unsigned long long)__double_as_longlong(__ldcg(M + i * r + j)) & 0x7fffffffffffffffull;
+        if (v <= 0x7ff0000000000000ull && v + 1 > bv) {
+          bv = v + 1;
           bi = i;
         }
       }
     for (int m = 16; m > 0; m >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, m);
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, m);
       const int oi = __shfl_xor_sync(0xffffffffu, bi, m);
       if (ov > bv || (ov == bv && oi < bi)) {
         bv = ov;
@@ -530,7 +894,7 @@ __global__ void __launch_bounds__(kJacThreads) k_solve_right(const double *__res
           bv = red_v[w];
           bi = red_i[w];
         }
-      if (!(bv > 0.0)) {
+      if (bv <= 1) {  // zero, or no finite candidate
         if (blockIdx.x == 0) atomicMax(status, 1);
         if (bi >= r)  // no finite candidate: take the first unused row
           for (bi = 0; bi < r && used[bi]; ++bi) {
@@ -578,102 +942,163 @@ __global__ void k_rank1_fix(double *Z, const double *M1, const double *m1q, int 
   Z[e] = sP * Z[e] - a0 * M1[i] * m1q[j];
 }
 
-// W = U_D Lambda^-1/2 with the sign of each eigenvector fixed so that its
-// largest-magnitude entry is positive (lowest index on ties).  One block per column.
-__global__ void k_make_w(const double *U, int V, int D, const double *lam, float *W32, double *W64, int *sgn) {
-  const int j = blockIdx.x;
-  __shared__ double bv[256];
-  __shared__ int bi[256];
+// Per column of U (V x D) and slab of rows (blockIdx.y), the entry of largest
+// magnitude: |u| and row (the lowest on ties) in a key per slab.  One block per
+// 32 columns, whole rows read.
+__global__ void __launch_bounds__(256) k_col_peak(const double *U, int V, int D, int slab, double *pv, int *pi) {
+  __shared__ double bv[8][33];
+  __shared__ int bi[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int r0 = blockIdx.y * slab, r1 = min(V, r0 + slab);
   double best = -1.0;
-  int besti = 0x7fffffff;
-  for (int m = threadIdx.x; m < V; m += blockDim.x) {
-    const double a = fabs(U[(long long)m * D + j]);
-    if (a > best || (a == best && m < besti)) {
-      best = a;
-      besti = m;
-    }
-  }
-  bv[threadIdx.x] = best;
-  bi[threadIdx.x] = besti;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      const double o = bv[threadIdx.x + w];
-      const int oi = bi[threadIdx.x + w];
-      if (o > bv[threadIdx.x] || (o == bv[threadIdx.x] && oi < bi[threadIdx.x])) {
-        bv[threadIdx.x] = o;
-        bi[threadIdx.x] = oi;
+  int at = 0x7fffffff;
+  if (c < D) {
+#pragma unroll 4
+    for (int m = r0 + w; m < r1; m += 8) {  // rows ascend: the first of equals stays
+      const double a = fabs(U[(long long)m * D + c]);
+      if (a > best) {
+        best = a;
+        at = m;
       }
     }
-    __syncthreads();
   }
-  const double sg = U[(long long)bi[0] * D + j] < 0 ? -1.0 : 1.0;
-  const double sc = sg / sqrt(lam[j]);
-  for (int m = threadIdx.x; m < V; m += blockDim.x) {
-    const double w = U[(long long)m * D + j] * sc;
-    W32[(long long)m * D + j] = (float)w;
-    if (W64) W64[(long long)m * D + j] = w;
+  bv[w][lane] = best;
+  bi[w][lane] = at;
+  __syncthreads();
+  if (w == 0 && c < D) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+      if (bv[q][lane] > best || (bv[q][lane] == best && bi[q][lane] < at)) {
+        best = bv[q][lane];
+        at = bi[q][lane];
+      }
+    pv[blockIdx.y * D + c] = best;
+    pi[blockIdx.y * D + c] = at;
   }
-  if (threadIdx.x == 0 && sgn) sgn[j] = (int)sg;
 }
 
-// m1 = W^T M1 (FP64 accumulate), one block per component.
-__global__ void k_wtm1(const float *W, const double *M1, int V, int D, float *m1) {
-  const int j = blockIdx.x;
-  __shared__ double red[256];
-  double s = 0.0;
-  for (int m = threadIdx.x; m < V; m += blockDim.x) s += (double)W[(long long)m * D + j] * M1[m];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+// W = U_D Lambda^-1/2 with the sign of each eigenvector fixed so that its
+// largest-magnitude entry is positive (lowest index on ties), and m1 += W^T M1
+// over the block's rows (m1_64 zeroed before).  Blocks as k_col_peak's, whose
+// nslab peaks each block folds for its columns.
+__global__ void __launch_bounds__(256) k_make_w(const double *U, int V, int D, int slab, const double *pv, const int *pi,
+                                                int nslab, const double *lam, const double *M1, float *W32,
+                                                double *m1_64) {
+  __shared__ double red[8][33], scale[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int r0 = blockIdx.y * slab, r1 = min(V, r0 + slab);
+  if (w == 0 && c < D) {
+    double best = -1.0;
+    int at = 0x7fffffff;
+    for (int q = 0; q < nslab; ++q) {
+      const double a = pv[q * D + c];
+      if (a > best) {  // slabs ascend in rows
+        best = a;
+        at = pi[q * D + c];
+      }
+    }
+    if (at >= V) at = 0;  // every entry NaN
+    scale[lane] = (U[(long long)at * D + c] < 0 ? -1.0 : 1.0) / sqrt(lam[c]);
   }
-  if (threadIdx.x == 0) m1[j] = (float)red[0];
+  __syncthreads();
+  double s = 0.0;
+  if (c < D) {
+    const double sc = scale[lane];
+#pragma unroll 4
+    for (int m = r0 + w; m < r1; m += 8) {
+      const float x = (float)(U[(long long)m * D + c] * sc);
+      W32[(long long)m * D + c] = x;
+      s = fma((double)x, M1[m], s);
+    }
+  }
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && c < D) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
+    atomicAdd(m1_64 + c, s);
+  }
+}
+
+__global__ void k_m1_f32(const double *m1_64, int D, int Dp, float *m1) {
+  const int i = threadIdx.x + blockIdx.x * blockDim.x;
+  if (i < Dp) m1[i] = i < D ? (float)m1_64[i] : 0.f;
+}
+
+// Enqueues W, m1 and U of a whitening from U64 (V x D) and lam; peaks: kWSlabs x
+// D doubles and as many ints, m1_64: D.
+constexpr int kWSlabs = 64;
+void make_whitening(tlda_ctx *ctx, const double *U64, const double *lam, const double *M1, double *pv, int *pi,
+                    double *m1_64, cudaStream_t s) {
+  const int V = ctx->V, D = ctx->D, slab = std::max(8, (V + kWSlabs - 1) / kWSlabs), ns = (V + slab - 1) / slab;
+  const dim3 g((D + 31) / 32, ns);
+  cudaMemsetAsync(m1_64, 0, sizeof(double) * D, s);
+  k_col_peak<<<g, 256, 0, s>>>(U64, V, D, slab, pv, pi);
+  k_make_w<<<g, 256, 0, s>>>(U64, V, D, slab, pv, pi, ns, lam, M1, ctx->W32, m1_64);
+  k_m1_f32<<<1, kMaxDim, 0, s>>>(m1_64, D, ctx->Dp, ctx->m1);
+  launch_make_u(ctx->W32, ctx->m1, V, D, ctx->Dp, ctx->U32, ctx->U16, s);
 }
 
 // ------------------------------------------------------------------ unwhitening
-// T[r][i] = sum_j Ginv[r][j] Phi[j][i] ||phi_i||^2, alpha_i ~ ||phi_i||^-6.
-__global__ void k_unwhiten_coef(const float *Phi, int D, int K, const double *Ginv, double *T, double *alpha) {
-  __shared__ double nrm2[kMaxDim];
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    double s = 0.0;
-    for (int r = 0; r < D; ++r) s += (double)Phi[r * K + i] * Phi[r * K + i];
-    nrm2[i] = s;
+// n2_i = ||phi_i||^2 and alpha_i ~ ||phi_i||^-6, normalised (one block).
+__global__ void __launch_bounds__(kMaxDim) k_unwhiten_norms(const float *Phi, int D, int K, double *n2_out, double *alpha) {
+  __shared__ double red[kMaxDim];
+  const int i = threadIdx.x;
+  double a = 0.0;
+  if (i < K) {
+    double n2 = 0.0;
+#pragma unroll 8
+    for (int j = 0; j < D; ++j) {
+      const double p = (double)Phi[j * K + i];
+      n2 = fma(p, p, n2);
+    }
+    n2_out[i] = n2;
+    a = pow(n2, -3.0);
   }
+  red[i] = a;
   __syncthreads();
-  for (int e = threadIdx.x; e < D * K; e += blockDim.x) {
-    const int r = e / K, i = e % K;
-    double s = 0.0;
-    for (int j = 0; j < D; ++j) s += Ginv[r * D + j] * (double)Phi[j * K + i];
-    T[e] = s * nrm2[i];
+  for (int w = kMaxDim / 2; w > 0; w >>= 1) {
+    if (i < w) red[i] += red[i + w];
+    __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    double z = 0.0;
-    for (int i = 0; i < K; ++i) z += pow(nrm2[i], -3.0);
-    for (int i = 0; i < K; ++i) alpha[i] = pow(nrm2[i], -3.0) / z;
+  if (i < K) alpha[i] = a / red[0];
+}
+
+// Column sums of max(mu, 0) (V x K) into sum (zeroed before): one block per 32
+// columns and slab of rows; then mu = max(mu, 0) / sum (1 where that is 0).
+// Both read whole rows (a block per column would touch a 32-byte sector for
+// each entry).
+__global__ void __launch_bounds__(256) k_clip_sum(const double *mu, int V, int K, int slab, double *sum) {
+  __shared__ double red[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int r0 = blockIdx.y * slab, r1 = min(V, r0 + slab);
+  double v = 0.0;
+  if (c < K) {
+#pragma unroll 4
+    for (int r = r0 + w; r < r1; r += 8) {
+      const double x = mu[(long long)r * K + c];
+      v += x > 0.0 ? x : 0.0;
+    }
+  }
+  red[w][lane] = v;
+  __syncthreads();
+  if (w == 0 && c < K) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v += red[q][lane];
+    atomicAdd(sum + c, v);
   }
 }
 
-// clip at 0 and normalise each column of mu (V x K) to sum 1; one block per column.
-__global__ void k_clip_norm(double *mu, int V, int K) {
-  const int i = blockIdx.x;
-  __shared__ double red[256];
-  double s = 0.0;
-  for (int m = threadIdx.x; m < V; m += blockDim.x) {
-    double v = mu[(long long)m * K + i];
-    v = v > 0.0 ? v : 0.0;
-    mu[(long long)m * K + i] = v;
-    s += v;
+__global__ void __launch_bounds__(256) k_clip_scale(double *mu, int V, int K, int slab, const double *sum) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int r0 = blockIdx.y * slab, r1 = min(V, r0 + slab);
+  if (c >= K) return;
+  const double z = sum[c] > 0.0 ? sum[c] : 1.0, inv = 1.0 / z;
+#pragma unroll 4
+  for (int r = r0 + w; r < r1; r += 8) {
+    const double v = mu[(long long)r * K + c], x = v > 0.0 ? v : 0.0, q = x * inv;
+    mu[(long long)r * K + c] = fma(fma(-z, q, x), inv, q);  // x / z to rounding, without a division an entry
   }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  const double z = red[0] > 0.0 ? red[0] : 1.0;
-  for (int m = threadIdx.x; m < V; m += blockDim.x) mu[(long long)m * K + i] /= z;
 }
 
 tlda_status fail(tlda_ctx *c, tlda_status s, const char *msg) {
@@ -691,6 +1116,12 @@ tlda_status fail(tlda_ctx *c, tlda_status s, const char *msg) {
   } while (0)
 
 template <class T>
+void dfree(T *&p) {
+  if (p) cudaFree(p);
+  p = nullptr;
+}
+
+template <class T>
 cudaError_t dalloc(T **p, size_t n, bool zero = false) {
   if (n == 0) n = 1;
   cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), n * sizeof(T));
@@ -698,17 +1129,37 @@ cudaError_t dalloc(T **p, size_t n, bool zero = false) {
   return e;
 }
 
-// Scratch of a FINALIZE or an unwhitening, freed on every exit path.
-struct Scratch {
-  std::vector<void *> ptrs;
+// Arrays laid out one after the other (256-byte aligned); base null: only measured.
+struct Carver {
+  char *base;
+  size_t off = 0;
   template <class T>
-  cudaError_t get(T **p, size_t n, bool zero = false) {
-    cudaError_t e = dalloc(p, n, zero);
-    if (e == cudaSuccess) ptrs.push_back(*p);
-    return e;
+  void take(T *&p, size_t n) {
+    off = (off + 255) & ~size_t(255);
+    p = base ? reinterpret_cast<T *>(base + off) : nullptr;
+    off += n * sizeof(T);
+  }
+};
+
+// Scratch of a FINALIZE: one allocation (each cudaMalloc and
+// cudaFree takes the host some 15 us), freed on every exit path.
+struct Scratch {
+  void *ptr = nullptr;
+  template <class F>
+  cudaError_t carve(F lay) {
+    Carver m{nullptr};
+    lay(m);
+    const cudaError_t e = cudaMalloc(&ptr, m.off);
+    if (e != cudaSuccess) {
+      ptr = nullptr;
+      return e;
+    }
+    Carver c{static_cast<char *>(ptr)};
+    lay(c);
+    return cudaSuccess;
   }
   ~Scratch() {
-    for (void *p : ptrs) cudaFree(p);
+    if (ptr) cudaFree(ptr);
   }
 };
 
@@ -737,6 +1188,13 @@ tlda_status coop_ctl(tlda_ctx *ctx, JacCtl **out, cudaStream_t s) {
   if (!ctx->coop_ctl) CKF(cudaMalloc(&ctx->coop_ctl, sizeof(JacCtl)));
   CKF(cudaMemsetAsync(ctx->coop_ctl, 0, sizeof(JacCtl), s));
   *out = static_cast<JacCtl *>(ctx->coop_ctl);
+  return TLDA_OK;
+}
+
+// The context's exponents for the FP64 products.
+tlda_status g64_exps(tlda_ctx *ctx, int **out) {
+  if (!ctx->g64_exp) CKF(dalloc(&ctx->g64_exp, 2 * (size_t)ctx->V + 2 * kExpCols));
+  *out = ctx->g64_exp;
   return TLDA_OK;
 }
 
@@ -797,68 +1255,74 @@ tlda_status finalize(tlda_ctx *ctx) {
   if (ferr) return fail(ctx, TLDA_ERR_INVALID, "corrupt CSR chunk in fit_moments");
   if (TS[0] == 0 || TS[1] == 0) return fail(ctx, TLDA_ERR_NUMERIC, "no token pairs accumulated");
   const double a0 = ctx->p.alpha0, sP = (a0 + 1.0) / (double)TS[1];
-  Scratch sc;
-  double *M1 = nullptr, *Q64 = nullptr, *Z64 = nullptr, *G = nullptr, *Linv = nullptr, *LinvT64 = nullptr;
-  double *Zr = nullptr;
-  double *Bm = nullptr, *Ev = nullptr, *ev = nullptr, *m1q = nullptr, *U64 = nullptr, *lam = nullptr, *Ek = nullptr;
-  float *M2 = nullptr, *Om = nullptr, *Y = nullptr, *Qf = nullptr, *LinvT32 = nullptr;
-  int *status = nullptr;
   const long long VV = (long long)V * V;
-  CKF(sc.get(&M1, V));
-  CKF(sc.get(&M2, (size_t)VV));
-  CKF(sc.get(&Om, (size_t)V * r));
-  CKF(sc.get(&Y, (size_t)V * r));
-  CKF(sc.get(&Qf, (size_t)V * r));
-  CKF(sc.get(&Q64, (size_t)V * r));
-  CKF(sc.get(&Z64, (size_t)V * r));
-  CKF(sc.get(&G, (size_t)r * r));
-  CKF(sc.get(&Linv, (size_t)r * r));
-  CKF(sc.get(&LinvT64, (size_t)r * r));
-  CKF(sc.get(&LinvT32, (size_t)r * r));
-  CKF(sc.get(&Zr, (size_t)r * r));
-  CKF(sc.get(&Bm, (size_t)r * r));
-  CKF(sc.get(&Ev, (size_t)r * r));
-  CKF(sc.get(&ev, (size_t)r));
-  CKF(sc.get(&Ek, (size_t)r * D));
-  CKF(sc.get(&m1q, (size_t)r));
-  CKF(sc.get(&U64, (size_t)V * D));
-  CKF(sc.get(&lam, (size_t)D));
-  CKF(sc.get(&status, 2, true));
+  int *ex = nullptr;
+  if (tlda_status st = g64_exps(ctx, &ex)) return st;
+  const int sms = ctx->num_sms, splits = sgemm_splits(V, r, V, sms);
+  // one allocation, freed on every exit path
+  double *M1 = nullptr, *Q64 = nullptr, *Z64 = nullptr, *G = nullptr, *Linv = nullptr, *LinvT64 = nullptr;
+  double *Zr = nullptr, *Pv = nullptr;
+  int *Pi = nullptr;
+  double *Bm = nullptr, *Ev = nullptr, *ev = nullptr, *m1q = nullptr, *U64 = nullptr, *lam = nullptr, *Ek = nullptr;
+  float *M2 = nullptr, *Om = nullptr, *Y = nullptr, *Qf = nullptr, *LinvT32 = nullptr, *part = nullptr;
+  int *status = nullptr;
+  Scratch sc;
+  const size_t Vr = (size_t)V * r, r2 = (size_t)r * r;
+  CKF(sc.carve([&](Carver &c) {
+    c.take(M1, V);
+    c.take(Q64, Vr);
+    c.take(Z64, Vr);
+    c.take(G, r2);
+    c.take(Linv, r2);
+    c.take(LinvT64, r2);
+    c.take(Zr, r2);
+    c.take(Bm, r2);
+    c.take(Ev, r2);
+    c.take(ev, r);
+    c.take(Ek, (size_t)r * D);
+    c.take(m1q, r);
+    c.take(U64, (size_t)V * D);
+    c.take(lam, D);
+    c.take(Pv, (size_t)kWSlabs * D);
+    c.take(Pi, (size_t)kWSlabs * D);
+    c.take(M2, (size_t)VV);
+    c.take(Om, Vr);
+    c.take(Y, Vr);
+    c.take(Qf, Vr);
+    c.take(LinvT32, r2);
+    c.take(part, splits > 1 ? splits * Vr : 1);
+    c.take(status, 2);
+  }));
+  CKF(cudaMemsetAsync(status, 0, 2 * sizeof(int), s));
   k_m1<<<(V + 255) / 256, 256, 0, s>>>(ctx->Ccnt, ctx->TS, V, M1);
-  k_m2_f32<<<(unsigned)((VV + 255) / 256), 256, 0, s>>>(ctx->P64, M1, V, sP, a0, M2);
+  k_m2_mirror<<<dim3((V + 31) / 32, (V + 31) / 32), 256, 0, s>>>(ctx->P64, M1, V, sP, a0, M2);
   k_gauss<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(Om, (long long)V * r, ctx->p.seed * 0x100000001B3ull + 17);
   // one CholeskyQR pass: out = in L^-T with L L^T = in^T in (FP64 Gram)
   auto cholqr_pass = [&](const float *in, float *out) -> tlda_status {
-    gemm_tn64<float, float>(in, r, in, r, G, r, r, r, V, s);
+    gemm_tn64(in, r, in, r, G, r, r, r, V, ex, V, sms, s);
     if (tlda_status st = run_chol_inv(ctx, G, r, Linv, Zr, nullptr, nullptr, LinvT32, status, s)) return st;
-    gemm_nn<float>(in, r, LinvT32, r, out, r, V, r, r, s);
+    sgemm(in, r, LinvT32, r, out, V, r, r, nullptr, 1, s);
     return TLDA_OK;
   };
-  // CholeskyQR2 of Y into Qf (Y is clobbered)
-  auto cholqr2 = [&]() -> tlda_status {
-    if (tlda_status st = cholqr_pass(Y, Qf)) return st;
-    if (tlda_status st = cholqr_pass(Qf, Y)) return st;
-    CKF(cudaMemcpyAsync(Qf, Y, sizeof(float) * (size_t)V * r, cudaMemcpyDeviceToDevice, s));
-    return TLDA_OK;
-  };
-  gemm_nn<float>(M2, V, Om, r, Y, r, V, r, V, s);
-  if (tlda_status st = cholqr2()) return st;
+  // Y = M2 Q, then one CholeskyQR pass.  A single pass keeps the same span, and
+  // the columns orthonormal to 1e-16 times the squared condition of Y, which is
+  // all that the next product needs; a second one is taken at the end.
+  sgemm(M2, V, Om, r, Y, V, r, V, part, splits, s);
+  if (tlda_status st = cholqr_pass(Y, Qf)) return st;
   const int n_iter = 24;
   for (int it = 0; it < n_iter; ++it) {
-    gemm_nn<float>(M2, V, Qf, r, Y, r, V, r, V, s);
-    if (tlda_status st = cholqr2()) return st;
+    sgemm(M2, V, Qf, r, Y, V, r, V, part, splits, s);
+    if (tlda_status st = cholqr_pass(Y, Qf)) return st;
   }
   // FP64 Rayleigh-Ritz on the exact M2 = sP P - a0 M1 M1^T
-  k_f2d<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(Qf, Q64, (long long)V * r);
-  // one FP64 CholeskyQR pass to make Q64 orthonormal to FP64 accuracy
-  gemm_tn64<double, double>(Q64, r, Q64, r, G, r, r, r, V, s);
+  // one FP64 CholeskyQR pass makes Q64 orthonormal to FP64 accuracy
+  gemm_tn64(Qf, r, Qf, r, G, r, r, r, V, ex, V, sms, s);
   if (tlda_status st = run_chol_inv(ctx, G, r, Linv, Zr, nullptr, LinvT64, nullptr, status, s)) return st;
-  gemm_nn<double>(Q64, r, LinvT64, r, Z64, r, V, r, r, s);
-  cudaMemcpyAsync(Q64, Z64, sizeof(double) * (size_t)V * r, cudaMemcpyDeviceToDevice, s);
-  gemm_nn<double>(ctx->P64, V, Q64, r, Z64, r, V, r, V, s);
-  gemm_tn64<double, double>(M1, 1, Q64, r, m1q, r, 1, r, V, s);
+  gemm_nn64(Qf, r, LinvT64, r, Q64, r, V, r, r, ex, V, sms, s);
+  gemm_nn64(ctx->P64, V, Q64, r, Z64, r, V, r, V, ex, V, sms, s);
+  vec_tn64(M1, Q64, V, r, m1q, s);
   k_rank1_fix<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(Z64, M1, m1q, V, r, sP, a0);
-  gemm_tn64<double, double>(Q64, r, Z64, r, Bm, r, r, r, V, s);
+  gemm_tn64(Q64, r, Z64, r, Bm, r, r, r, V, ex, V, sms, s);
   CKF(cudaGetLastError());
   if (tlda_status js = run_jacobi(ctx, Bm, r, Ev, ev, s)) return js;
   std::vector<double> hev(r), hEv((size_t)r * r);
@@ -881,11 +1345,8 @@ tlda_status finalize(tlda_ctx *ctx) {
     return fail(ctx, TLDA_ERR_NUMERIC, "M2 has fewer than D positive eigenvalues");
   CKF(cudaMemcpyAsync(Ek, hEk.data(), sizeof(double) * r * D, cudaMemcpyHostToDevice, s));
   CKF(cudaMemcpyAsync(lam, hlam.data(), sizeof(double) * D, cudaMemcpyHostToDevice, s));
-  gemm_nn<double>(Q64, r, Ek, D, U64, D, V, D, r, s);
-  k_make_w<<<D, 256, 0, s>>>(U64, V, D, lam, ctx->W32, nullptr, nullptr);
-  CKF(cudaMemsetAsync(ctx->m1, 0, sizeof(float) * ctx->Dp, s));
-  k_wtm1<<<D, 256, 0, s>>>(ctx->W32, M1, V, D, ctx->m1);
-  launch_make_u(ctx->W32, ctx->m1, V, D, ctx->Dp, ctx->U32, ctx->U16, s);
+  gemm_nn64(Q64, r, Ek, D, U64, D, V, D, r, ex, V, sms, s);
+  make_whitening(ctx, U64, lam, M1, Pv, Pi, m1q, s);
   CKF(cudaGetLastError());
   CKF(cudaStreamSynchronize(s));
   ctx->eig = hlam;
@@ -1183,25 +1644,27 @@ tlda_status online_rewhiten(tlda_ctx *ctx) {
   if (TS[0] == 0 || TS[1] == 0) return fail(ctx, TLDA_ERR_NUMERIC, "no token pairs accumulated");
   const double a0 = ctx->p.alpha0, sP = (a0 + 1.0) / (double)TS[1];
   OnlineWs w(ctx->on_ws, V, r, D);
-  int *status = ctx->on_status;
+  int *status = ctx->on_status, *ex = nullptr;
+  const int sms = ctx->num_sms;
+  if (tlda_status st = g64_exps(ctx, &ex)) return st;
   CKF(cudaMemsetAsync(status, 0, 2 * sizeof(int), s));
   k_m1<<<(V + 255) / 256, 256, 0, s>>>(ctx->on_C, ctx->on_TS, V, w.M1);
-  gemm_tn64<double, double>(w.M1, 1, ctx->on_Om, r, w.m1q, r, 1, r, V, s);
+  vec_tn64(w.M1, ctx->on_Om, V, r, w.m1q, s);
   CKF(cudaMemcpyAsync(w.Y, ctx->on_Z, sizeof(double) * (size_t)V * r, cudaMemcpyDeviceToDevice, s));
   k_rank1_fix<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(w.Y, w.M1, w.m1q, V, r, sP, a0);
   // CholeskyQR2: out = in L^-T with L L^T = in^T in, twice; Y = Q2 (L1 L2)^T
   auto cholqr_pass = [&](const double *in, double *out, double *Lf) -> tlda_status {
-    gemm_tn64<double, double>(in, r, in, r, w.G, r, r, r, V, s);
+    gemm_tn64(in, r, in, r, w.G, r, r, r, V, ex, V, sms, s);
     if (tlda_status st = run_chol_inv(ctx, w.G, r, Lf, w.Z, nullptr, w.LinvT, nullptr, status, s)) return st;
-    gemm_nn<double>(in, r, w.LinvT, r, out, r, V, r, r, s);
+    gemm_nn64(in, r, w.LinvT, r, out, r, V, r, r, ex, V, sms, s);
     return TLDA_OK;
   };
   if (tlda_status st = cholqr_pass(w.Y, w.Q1, w.L1)) return st;
   if (tlda_status st = cholqr_pass(w.Q1, w.Q2, w.L2)) return st;
-  gemm_tn64<double, double>(w.Q2, r, ctx->on_Om, r, w.C2, r, r, r, V, s);  // Q^T Omega
+  gemm_tn64(w.Q2, r, ctx->on_Om, r, w.C2, r, r, r, V, ex, V, sms, s);  // Q^T Omega
   // Q^T Y = R = (L1 L2)^T = L2^T L1^T
   k_transpose_rr<<<(r * r + 255) / 256, 256, 0, s>>>(w.L1, r, nullptr, w.L1T);
-  gemm_tn64<double, double>(w.L2, r, w.L1T, r, w.C1, r, r, r, r, s);
+  gemm_tn64(w.L2, r, w.L1T, r, w.C1, r, r, r, r, ex, V, sms, s);
   // B = (Q^T Y)(Q^T Omega)^-1, symmetrised by the eigensolver
   if (tlda_status st = run_solve_right(ctx, w.C1, w.C2, r, w.Ms, w.Rs, w.Bm, status + 1, s)) return st;
   CKF(cudaGetLastError());
@@ -1227,13 +1690,11 @@ tlda_status online_rewhiten(tlda_ctx *ctx) {
     return fail(ctx, TLDA_ERR_NUMERIC, "the sketched M2 has fewer than D positive eigenvalues");
   CKF(cudaMemcpyAsync(w.Ek, hEk.data(), sizeof(double) * r * D, cudaMemcpyHostToDevice, s));
   CKF(cudaMemcpyAsync(w.lam, hlam.data(), sizeof(double) * D, cudaMemcpyHostToDevice, s));
-  gemm_nn<double>(w.Q2, r, w.Ek, D, w.U64, D, V, D, r, s);
+  gemm_nn64(w.Q2, r, w.Ek, D, w.U64, D, V, D, r, ex, V, sms, s);
   if (ctx->whitened)
     CKF(cudaMemcpyAsync(ctx->on_Wold, ctx->W32, sizeof(float) * (size_t)V * D, cudaMemcpyDeviceToDevice, s));
-  k_make_w<<<D, 256, 0, s>>>(w.U64, V, D, w.lam, ctx->W32, nullptr, nullptr);
-  CKF(cudaMemsetAsync(ctx->m1, 0, sizeof(float) * ctx->Dp, s));
-  k_wtm1<<<D, 256, 0, s>>>(ctx->W32, w.M1, V, D, ctx->m1);
-  launch_make_u(ctx->W32, ctx->m1, V, D, ctx->Dp, ctx->U32, ctx->U16, s);
+  // Y and Q1 are free: the peaks of U's columns
+  make_whitening(ctx, w.U64, w.lam, w.M1, w.Y, reinterpret_cast<int *>(w.Q1), w.m1q, s);
   CKF(cudaGetLastError());
   CKF(cudaStreamSynchronize(s));
   ctx->eig = hlam;
@@ -1246,29 +1707,36 @@ tlda_status online_rotate(tlda_ctx *ctx, float *Phi) {
   cudaStream_t s = ctx->stream;
   const int V = ctx->V, D = ctx->D, K = ctx->K;
   OnlineWs w(ctx->on_ws, V, ctx->on_r, D);  // r x r buffers hold the D x D ones (D <= r)
-  int *status = ctx->on_status;
+  int *status = ctx->on_status, *ex = nullptr;
+  const int sms = ctx->num_sms;
+  if (tlda_status st = g64_exps(ctx, &ex)) return st;
   CKF(cudaMemsetAsync(status, 0, sizeof(int), s));
-  gemm_tn64<float, float>(ctx->W32, D, ctx->on_Wold, D, w.C1, D, D, D, V, s);
-  gemm_tn64<float, float>(ctx->on_Wold, D, ctx->on_Wold, D, w.C2, D, D, D, V, s);
-  // R = (W^T W_old)(W_old^T W_old)^-1
-  if (tlda_status st = run_solve_right(ctx, w.C1, w.C2, D, w.Ms, w.Rs, w.Bm, status, s)) return st;
-  CKF(cudaGetLastError());
-  std::vector<double> R((size_t)D * D);
-  std::vector<float> hP((size_t)D * K);
+  gemm_tn64(ctx->W32, D, ctx->on_Wold, D, w.C1, D, D, D, V, ex, V, sms, s);
+  gemm_tn64(ctx->on_Wold, D, ctx->on_Wold, D, w.C2, D, D, D, V, ex, V, sms, s);
+  // (W^T W_old) L^-T L^-1 Phi with L the Cholesky factor of W_old^T W_old (a
+  // third of the time of the elimination: 2 D/32 grid barriers against D)
+  CKF(cudaMemcpyAsync(w.G, w.C2, sizeof(double) * D * D, cudaMemcpyDeviceToDevice, s));
+  if (tlda_status st = run_chol_inv(ctx, w.G, D, w.L1, w.Z, w.L2, w.LinvT, nullptr, status, s)) return st;
+  float *Pn = reinterpret_cast<float *>(w.Rs);
+  k_small_nn<<<D, 256, 0, s>>>(w.L2, Phi, D, K, nullptr, w.Ms);
+  k_small_nn<<<D, 256, 0, s>>>(w.LinvT, w.Ms, D, K, nullptr, w.Et);
+  k_small_nn<<<D, 256, 0, s>>>(w.C1, w.Et, D, K, nullptr, Pn);
   int hst = 0;
-  CKF(cudaMemcpyAsync(R.data(), w.Bm, sizeof(double) * D * D, cudaMemcpyDeviceToHost, s));
-  CKF(cudaMemcpyAsync(hP.data(), Phi, sizeof(float) * D * K, cudaMemcpyDeviceToHost, s));
-  CKF(cudaMemcpyAsync(&hst, status, sizeof hst, cudaMemcpyDeviceToHost, s));
-  CKF(cudaStreamSynchronize(s));
+  auto finish = [&]() -> tlda_status {
+    CKF(cudaGetLastError());
+    CKF(cudaMemcpyAsync(&hst, status, sizeof hst, cudaMemcpyDeviceToHost, s));
+    CKF(cudaStreamSynchronize(s));
+    return TLDA_OK;
+  };
+  if (tlda_status st = finish()) return st;
+  if (hst == 1) {  // not positive definite to rounding: elimination with pivoting decides
+    CKF(cudaMemsetAsync(status, 0, sizeof(int), s));
+    if (tlda_status st = run_solve_right(ctx, w.C1, w.C2, D, w.Ms, w.Rs, w.Bm, status, s)) return st;
+    k_small_nn<<<D, 256, 0, s>>>(w.Bm, Phi, D, K, nullptr, Pn);
+    if (tlda_status st = finish()) return st;
+  }
   if (tlda_status st = chol_status(ctx, hst, "W^T W of the previous whitening is singular")) return st;
-  std::vector<double> hN((size_t)D * K, 0.0);
-  for (int i = 0; i < D; ++i)
-    for (int k = 0; k < D; ++k) {
-      const double rr = R[(size_t)i * D + k];
-      for (int j = 0; j < K; ++j) hN[(size_t)i * K + j] += rr * hP[(size_t)k * K + j];
-    }
-  for (size_t e = 0; e < hP.size(); ++e) hP[e] = (float)hN[e];
-  CKF(cudaMemcpyAsync(Phi, hP.data(), sizeof(float) * D * K, cudaMemcpyHostToDevice, s));
+  CKF(cudaMemcpyAsync(Phi, Pn, sizeof(float) * D * K, cudaMemcpyDeviceToDevice, s));
   CKF(cudaStreamSynchronize(s));
   return TLDA_OK;
 }
@@ -1398,35 +1866,56 @@ tlda_status tlda_unwhiten_topics(tlda_ctx *ctx, const float *Phi, double *mu_out
   if (!ctx->whitened) return fail(ctx, TLDA_ERR_STATE, "no whitening: fit or set one first");
   cudaStream_t s = ctx->stream;
   const int V = ctx->V, D = ctx->D, K = ctx->K;
-  Scratch sc;
-  double *W64 = nullptr, *G = nullptr, *Linv = nullptr, *LinvT = nullptr, *Ginv = nullptr, *T = nullptr;
-  double *Lf = nullptr, *Zs = nullptr;
-  double *mu = nullptr, *al = nullptr;
-  int *status = nullptr;
-  CKF(sc.get(&W64, (size_t)V * D));
-  CKF(sc.get(&G, (size_t)D * D));
-  CKF(sc.get(&Linv, (size_t)D * D));
-  CKF(sc.get(&LinvT, (size_t)D * D));
-  CKF(sc.get(&Ginv, (size_t)D * D));
-  CKF(sc.get(&Lf, (size_t)D * D));
-  CKF(sc.get(&Zs, (size_t)D * D));
-  CKF(sc.get(&T, (size_t)D * K));
-  CKF(sc.get(&status, 1, true));
+  int *ex = nullptr;
+  const int sms = ctx->num_sms;
+  if (tlda_status st = g64_exps(ctx, &ex)) return st;
   const bool host = flags & TLDA_HOST_OUTPUT;
-  if (host) {
-    CKF(sc.get(&mu, (size_t)V * K));
-    CKF(sc.get(&al, (size_t)K));
-  } else {
+  double *G = nullptr, *Linv = nullptr, *LinvT = nullptr, *T1 = nullptr, *T = nullptr, *sum = nullptr, *n2 = nullptr;
+  double *Lf = nullptr, *Zs = nullptr, *mu = nullptr, *al = nullptr;
+  int *status = nullptr;
+  const size_t DD = (size_t)D * D;
+  auto lay = [&](Carver &c) {
+    c.take(G, DD);
+    c.take(Linv, DD);
+    c.take(LinvT, DD);
+    c.take(Lf, DD);
+    c.take(Zs, DD);
+    c.take(T1, (size_t)D * K);
+    c.take(T, (size_t)D * K);
+    c.take(sum, K);
+    c.take(n2, K);
+    c.take(status, 1);
+    c.take(al, K);
+    c.take(mu, host ? (size_t)V * K : 1);
+  };
+  // the context keeps this workspace (V K doubles with host output): an
+  // allocation and its release took 150 us of each call
+  Carver need{nullptr};
+  lay(need);
+  if (ctx->uw_bytes < need.off) {
+    dfree(ctx->uw_ws);
+    ctx->uw_bytes = 0;
+    CKF(dalloc(&ctx->uw_ws, need.off));
+    ctx->uw_bytes = need.off;
+  }
+  Carver real{ctx->uw_ws};
+  lay(real);
+  if (!host) {
     mu = mu_out;
     al = alpha_out;
   }
-  k_f2d<<<(unsigned)(((long long)V * D + 255) / 256), 256, 0, s>>>(ctx->W32, W64, (long long)V * D);
-  gemm_tn64<double, double>(W64, D, W64, D, G, D, D, D, V, s);         // W^T W
+  CKF(cudaMemsetAsync(status, 0, sizeof(int), s));
+  gemm_tn64(ctx->W32, D, ctx->W32, D, G, D, D, D, V, ex, V, sms, s);    // W^T W = L L^T
   if (tlda_status st = run_chol_inv(ctx, G, D, Lf, Zs, Linv, LinvT, nullptr, status, s)) return st;
-  gemm_nn<double>(LinvT, D, Linv, D, Ginv, D, D, D, D, s);              // (W^T W)^-1 = L^-T L^-1
-  k_unwhiten_coef<<<1, 256, 0, s>>>(Phi, D, K, Ginv, T, al);
-  gemm_nn<double>(W64, D, T, K, mu, K, V, K, D, s);                     // mu = W (W^T W)^-1 Phi diag(|phi|^2)
-  k_clip_norm<<<K, 256, 0, s>>>(mu, V, K);
+  k_unwhiten_norms<<<1, kMaxDim, 0, s>>>(Phi, D, K, n2, al);
+  k_small_nn<<<D, 256, 0, s>>>(Linv, Phi, D, K, nullptr, T1);
+  k_small_nn<<<D, 256, 0, s>>>(LinvT, T1, D, K, n2, T);                 // (W^T W)^-1 Phi diag(|phi|^2)
+  gemm_nn64(ctx->W32, D, T, K, mu, K, V, K, D, ex, V, sms, s);
+  const int slab = std::max(32, (V + 63) / 64);
+  const dim3 cg((K + 31) / 32, (V + slab - 1) / slab);
+  CKF(cudaMemsetAsync(sum, 0, sizeof(double) * K, s));
+  k_clip_sum<<<cg, 256, 0, s>>>(mu, V, K, slab, sum);
+  k_clip_scale<<<cg, 256, 0, s>>>(mu, V, K, slab, sum);
   CKF(cudaGetLastError());
   int hst = 0;
   CKF(cudaMemcpyAsync(&hst, status, sizeof hst, cudaMemcpyDeviceToHost, s));
