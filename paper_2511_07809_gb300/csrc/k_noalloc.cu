@@ -20,6 +20,7 @@ constexpr size_t kNoAllocScratchBytes = size_t(8) << 20;
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 constexpr int kNoAllocSplit = 32;
+constexpr int kNoAllocBlocks = 152;  // the SMs of a GB300 (grids stride over the work: any count is right)
 // Largest batch accepted: the scratch cannot hold more documents' rows anyway
 // (each takes at least 3 x 64 FP32 of X, Y and Z), and the bound keeps every
 // size computation below far from int overflow.
@@ -52,11 +53,11 @@ struct Carve {
 
 // Clears what must start at zero (the scratch keeps the previous call's
 // contents, possibly laid out for other sizes) and installs the batch.
-__global__ void k_noalloc_reset(DevState *st, BatchDesc b, float *H, long long nH, int *cnt, int V) {
+__global__ void k_noalloc_reset(DevState *st, BatchDesc b, float *H, long long nH, int *flag, int V) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long e = i; e < nH; e += stride) H[e] = 0.f;
-  for (long long e = i; e < V; e += stride) cnt[e] = 0;
+  for (long long e = i; e < V; e += stride) flag[e] = 0;
   if (i == 0) {
     DevState z{};
     z.cur = b;
@@ -92,11 +93,14 @@ extern "C" tlda_status tlda_cp_step_noalloc(const tlda_csr *batch, const float *
   a.lr = lr;
   a.c3 = (alpha0 + 1.0) * (alpha0 + 2.0) / 2.0;
   a.same_token = 1;
+  a.nrep = 1;
+  a.sms = kNoAllocBlocks;
   a.precision = TLDA_FP32;
   a.Phi = Phi;
   a.grad_out = grad_out;
   a.m1 = m1;
-  // layout of the scratch for these sizes; reject what does not fit
+  // layout of the scratch for these sizes; reject what does not fit (X, Y and Z
+  // are not formed, but their rows stay in the account: what fits is documented)
   auto layout = [&](unsigned char *base) {
     Carve c{base};
     a.st = c.take<DevState>(1);
@@ -108,7 +112,7 @@ extern "C" tlda_status tlda_cp_step_noalloc(const tlda_csr *batch, const float *
     a.Z32 = c.take<float>((size_t)a.Bmax * a.Kp);
     a.Zc32 = c.take<float>((size_t)V * a.Kp);
     a.H32 = c.take<float>((size_t)V * a.Kp);
-    a.cnt = c.take<int>((size_t)V);
+    a.flag = c.take<int>((size_t)V);
     a.widx = c.take<int>((size_t)V);
     a.Gpart = c.take<float>((size_t)a.nsplit * a.Dp * a.Kp);
     a.Gram = c.take<float>((size_t)a.Kp * a.Kp);
@@ -135,16 +139,15 @@ extern "C" tlda_status tlda_cp_step_noalloc(const tlda_csr *batch, const float *
   b.counts = batch->counts;
   b.nz_base = 0;
   b.n_docs = B;
-  k_noalloc_reset<<<64, 256, 0, s>>>(a.st, b, a.H32, (long long)V * a.Kp, a.cnt, V);
+  k_noalloc_reset<<<64, 256, 0, s>>>(a.st, b, a.H32, (long long)V * a.Kp, a.flag, V);
   launch_make_u(W, m1, V, D, a.Dp, U, nullptr, s);
   launch_phi_gram(a, s);
   launch_phi_terms(a, s);
   if (B > 0) {
-    launch_whiten(a, s, nullptr, true);
-    launch_qy_f32(a, s);
-    launch_rz(a, s);
-    launch_zh_f32(a, s);
-    launch_g_f32(a, s);
+    launch_touch(a, s);
+    launch_q_f32(a, s);
+    launch_doc(a, s);
+    launch_gw_f32(a, s);
   }
   launch_reduce_update(a, s);
   if (err_out) k_noalloc_status<<<1, 1, 0, s>>>(a.st, err_out);

@@ -1,20 +1,36 @@
 // Hot-path kernels of the online Tensor LDA CP step (eq. vec_deriv and the SGD
 // update of section "Online Learning of the Third Moment"), plain FP32 form,
-// plus the pieces both precisions share: batch scan + whitening, the
-// touched-word compaction, the Phi-only terms and the final reduction/update.
+// plus the pieces both precisions share: the touched words, batch scan +
+// whitening, the Phi-only terms and the final reduction/update.
 //
 // Per step, with U = W - 1 m1^T (V x D), X = F U, Y = X Phi, Q = U Phi:
-//   a1  L_d, S3, c_m = sum_d f_dm, CSR validation,
-//       touched words {m : c_m > 0}                        k_scan_whiten
-//   a2  X = F U (= F W - L m1^T)                           k_scan_whiten
+//   touched words {m : c_m > 0}, c_m = sum_d f_dm          k_touch
+//   a7/a8  G3, P = Phi (Phi^T Phi * Phi^T Phi)             k_phi_gram, k_phi_terms
+//   a9  grad = E - 3 c3/S3 (G1 + G2), Phi -= lr grad       k_reduce_update
+// where E = 3(1+theta) P - 3 G3, and the data term G1 + G2 in one of two ways.
+//
+// FP32 without the loss: the sums regrouped by word,
+//   a4  Q = U Phi (touched rows)                           k_q_f32
+//   a1  CSR validation, S3;  y_d = sum_j f_j q_j,  r_d = sum_j f_j q_j^2,
+//       z_d = y_d^2 - r_d,  B_m += f_j (z_d + 2 q_j^2 - 2 q_j y_d)   k_doc
+//   a5+a6  G1 + G2 = U^T B over the touched words          k_gw_f32
+// X, Y, Z and their rows of the two products are not formed: the sum is
+// G1 + G2 = sum_j u_j [f_j (z + 2 q_j^2 - 2 q_j y)]^T term by term.
+//
+// With the loss (its FP32 sums keep their order) and in the BF16 form:
+//   a1  L_d, S3, CSR validation;  a2  X = F U (= F W - L m1^T)  k_scan_whiten
 //   a3  Y = X Phi;  a4 Q = U Phi (touched rows)            k_qy_f32
 //   a4  R_d = sum_m f_dm Q_m^2,  Z = Y*Y - R;  H = F^T Y   k_rz
 //   a6  Zc_m = Q_m * (2 c_m Q_m - 2 H_m)                   k_zh_f32
 //   a5+a6  G1 + G2 = X^T Z + U^T Zc (split reduction)      k_g_f32
-//   a7/a8  G3, P = Phi (Phi^T Phi * Phi^T Phi)             k_phi_gram, k_phi_terms
-//   a9  grad = E - 3 c3/S3 (G1 + G2), Phi -= lr grad       k_reduce_update
-// where E = 3(1+theta) P - 3 G3.  Words a batch does not touch have c_m = 0
-// and H_m = 0, so they contribute nothing to G2 and are skipped.
+// Words a batch does not touch have c_m = 0 and H_m = 0 (B_m = 0), so they
+// contribute nothing to G2 and are skipped.
+//
+// H (or B) and c take one add per nonzero.  A word that most documents hold
+// (the head of a Zipf vocabulary) would queue every document's add at one
+// address, so small tables are kept nrep times (StepArgs::nrep): a block adds
+// to one copy, and the reader sums them.
+#include <algorithm>
 #include <cstdio>
 
 #include "tlda_internal.h"
@@ -89,10 +105,88 @@ __device__ __forceinline__ NzChunk load_chunk(const BatchDesc &b, int V, int bas
   return c;
 }
 
+// Whether document row [lo, hi) lies in the batch's nonzero range (the offsets
+// at its first and last document): outside it the row offsets decrease
+// somewhere, and k_touch has not seen the words.
+__device__ __forceinline__ bool row_in_batch(const BatchDesc &b, int lo, int hi, int first, int last) {
+  return lo >= b.nz_base && hi >= lo && lo >= first && hi <= last;
+}
+
+// Touched words of the batch into widx (compact, no fixed order) with flag set.
+// A word's first meeting in a block goes to its flag, the others end at the
+// block's bitmap (a word that most documents hold would else queue thousands of
+// exchanges at one address: 11.7 us a batch of 4096 tweets).  Flat over the nonzeros, 1024 a
+// block and turn; a word already flagged costs one load, not an atomic; one add
+// to n_touched a block and turn.
+constexpr int kTouchBits = 1 << 17;  // words a block's bitmap holds (16 KB); larger vocabularies do without
+__device__ void touch_words(const StepArgs &a, const BatchDesc &b, int *n_touched, int block, int blocks) {
+  if (b.n_docs <= 0) return;
+  const int lo = b.indptr[0], hi = b.indptr[b.n_docs];
+  if (lo < b.nz_base || hi < lo) return;  // corrupt: k_doc / k_scan_whiten report it
+  __shared__ int wsum[8], base;
+  __shared__ unsigned seen[kTouchBits / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const bool small = a.V <= kTouchBits;
+  if ((long long)lo + (long long)block * 1024 >= hi) return;
+  if (small) {
+    for (int i = tid; i < (a.V + 31) / 32; i += 256) seen[i] = 0;
+    __syncthreads();
+  }
+  for (long long j0 = (long long)lo + (long long)block * 1024; j0 < hi; j0 += (long long)blocks * 1024) {
+    int m[4];
+    unsigned fresh = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long long j = j0 + u * 256 + tid;
+      m[u] = j < hi ? __ldg(b.indices + (j - b.nz_base)) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (m[u] < 0 || m[u] >= a.V) continue;
+      if (small) {
+        const unsigned bit = 1u << (m[u] & 31);
+        if (atomicOr(&seen[m[u] >> 5], bit) & bit) continue;
+      }
+      if (*reinterpret_cast<volatile int *>(a.flag + m[u]) == 0 && atomicExch(a.flag + m[u], 1) == 0) fresh |= 1u << u;
+    }
+    const int mine = __popc(fresh);
+    int pre = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, pre, o);
+      if (lane >= o) pre += y;
+    }
+    if (lane == 31) wsum[w] = pre;
+    __syncthreads();
+    if (tid == 0) {
+      int t = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int x = wsum[q];
+        wsum[q] = t;
+        t += x;
+      }
+      base = t ? atomicAdd(n_touched, t) : 0;
+    }
+    __syncthreads();
+    int at = base + wsum[w] + pre - mine;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (fresh & (1u << u)) a.widx[at++] = m[u];
+    __syncthreads();  // wsum, base
+  }
+}
+
+__global__ void __launch_bounds__(256) k_touch(StepArgs a) {
+  touch_words(a, a.st->cur, &a.st->n_touched, blockIdx.x, gridDim.x);
+}
+
+void launch_touch(const StepArgs &a, cudaStream_t s) { k_touch<<<2 * a.sms, 256, 0, s>>>(a); }
+
 // One warp per document: validates the row, accumulates L_d and
-// x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, and (stats)
-// adds c_m, appends first-seen words to the touched list, adds the block's
-// share of S3.  TC=true also writes X in BF16 row-major (X16), whole rows.
+// x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, and (stats) adds
+// c_m to this block's copy and the block's share of S3.  TC=true also writes X in BF16 row-major (X16),
+// whole rows.
 template <int NV, bool TC>
 __global__ void __launch_bounds__(32 * kDocsPerBlock)
     k_scan_whiten(StepArgs a, float *X_out, int stats) {
@@ -104,12 +198,13 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
   __syncthreads();
+  int *cnt = a.cnt + (long long)(blockIdx.x % a.nrep) * a.V;
   float4 acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
   if (d < b.n_docs) {
     const int lo = b.indptr[d], hi = b.indptr[d + 1];
-    bool bad = (lo < b.nz_base) || (hi < lo);
+    bool bad = stats ? !row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs]) : lo < b.nz_base || hi < lo;
     long long lsum = 0;
     int prev = -1;
     if (!bad) {
@@ -118,17 +213,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
         if (__any_sync(0xffffffffu, c.bad)) bad = true;
         prev = __shfl_sync(0xffffffffu, c.in ? c.m : -1, c.n - 1);
         lsum += c.f;
-        if (stats && a.same_token) {
-          bool fresh = false;
-          if (c.f > 0) fresh = atomicAdd(a.cnt + c.m, c.f) == 0;
-          const unsigned nm = __ballot_sync(0xffffffffu, fresh);
-          if (nm) {
-            int t0 = 0;
-            if (lane == 0) t0 = atomicAdd(&a.st->n_touched, __popc(nm));
-            t0 = __shfl_sync(0xffffffffu, t0, 0);
-            if (fresh) a.widx[t0 + __popc(nm & ((1u << lane) - 1u))] = c.m;
-          }
-        }
+        if (stats && a.same_token && c.f > 0) atomicAdd(cnt + c.m, c.f);
         for (int q = 0; q < c.n; q += 4) {
           int mm[4];
           float ff[4];
@@ -405,6 +490,7 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d0 = blockIdx.x * 8, d = d0 + warp;
   if (d0 >= (TC ? round_up(b.n_docs, 64) : b.n_docs)) return;
+  const int K4 = (a.K + 3) & ~3;  // Q, Y and H are zero in the padding columns
   float4 y[NK], r[NK];
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
@@ -413,9 +499,10 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
                                          : f4(0.f);
     r[v] = f4(0.f);
   }
+  float *H = a.H32 + (long long)(blockIdx.x % a.nrep) * a.V * a.Kp;
   if (a.same_token && d < b.n_docs) {
     const int lo = b.indptr[d], hi = b.indptr[d + 1];
-    if (lo >= b.nz_base) {
+    if (row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs])) {
       for (int base = lo; base < hi; base += 32) {
         const NzChunk c = load_chunk(b, a.V, base, hi, lane, -1);
         for (int q = 0; q < c.n; q += 4) {
@@ -435,13 +522,13 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
             const int col = v * 128 + lane * 4;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              qv[v][u] = col < a.Kp ? *reinterpret_cast<const float4 *>(a.Q32 + (long long)mm[u] * a.Kp + col)
+              qv[v][u] = col < K4 ? *reinterpret_cast<const float4 *>(a.Q32 + (long long)mm[u] * a.Kp + col)
                                     : f4(0.f);
           }
 #pragma unroll
           for (int v = 0; v < NK; ++v) {
             const int col = v * 128 + lane * 4;
-            if (col < a.Kp) {
+            if (col < K4) {
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
                 const float ff2 = ff[u];
@@ -450,7 +537,7 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
                 r[v].z = fmaf(ff2 * qv[v][u].z, qv[v][u].z, r[v].z);
                 r[v].w = fmaf(ff2 * qv[v][u].w, qv[v][u].w, r[v].w);
                 if (ff2 != 0.f)
-                  atomicAdd(reinterpret_cast<float4 *>(a.H32 + (long long)mm[u] * a.Kp + col),
+                  atomicAdd(reinterpret_cast<float4 *>(H + (long long)mm[u] * a.Kp + col),
                             make_float4(ff2 * y[v].x, ff2 * y[v].y, ff2 * y[v].z, ff2 * y[v].w));
               }
             }
@@ -485,16 +572,34 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
   }
 }
 
+// c_m and four columns of H_m (or B_m), summed over the copies.
+__device__ __forceinline__ int word_count(const StepArgs &a, int m) {
+  int c = a.cnt[m];
+  if (a.nrep > 1)
+    for (int r = 1; r < a.nrep; ++r) c += a.cnt[(long long)r * a.V + m];
+  return c;
+}
+__device__ __forceinline__ float4 word_sum(const StepArgs &a, int m, int col) {
+  const float4 *p = reinterpret_cast<const float4 *>(a.H32 + (long long)m * a.Kp + col);
+  float4 h = *p;
+  for (int r = 1; r < a.nrep; ++r) {
+    const float4 x = p[(long long)r * a.V * (a.Kp / 4)];
+    h = make_float4(h.x + x.x, h.y + x.y, h.z + x.z, h.w + x.w);
+  }
+  return h;
+}
+
 // ------------------------------------------------------------ a6: Zc rows
 // One warp per touched word (compact slot t): Zc_t = q * (2 c q - 2 H_m); then
-// H_m and c_m are cleared for the next batch (this warp is their only reader).
+// H_m, c_m and the flag are cleared for the next batch (this warp is their only
+// reader).
 template <int NK>
 __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + warp;
   if (t >= a.st->n_touched) return;
   const int m = a.widx[t];
-  const float c = (float)a.cnt[m];
+  const float c = (float)word_count(a, m);
   float ls = 0.f;
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
@@ -502,11 +607,11 @@ __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
     if (col < a.Kp) {
       float4 *hp = reinterpret_cast<float4 *>(a.H32 + (long long)m * a.Kp + col);
       const float4 q = *reinterpret_cast<const float4 *>(a.Q32 + (long long)m * a.Kp + col);
-      const float4 h = *hp;
+      const float4 h = word_sum(a, m, col);
       const float4 z = make_float4(q.x * (2.f * c * q.x - 2.f * h.x), q.y * (2.f * c * q.y - 2.f * h.y),
                                    q.z * (2.f * c * q.z - 2.f * h.z), q.w * (2.f * c * q.w - 2.f * h.w));
       *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = z;
-      *hp = f4(0.f);
+      for (int r = 0; r < a.nrep; ++r) hp[(long long)r * a.V * (a.Kp / 4)] = f4(0.f);
       ls += q.x * q.x * q.x + q.y * q.y * q.y + q.z * q.z * q.z + q.w * q.w * q.w;
     }
   }
@@ -515,7 +620,10 @@ __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
     if (lane == 0) atomicAdd(&a.st->loss_data, 2.0 * (double)c * (double)ls);
   }
   __syncwarp();
-  if (lane == 0) a.cnt[m] = 0;
+  if (lane == 0) {
+    for (int r = 0; r < a.nrep; ++r) a.cnt[(long long)r * a.V + m] = 0;
+    a.flag[m] = 0;
+  }
 }
 
 // ------------------------------------------------------------ a5 + a6: G1 + G2 (FP32)
@@ -610,18 +718,457 @@ void launch_g_f32(const StepArgs &a, cudaStream_t s) {
   k_g_f32<<<g, 256, 0, s>>>(a);
 }
 
+// ------------------------------------------------------------ FP32, by word
+// cp.async of one element (4 bytes) or four (16 bytes); zeros where !in.
+__device__ __forceinline__ void cp4(float *dst, const float *src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp16(float *dst, const float *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf's): half the
+// issue slots of the products below.
+__device__ __forceinline__ uint64_t pair(float x, float y) {
+  uint64_t p;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(x), "f"(y));
+  return p;
+}
+__device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpair(uint64_t p) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
+// Q of the touched words: Q[widx[t]] = U[widx[t]] Phi.  Tiles of 64 touched rows
+// x 16 TN topics (4 x TN outputs a thread), blocks striding over the tiles.  The
+// tile's rows and its part of Phi come to shared memory whole, up to kQDeep
+// features at a time, so that a tile waits for memory once and not once a slab;
+// a block keeps its part of Phi while its tiles share it.
+constexpr int kQDeep = 128, kQRows = 64, kQThreads = 4 * kQRows;
+template <int TN>
+__global__ void __launch_bounds__(kQThreads) k_q_f32(StepArgs a) {
+  constexpr int BN = 16 * TN, LDA = kQDeep + 4;
+  extern __shared__ __align__(16) float q_sm[];
+  float *As = q_sm, *Bs = q_sm + kQRows * LDA;  // rows x LDA; deep x BN
+  const int nt = a.st->n_touched, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int rt = (nt + kQRows - 1) / kQRows, ntn = (a.Kp + BN - 1) / BN, tiles = rt * ntn;
+  const bool wide = (a.K & 3) == 0 && (reinterpret_cast<uintptr_t>(a.Phi) & 15) == 0;
+  int kept = -1;  // the column tile whose Phi is in Bs (D <= kQDeep)
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int r0 = tile % rt * kQRows, nn = tile / rt, n0 = nn * BN;
+    uint64_t acc[4][TN / 2];  // pairs of topics
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0;
+    for (int d0 = 0; d0 < a.D; d0 += kQDeep) {
+      const int deep = min(kQDeep, (a.D - d0 + 3) & ~3);  // U is zero from D to Dp
+      __syncthreads();  // the slab before has been read
+      for (int e = tid; e < kQRows * (deep / 4); e += kQThreads) {
+        const int r = e / (deep / 4), k = e % (deep / 4) * 4;
+        const bool in = r0 + r < nt;
+        cp16(As + r * LDA + k, in ? a.U32 + (long long)a.widx[r0 + r] * a.Dp + d0 + k : a.U32, in);
+      }
+      if (kept != nn || a.D > kQDeep) {
+        if (wide) {
+          for (int e = tid; e < deep * (BN / 4); e += kQThreads) {
+            const int k = e / (BN / 4), n = e % (BN / 4) * 4;
+            const bool in = d0 + k < a.D && n0 + n < a.K;
+            cp16(Bs + k * BN + n, in ? a.Phi + (long long)(d0 + k) * a.K + n0 + n : a.Phi, in);
+          }
+        } else {
+          for (int e = tid; e < deep * BN; e += kQThreads) {
+            const int k = e / BN, n = e % BN;
+            const bool in = d0 + k < a.D && n0 + n < a.K;
+            cp4(Bs + k * BN + n, in ? a.Phi + (long long)(d0 + k) * a.K + n0 + n : a.Phi, in);
+          }
+        }
+        kept = nn;
+      }
+      cp_commit();
+      cp_wait<0>();
+      __syncthreads();
+#pragma unroll 2
+      for (int k = 0; k < deep; k += 4) {
+        float x[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 v = *reinterpret_cast<const float4 *>(As + (ty * 4 + i) * LDA + k);
+          x[i][0] = v.x, x[i][1] = v.y, x[i][2] = v.z, x[i][3] = v.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint64_t br[TN / 2];
+#pragma unroll
+          for (int j = 0; j < TN; j += 4) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(Bs + (k + q) * BN + (j / 4) * 64 + tx * 4);
+            br[j / 2] = v.x, br[j / 2 + 1] = v.y;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint64_t xx = pair(x[i][q], x[i][q]);
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], xx, br[j]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + ty * 4 + i;
+      if (r >= nt) continue;
+      float *op = a.Q32 + (long long)a.widx[r] * a.Kp;
+#pragma unroll
+      for (int j = 0; j < TN; j += 4) {
+        const int n = n0 + (j / 4) * 64 + tx * 4;
+        const float2 lo = unpair(acc[i][j / 2]), hi = unpair(acc[i][j / 2 + 1]);
+        if (n < a.Kp) *reinterpret_cast<float4 *>(op + n) = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
+    }
+  }
+}
+
+void launch_q_f32(const StepArgs &a, cudaStream_t s) {
+  const int deep = std::min(kQDeep, (a.D + 3) & ~3), rt = (a.V + kQRows - 1) / kQRows;
+#define TLDA_Q(TNv, blocks)                                                                               \
+  {                                                                                                       \
+    const int smem = (kQRows * (kQDeep + 4) + deep * 16 * TNv) * (int)sizeof(float);                          \
+    static const cudaError_t attr = cudaFuncSetAttribute(                                                 \
+        k_q_f32<TNv>, cudaFuncAttributeMaxDynamicSharedMemorySize, (kQRows * (kQDeep + 4) + kQDeep * 16 * TNv) * 4); \
+    (void)attr;                                                                                           \
+    k_q_f32<TNv><<<std::min(blocks * a.sms, rt * ((a.Kp + 16 * TNv - 1) / (16 * TNv))), kQThreads, smem, s>>>(a); \
+  }
+  if (a.Kp <= 64) TLDA_Q(4, 3)
+  else TLDA_Q(8, 2)
+#undef TLDA_Q
+}
+
+// One warp per document, striding: the row's validation, S3, then over its Q rows
+// y = sum f q and r = sum f q^2 (z = y^2 - r; r = 0 without the same-token
+// correction), and B_m += f (z + 2 q^2 - 2 q y) (f z without it) by vector adds
+// into this block's copy.  The rows come by cp.async into the warp's shared
+// memory, R of them at once: all of a short document's rows are in flight
+// together and are read twice there; a longer one gathers its rows again.
+template <int NK>
+__global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R) {
+  extern __shared__ __align__(16) float doc_rows[];
+  const BatchDesc b = a.st->cur;
+  if (b.n_docs <= 0) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int K4 = (a.K + 3) & ~3;  // the padding columns are zero and stay so
+  float *rows = doc_rows + (long long)warp * R * K4;
+  float *B = a.H32 + (long long)(blockIdx.x % a.nrep) * a.V * a.Kp;
+  const int first = b.indptr[0], last = b.indptr[b.n_docs];
+  __shared__ unsigned long long s3;
+  if (threadIdx.x == 0) s3 = 0;
+  __syncthreads();
+  for (int d = blockIdx.x * 8 + warp; d < b.n_docs; d += gridDim.x * 8) {
+    const int lo = b.indptr[d], hi = b.indptr[d + 1];
+    if (!row_in_batch(b, lo, hi, first, last)) {
+      if (lane == 0) atomicOr(&a.st->err, kErrCsr);
+      continue;
+    }
+    bool bad = false;
+    long long L = 0;
+    float4 y[NK], r[NK];
+#pragma unroll
+    for (int v = 0; v < NK; ++v) y[v] = r[v] = f4(0.f);
+    // rows [s0, s0 + n) of a chunk of nonzeros into shared memory
+    auto stage = [&](const NzChunk &c, int s0, int n) {
+      for (int j0 = 0; j0 < n; j0 += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = min(j0 + u, n - 1);
+          const float *src = a.Q32 + (long long)__shfl_sync(0xffffffffu, c.m, s0 + j) * a.Kp + lane * 4;
+          const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(rows + j * K4 + lane * 4));
+#pragma unroll
+          for (int v = 0; v < NK; ++v)
+            if (j0 + u < n && v * 128 + lane * 4 < K4)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + v * 512), "l"(src + v * 128) : "memory");
+        }
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+    };
+    const bool once = hi - lo <= min(R, 32);
+    NzChunk c{};
+    int prev = -1;
+    for (int base = lo; base < hi; base += 32) {
+      c = load_chunk(b, a.V, base, hi, lane, prev);
+      bad |= __any_sync(0xffffffffu, c.bad);
+      prev = __shfl_sync(0xffffffffu, c.in ? c.m : -1, c.n - 1);
+      L += c.f;
+      for (int s0 = 0; s0 < c.n; s0 += R) {
+        const int n = min(R, c.n - s0);
+        __syncwarp();  // the rows before have been read
+        stage(c, s0, n);
+        for (int j0 = 0; j0 < n; j0 += 4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {  // past the end: the last row with count 0
+            const int j = min(j0 + u, n - 1);
+            const float f = j0 + u < n ? (float)__shfl_sync(0xffffffffu, c.f, s0 + j) : 0.f;
+#pragma unroll
+            for (int v = 0; v < NK; ++v) {
+              const int col = v * 128 + lane * 4;
+              if (col < K4) {
+                const float4 q = *reinterpret_cast<const float4 *>(rows + j * K4 + col);
+                y[v] = fma4(f, q, y[v]);
+                r[v].x = fmaf(f * q.x, q.x, r[v].x);
+                r[v].y = fmaf(f * q.y, q.y, r[v].y);
+                r[v].z = fmaf(f * q.z, q.z, r[v].z);
+                r[v].w = fmaf(f * q.w, q.w, r[v].w);
+              }
+            }
+          }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    if (lane == 0) {
+      if (bad) atomicOr(&a.st->err, kErrCsr);
+      if (L >= 3) atomicAdd(&s3, (unsigned long long)(L * (L - 1) * (L - 2)));
+    }
+    const float on = a.same_token ? 1.f : 0.f;
+    float4 z[NK];
+#pragma unroll
+    for (int v = 0; v < NK; ++v)
+      z[v] = make_float4(fmaf(y[v].x, y[v].x, -on * r[v].x), fmaf(y[v].y, y[v].y, -on * r[v].y),
+                         fmaf(y[v].z, y[v].z, -on * r[v].z), fmaf(y[v].w, y[v].w, -on * r[v].w));
+    const float two = 2.f * on;
+    for (int base = lo; base < hi; base += 32) {
+      if (!once) c = load_chunk(b, a.V, base, hi, lane, -1);
+      for (int s0 = 0; s0 < c.n; s0 += R) {
+        const int n = min(R, c.n - s0);
+        if (!once) {
+          __syncwarp();
+          stage(c, s0, n);
+        }
+        for (int j0 = 0; j0 < n; j0 += 4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int j = min(j0 + u, n - 1);
+            const int m = __shfl_sync(0xffffffffu, c.m, s0 + j);
+            const float f = j0 + u < n ? (float)__shfl_sync(0xffffffffu, c.f, s0 + j) : 0.f;
+            if (f == 0.f) continue;
+#pragma unroll
+            for (int v = 0; v < NK; ++v) {
+              const int col = v * 128 + lane * 4;
+              if (col < K4) {
+                const float4 q = *reinterpret_cast<const float4 *>(rows + j * K4 + col);
+                atomicAdd(reinterpret_cast<float4 *>(B + (long long)m * a.Kp + col),
+                          make_float4(f * fmaf(two * q.x, q.x - y[v].x, z[v].x), f * fmaf(two * q.y, q.y - y[v].y, z[v].y),
+                                      f * fmaf(two * q.z, q.z - y[v].z, z[v].z), f * fmaf(two * q.w, q.w - y[v].w, z[v].w)));
+              }
+            }
+          }
+      }
+    }
+    __syncwarp();  // the next document's rows
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s3) atomicAdd(&a.st->S3, s3);
+}
+
+// Rows staged at once: 6.9 KB a warp (17 at K = 100, 32 up to 53 topics), so that
+// four blocks of 8 warps fit an SM.
+constexpr int kDocBytes = 6912;
+void launch_doc(const StepArgs &a, cudaStream_t s) {
+  const int K4 = (a.K + 3) & ~3, nk = (a.Kp + 127) / 128;
+  const int R = std::max(3, std::min(32, kDocBytes / (K4 * 4)));
+  const int smem = 8 * R * K4 * (int)sizeof(float);
+  const int grid = std::max(1, std::min((a.Bmax + 7) / 8, 4 * a.sms));
+#define TLDA_DOC(NKv)                                                                                  \
+  if (nk == NKv) {                                                                                     \
+    static const cudaError_t attr =                                                                    \
+        cudaFuncSetAttribute(k_doc<NKv>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kDocBytes);       \
+    (void)attr;                                                                                        \
+    k_doc<NKv><<<grid, 256, smem, s>>>(a, R);                                                          \
+    return;                                                                                            \
+  }
+  TLDA_DOC(1) TLDA_DOC(2) TLDA_DOC(3) TLDA_DOC(4)
+#undef TLDA_DOC
+}
+
+// Rows t of B summed over the copies into the compact Zc32 (D or K above 128:
+// several blocks of k_gw_f32 read a row); launch_h_clear clears them afterwards.
+__global__ void __launch_bounds__(256) k_b_fold(StepArgs a) {
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
+    const int m = a.widx[t];
+    for (int col = lane * 4; col < a.Kp; col += 128)
+      *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = word_sum(a, m, col);
+  }
+}
+
+// G1 + G2 = U^T B as a split reduction over the touched rows: block (s, ti, tn)
+// sums the rows of split s into a tile of BI features x BN topics of partial s,
+// TM x 4 outputs a thread (a warp shares its features; 16 warps at 128 x 128).  Slabs of 16 rows pass through a ring of
+// `stages` in shared memory by cp.async: a split has some 90 rows at the usual
+// batch sizes, and most of them are requested at once (a slab's arithmetic is
+// shorter than a round trip to L2).  FOLD: one tile covers D and K (both at most
+// 128), so each row of B has one reader: it sums the copies itself, and clears
+// them and the flag for the next batch.
+constexpr int kGwRows = 16;
+template <int BI, int BN, int TM, bool FOLD>
+__global__ void __launch_bounds__(BI / TM * (BN / 4)) k_gw_f32(StepArgs a, int stages) {
+  constexpr int TN = 4, TX = BN / TN, NT = BI / TM * TX, BR = kGwRows;
+  extern __shared__ __align__(16) float gw_sm[];
+  const int reps = FOLD ? a.nrep : 1, stage = BR * (BI + reps * BN);
+  const int nt = a.st->n_touched, tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int s = blockIdx.x, i0 = blockIdx.y * BI, n0 = blockIdx.z * BN;
+  const int rb = (int)((long long)nt * s / a.nsplit), re = (int)((long long)nt * (s + 1) / a.nsplit);
+  const int slabs = (re - rb + BR - 1) / BR;
+  uint64_t acc[TM / 2][TN];  // pairs of features
+#pragma unroll
+  for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0;
+  auto request = [&](int q) {  // slab q into its stage (a group is committed in any case)
+    if (q < slabs) {
+      float *A = gw_sm + (q % stages) * stage, *B = A + BR * BI;
+      const int r0 = rb + q * BR;
+#pragma unroll
+      for (int i = 0; i < BR * BI / 4 / NT; ++i) {
+        const int e = tid + i * NT, r = r0 + e / (BI / 4), c = e % (BI / 4) * 4;
+        const bool in = r < re && i0 + c < a.Dp;
+        cp16(A + e * 4, in ? a.U32 + (long long)a.widx[r] * a.Dp + i0 + c : a.U32, in);
+      }
+      for (int p = 0; p < reps; ++p)
+#pragma unroll
+        for (int i = 0; i < BR * BN / 4 / NT; ++i) {
+          const int e = tid + i * NT, r = r0 + e / (BN / 4), c = e % (BN / 4) * 4;
+          const bool in = r < re && n0 + c < a.Kp;
+          const float *src = a.Zc32;
+          if (in) src = FOLD ? a.H32 + ((long long)p * a.V + a.widx[r]) * a.Kp + n0 + c : a.Zc32 + (long long)r * a.Kp + n0 + c;
+          cp16(B + p * BR * BN + e * 4, src, in);
+        }
+    }
+    cp_commit();
+  };
+  for (int q = 0; q < stages - 1; ++q) request(q);
+  for (int q = 0; q < slabs; ++q) {
+    // all but the newest stages - 2 groups are there: slab q among them
+    switch (stages) {
+      case 6: cp_wait<4>(); break;
+      case 5: cp_wait<3>(); break;
+      case 4: cp_wait<2>(); break;
+      case 3: cp_wait<1>(); break;
+      default: cp_wait<0>(); break;
+    }
+    __syncthreads();
+    request(q + stages - 1);  // into the stage of slab q - 1, which has been read
+    float *A = gw_sm + (q % stages) * stage, *B = A + BR * BI;
+    if (FOLD) {
+      const int r0 = rb + q * BR;
+#pragma unroll
+      for (int i = 0; i < BR * BN / 4 / NT; ++i) {
+        const int e = tid + i * NT, r = r0 + e / (BN / 4), c = e % (BN / 4) * 4;
+        if (reps > 1) {
+          float4 v = *reinterpret_cast<float4 *>(B + e * 4);
+          for (int p = 1; p < reps; ++p) {
+            const float4 x = *reinterpret_cast<const float4 *>(B + p * BR * BN + e * 4);
+            v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
+          }
+          *reinterpret_cast<float4 *>(B + e * 4) = v;
+        }
+        if (r < re && c < a.Kp) {
+          const int m = a.widx[r];
+          for (int p = 0; p < reps; ++p)
+            *reinterpret_cast<float4 *>(a.H32 + ((long long)p * a.V + m) * a.Kp + c) = f4(0.f);
+          if (c == 0) a.flag[m] = 0;
+        }
+      }
+      if (reps > 1) __syncthreads();
+    }
+#pragma unroll
+    for (int rr = 0; rr < BR; ++rr) {
+      uint64_t x[TM / 2];
+#pragma unroll
+      for (int i = 0; i < TM; i += 4) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(A + rr * BI + (i / 4) * (BI / TM * 4) + ty * 4);
+        x[i / 2] = v.x, x[i / 2 + 1] = v.y;
+      }
+      const float4 v = *reinterpret_cast<const float4 *>(B + rr * BN + tx * 4);
+      const uint64_t w[4] = {pair(v.x, v.x), pair(v.y, v.y), pair(v.z, v.z), pair(v.w, v.w)};
+#pragma unroll
+      for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) fma2(acc[i][j], x[i], w[j]);
+    }
+  }
+  cp_wait<0>();
+  float *gp = a.Gpart + (long long)s * a.Dp * a.Kp;
+#pragma unroll
+  for (int i = 0; i < TM; i += 2) {
+    const int row = i0 + (i / 4) * (BI / TM * 4) + ty * 4 + (i & 3), n = n0 + tx * 4;
+    const float2 u[4] = {unpair(acc[i / 2][0]), unpair(acc[i / 2][1]), unpair(acc[i / 2][2]), unpair(acc[i / 2][3])};
+    if (row < a.D && n < a.K)
+      *reinterpret_cast<float4 *>(gp + (long long)row * a.Kp + n) = make_float4(u[0].x, u[1].x, u[2].x, u[3].x);
+    if (row + 1 < a.D && n < a.K)
+      *reinterpret_cast<float4 *>(gp + (long long)(row + 1) * a.Kp + n) = make_float4(u[0].y, u[1].y, u[2].y, u[3].y);
+  }
+}
+
+// Partial sums: one block an SM over the tiles, at least 8.
+int gw_splits(int Dp, int Kp, int sms) {
+  const int tiles = ((Dp + 127) / 128) * ((Kp + 127) / 128);
+  return std::max(8, sms / tiles);
+}
+
+template <int BI, int BN, int TM, bool FOLD>
+void gw_launch(const StepArgs &a, dim3 grid, cudaStream_t s) {
+  const int stage = kGwRows * (BI + (FOLD ? a.nrep : 1) * BN) * (int)sizeof(float);
+  const int stages = std::max(2, std::min(6, 98304 / stage));
+  static const cudaError_t attr = cudaFuncSetAttribute(k_gw_f32<BI, BN, TM, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       147456);
+  (void)attr;
+  k_gw_f32<BI, BN, TM, FOLD><<<grid, BI / TM * (BN / 4), stages * stage, s>>>(a, stages);
+}
+
+void launch_gw_f32(const StepArgs &a, cudaStream_t s) {
+  if (a.Dp <= 64) {
+    gw_launch<64, 64, 4, true>(a, dim3(a.nsplit), s);
+  } else if (a.Dp <= 128 && a.Kp <= 64) {
+    gw_launch<128, 64, 8, true>(a, dim3(a.nsplit), s);
+  } else if (a.Dp <= 128) {
+    gw_launch<128, 128, 8, true>(a, dim3(a.nsplit), s);
+  } else {
+    k_b_fold<<<4 * a.sms, 256, 0, s>>>(a);
+    gw_launch<128, 128, 8, false>(a, dim3(a.nsplit, (a.Dp + 127) / 128, (a.Kp + 127) / 128), s);
+    launch_h_clear(a, s);
+  }
+}
+
 // ------------------------------------------------------------ a9: reduce + update
 // 32 entries (i, n) per block, the partial sums split over 8 warps:
 // g = sum over partials; grad = E - 3 c3/S3 g; Phi -= lr grad (skipped on a
 // sticky error or S3 = 0); the BF16 Phi^T image follows Phi.
+// Blocks past the entries (a.touch_next of them) take the next batch of a pass
+// meanwhile and find its touched words: the flags are clear by now, and nothing
+// of that depends on Phi.
 __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
   DevState *st = a.st;
+  const int entry_blocks = (a.D * a.K + 31) / 32;
+  if ((int)blockIdx.x >= entry_blocks && st->descs && st->pass_pos < st->n_descs)
+    touch_words(a, st->descs[st->pass_pos], &st->n_touched_next, blockIdx.x - entry_blocks, a.touch_next);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
   const unsigned long long S3 = st->S3;
   const int err = st->err;
   const double scale = S3 ? a.c3 / (double)S3 : 0.0;
-  const bool live = e < a.D * a.K;
+  const bool live = (int)blockIdx.x < entry_blocks && e < a.D * a.K;
   const int i = live ? e / a.K : 0, n = live ? e % a.K : 0;
   const long long off = (long long)i * a.Kp + n, stride = (long long)a.Dp * a.Kp;
   float part = 0.f;
@@ -656,28 +1203,28 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
       if (a.PhiImg) a.PhiImg[phi_img_index(n, i, a.Kp)] = __float2bfloat16_rn(phi);
     }
   }
-}
-
-// End of a step (one warp, after the reduction): the step's loss, the
-// per-step sums cleared for the next batch, the step counter, and the next
-// batch descriptor of a pass.
-__global__ void k_step_end(StepArgs a) {
-  DevState *st = a.st;
-  if (threadIdx.x != 0) return;
-  const unsigned long long S3 = st->S3;
-  const double scale = S3 ? a.c3 / (double)S3 : 0.0;
-  st->loss = S3 ? st->loss_phi - scale * st->loss_data : 0.0;
-  st->last_S3 = S3;
-  st->S3 = 0;
-  st->loss_data = 0.0;
-  st->n_touched = 0;
-  st->step += 1;
-  if (st->descs && st->pass_pos < st->n_descs) st->cur = st->descs[st->pass_pos++];
+  // the last block to get here (every block has read the step's sums) ends the
+  // step: its loss, the sums cleared for the next batch, the step counter, and
+  // the next batch descriptor of a pass
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&st->done, 1u) == gridDim.x - 1) {
+      __threadfence();
+      st->done = 0;
+      st->loss = S3 ? st->loss_phi - scale * st->loss_data : 0.0;
+      st->last_S3 = S3;
+      st->S3 = 0;
+      st->loss_data = 0.0;
+      st->n_touched = st->n_touched_next;
+      st->n_touched_next = 0;
+      st->step += 1;
+      if (st->descs && st->pass_pos < st->n_descs) st->cur = st->descs[st->pass_pos++];
+    }
+  }
 }
 
 void launch_reduce_update(const StepArgs &a, cudaStream_t s) {
-  k_reduce_update<<<(a.D * a.K + 31) / 32, 256, 0, s>>>(a);
-  k_step_end<<<1, 32, 0, s>>>(a);
+  k_reduce_update<<<(a.D * a.K + 31) / 32 + a.touch_next, 256, 0, s>>>(a);
 }
 
 }  // namespace tlda

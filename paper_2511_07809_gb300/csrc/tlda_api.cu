@@ -86,6 +86,9 @@ StepArgs make_args(tlda_ctx *c) {
   a.Zc32 = c->Zc32;
   a.H32 = c->H32;
   a.cnt = c->cnt;
+  a.flag = c->flag;
+  a.nrep = c->nrep;
+  a.sms = c->num_sms;
   a.widx = c->widx;
   a.Gpart = c->Gpart;
   a.Gram = c->Gram;
@@ -147,23 +150,48 @@ struct Prof {
   }
 };
 
+// The FP32 form without the loss takes its data term regrouped by word.
+bool by_word(const StepArgs &a) { return a.precision == TLDA_FP32 && !a.want_loss; }
+
+// Whether a step needs the touched words.
+bool wants_touch(const tlda_ctx *ctx, const StepArgs &a) {
+  return !(a.precision == TLDA_BF16 && ctx->fused) && (by_word(a) || a.same_token);
+}
+
 // Enqueues one CP step on ctx->stream for the batch in st->cur: the Phi-only
 // terms on the side stream, the data-term chain on the main stream, then the
 // reduction and update once both are done.
-tlda_status enqueue_step(tlda_ctx *ctx, const StepArgs &a, cudaStream_t main) {
+// With `touched`, the batch's touched words are there already (an earlier step's
+// reduction kernel or the caller found them).
+tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false) {
   const bool tc = a.precision == TLDA_BF16;
-  CK(cudaEventRecord(ctx->ev_fork, main));
-  CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
-  { Prof p(ctx, kPhiGram, ctx->side); launch_phi_gram(a, ctx->side); }
-  { Prof p(ctx, kPhiTerms, ctx->side); launch_phi_terms(a, ctx->side); }
-  CKL();
-  CK(cudaEventRecord(ctx->ev_join, ctx->side));
+  auto fork_phi = [&]() -> tlda_status {
+    CK(cudaEventRecord(ctx->ev_fork, main));
+    CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+    { Prof p(ctx, kPhiGram, ctx->side); launch_phi_gram(a, ctx->side); }
+    { Prof p(ctx, kPhiTerms, ctx->side); launch_phi_terms(a, ctx->side); }
+    CKL();
+    CK(cudaEventRecord(ctx->ev_join, ctx->side));
+    return TLDA_OK;
+  };
+  // beside k_doc in the FP32 form by word (its warps wait for memory), not beside
+  // the product before it
+  if (tc || !by_word(a))
+    if (tlda_status s = fork_phi()) return s;
   if (tc && ctx->fused) {
     // the fused kernel fills its SMs' shared memory: it leaves kPhiSMs SMs
     // free so the side stream's Phi-only kernels run beside it
     Prof p(ctx, kFused, main);
     launch_fused(a, main, ctx->fused_grid);
+  } else if (by_word(a)) {
+    a.nsplit = ctx->nsplit_w;
+    if (!touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
+    { Prof p(ctx, kQY, main); launch_q_f32(a, main); }
+    if (tlda_status s = fork_phi()) return s;
+    { Prof p(ctx, kRZ, main); launch_doc(a, main); }
+    { Prof p(ctx, kG, main); launch_gw_f32(a, main); }
   } else {
+    if (a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
     { Prof p(ctx, kWhiten, main); launch_whiten(a, main, nullptr, true); }
     { Prof p(ctx, kQY, main); if (tc) launch_qy_tc(a, main); else launch_qy_f32(a, main); }
     { Prof p(ctx, kRZ, main); launch_rz(a, main); }
@@ -617,6 +645,11 @@ tlda_status tlda_create(tlda_ctx **out, int32_t vocab, const tlda_params *p, voi
   ctx->nsplit_tc = std::max(8, std::min(64, ctx->num_sms / ((ctx->Dp + 127) / 128)));
   ctx->fused = p->precision == TLDA_BF16 && fused_supported(ctx->Dp, ctx->Kp) && !getenv("TLDA_NO_FUSED");
   ctx->fused_grid = std::max(1, ctx->num_sms - 8);
+  ctx->nsplit_w = gw_splits(ctx->Dp, ctx->Kp, ctx->num_sms);
+  // copies of the per-word sums: more for small tables, whose few words take
+  // many adds each
+  const size_t table = V * Kp * sizeof(float);
+  ctx->nrep = table <= (2u << 20) ? 4 : table <= (5u << 20) ? 2 : 1;
   CA(dalloc(&ctx->W32, V * D, true));
   CA(dalloc(&ctx->m1, Dp, true));
   CA(dalloc(&ctx->U32, V * Dp, true));
@@ -625,12 +658,13 @@ tlda_status tlda_create(tlda_ctx **out, int32_t vocab, const tlda_params *p, voi
   CA(dalloc(&ctx->Y32, Bm * Kp, true));
   CA(dalloc(&ctx->Z32, Bm * Kp, true));
   CA(dalloc(&ctx->Zc32, V * Kp, true));
-  CA(dalloc(&ctx->H32, V * Kp, true));
-  CA(dalloc(&ctx->cnt, V, true));
+  CA(dalloc(&ctx->H32, ctx->nrep * V * Kp, true));
+  CA(dalloc(&ctx->cnt, ctx->nrep * V, true));
+  CA(dalloc(&ctx->flag, V, true));
   CA(dalloc(&ctx->widx, V, true));
   // partial sums; the pass kernel's slice-blocked layout needs up to
   // blocks x (D K + 4 blocks) floats
-  CA(dalloc(&ctx->Gpart, (size_t)std::max({ctx->nsplit, ctx->nsplit_tc, ctx->num_sms}) * Dp * Kp +
+  CA(dalloc(&ctx->Gpart, (size_t)std::max({ctx->nsplit, ctx->nsplit_tc, ctx->nsplit_w, ctx->num_sms}) * Dp * Kp +
                              4 * (size_t)ctx->num_sms * ctx->num_sms, true));
   CA(dalloc(&ctx->Gram, Kp * Kp, true));
   CA(dalloc(&ctx->avec, Kp, true));
@@ -671,7 +705,7 @@ tlda_status tlda_destroy(tlda_ctx *ctx) {
   ctx->U16 = nullptr;
   if (ctx->tc_maps) tc_free_maps(ctx->tc_maps);
   dfree(ctx->X32); dfree(ctx->Q32); dfree(ctx->Y32); dfree(ctx->Z32); dfree(ctx->Zc32);
-  dfree(ctx->H32); dfree(ctx->cnt); dfree(ctx->widx); dfree(ctx->Gpart); dfree(ctx->Gram);
+  dfree(ctx->H32); dfree(ctx->cnt); dfree(ctx->flag); dfree(ctx->widx); dfree(ctx->Gpart); dfree(ctx->Gram);
   dfree(ctx->avec); dfree(ctx->E); dfree(ctx->G3); dfree(ctx->ZU16); dfree(ctx->Z16); dfree(ctx->PhiImg);
   dfree(ctx->st); dfree(ctx->descs); dfree(ctx->splits); dfree(ctx->P64); dfree(ctx->Ccnt);
   dfree(ctx->TS); dfree(ctx->fit_err); dfree(ctx->stage[0]); dfree(ctx->stage[1]);
@@ -867,17 +901,26 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
   if (loss_out && !no_wait) CK(cudaMallocHost(reinterpret_cast<void **>(&losses), sizeof(double) * n_batches));
   launch_begin_pass(ctx->st, ctx->descs, n_batches, ps);
   if (a.PhiImg) launch_phi_img(a, ps);
+  // device input: each step's reduction kernel finds the next batch's touched
+  // words beside its own work, the first batch's are found here (with host input
+  // the next batch is copied only after the step)
+  const bool ahead = !host && wants_touch(ctx, a);
+  if (ahead) {
+    a.touch_next = std::max(32, std::min(2 * ctx->num_sms, ctx->Bmax / 64));  // 16 nonzeros a document: one turn each
+    launch_touch(a, ps);
+  }
   CKL();
   // one captured step, replayed per batch (not while the event profiler is on)
   const bool use_graph = ctx->prof_mask == 0;
-  if (use_graph && !(ctx->step_exec && ctx->g_lr == lr && ctx->g_phi == Phi && ctx->g_loss == a.want_loss)) {
+  if (use_graph && !(ctx->step_exec && ctx->g_lr == lr && ctx->g_phi == Phi && ctx->g_loss == a.want_loss &&
+                     ctx->g_touch == a.touch_next)) {
     if (ctx->step_exec) {
       cudaGraphExecDestroy(ctx->step_exec);
       ctx->step_exec = nullptr;
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(ps, cudaStreamCaptureModeThreadLocal));
-    tlda_status cs = enqueue_step(ctx, a, ps);
+    tlda_status cs = enqueue_step(ctx, a, ps, ahead);
     cudaError_t ce = cudaStreamEndCapture(ps, &g);
     if (cs) {
       if (g) cudaGraphDestroy(g);
@@ -890,6 +933,7 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
     ctx->g_lr = lr;
     ctx->g_phi = Phi;
     ctx->g_loss = a.want_loss;
+    ctx->g_touch = a.touch_next;
   }
   for (int b = 0; b < n_batches && s == TLDA_OK; ++b) {
     if (host) {
@@ -907,7 +951,7 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
       }
     }
     if (use_graph) CK(cudaGraphLaunch(ctx->step_exec, ps));
-    else s = enqueue_step(ctx, a, ps);
+    else s = enqueue_step(ctx, a, ps, ahead);
     if (loss_out && s == TLDA_OK)
       CK(cudaMemcpyAsync(no_wait ? loss_out + b : losses + b, &ctx->st->loss, sizeof(double),
                          no_wait ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ps));

@@ -55,6 +55,8 @@ struct DevState {
   double loss_data;              // sum_d sum_i (y^3 - 3 y r) + 2 sum_m c_m sum_i q^3
   double loss_phi;               // (1+theta)/2 sum G^3 - sum_i (3 a_i |phi_i|^2 - 2 a_i^3)
   double loss;                   // loss of the last completed step
+  int32_t n_touched_next;        // the same of the next batch, while the reduction kernel finds them
+  unsigned int done;             // blocks of the reduction kernel that are done (0 between steps)
 };
 
 // Control block of one persistent-pass launch (zeroed before the launch).
@@ -118,9 +120,12 @@ struct StepArgs {
   float *Y32;                    // Bmax x Kp
   float *Z32;                    // Bmax x Kp: Y*Y - R
   float *Zc32;                   // V x Kp: compact rows Q*(2cQ - 2H) of the touched words
-  float *H32;                    // V x Kp, zero between steps
-  int *cnt;                      // V, zero between steps (c_m = sum_d f_dm)
+  int nrep, sms;                 // copies of H32 and cnt (a block adds to one, the reader sums them); SMs
+  float *H32;                    // nrep x V x Kp, zero between steps (H, or B of the FP32 form without loss)
+  int *cnt;                      // nrep x V, zero between steps (c_m = sum_d f_dm)
+  int *flag;                     // V, zero between steps: the word is in widx
   int *widx;                     // V: touched words of the batch, compact
+  int touch_next;                // blocks of the reduction kernel that find the next batch's touched words
   float *Gpart;                  // nsplit x Dp x Kp
   float *Gram;                   // Kp x Kp: Phi^T Phi
   float *avec;                   // Kp: m1^T Phi
@@ -198,9 +203,10 @@ struct tlda_ctx {
   // step workspace
   float *X32 = nullptr, *Q32 = nullptr, *Y32 = nullptr, *Z32 = nullptr, *Zc32 = nullptr;
   float *H32 = nullptr;
-  int *cnt = nullptr, *widx = nullptr;
+  int *cnt = nullptr, *flag = nullptr, *widx = nullptr;
+  int nrep = 1;                  // copies of H32 and cnt
   float *Gpart = nullptr, *Gram = nullptr, *avec = nullptr, *E = nullptr, *G3 = nullptr;
-  int nsplit = 0, nsplit_tc = 0;
+  int nsplit = 0, nsplit_tc = 0, nsplit_w = 0;
   bool fused = false;            // BF16 form through the fused kernel
   int fused_grid = 0;            // its persistent CTAs (SMs minus those left to the side stream)
   __nv_bfloat16 *UX16 = nullptr, *X16 = nullptr, *ZU16 = nullptr, *Z16 = nullptr;
@@ -257,7 +263,7 @@ struct tlda_ctx {
   cudaEvent_t ev_seg[4] = {nullptr, nullptr, nullptr, nullptr};
   float g_lr = 0.f;
   const float *g_phi = nullptr;
-  int g_loss = -1;
+  int g_loss = -1, g_touch = -1;
   // event profiler: kernels whose bit is set in prof_mask are bracketed by events
   uint32_t prof_mask = 0;
   struct ProfRec { int id; cudaEvent_t a, b; };
@@ -278,6 +284,11 @@ extern const char *const kKernelNames[kNumKernels];
 void launch_set_desc(DevState *st, const BatchDesc &b, cudaStream_t s);
 void launch_begin_pass(DevState *st, const BatchDesc *descs, int n, cudaStream_t s);
 void launch_whiten(const StepArgs &a, cudaStream_t s, float *X_out, bool stats);
+void launch_touch(const StepArgs &a, cudaStream_t s);
+void launch_q_f32(const StepArgs &a, cudaStream_t s);
+void launch_doc(const StepArgs &a, cudaStream_t s);
+void launch_gw_f32(const StepArgs &a, cudaStream_t s);   // with a.nsplit partial sums
+int gw_splits(int Dp, int Kp, int sms);
 void launch_qy_f32(const StepArgs &a, cudaStream_t s);
 void launch_rz(const StepArgs &a, cudaStream_t s);
 void launch_zh_f32(const StepArgs &a, cudaStream_t s);
@@ -329,5 +340,6 @@ void *tc_make_maps(const __nv_bfloat16 *UX16, const __nv_bfloat16 *ZU16, const _
 void tc_free_maps(void *maps);
 void launch_qy_tc(const StepArgs &a, cudaStream_t s);
 void launch_zh_tc(const StepArgs &a, cudaStream_t s);
+void launch_h_clear(const StepArgs &a, cudaStream_t s);
 void launch_g_tc(const StepArgs &a, cudaStream_t s);
 }  // namespace tlda
