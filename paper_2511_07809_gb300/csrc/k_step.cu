@@ -181,15 +181,48 @@ __global__ void __launch_bounds__(256) k_touch(StepArgs a) {
   touch_words(a, a.st->cur, &a.st->n_touched, blockIdx.x, gridDim.x);
 }
 
+// The same for a batch given by value, which becomes the step's batch.
+__global__ void __launch_bounds__(256) k_touch_batch(StepArgs a, BatchDesc b) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.st->cur = b;
+  touch_words(a, b, &a.st->n_touched, blockIdx.x, gridDim.x);
+}
+
 void launch_touch(const StepArgs &a, cudaStream_t s) { k_touch<<<2 * a.sms, 256, 0, s>>>(a); }
+void launch_touch_batch(const StepArgs &a, const BatchDesc &b, cudaStream_t s) {
+  k_touch_batch<<<std::min(2 * a.sms, b.n_docs / 8 + 1), 256, 0, s>>>(a, b);  // 128 nonzeros a document: one turn
+}
+
+// Four U rows q .. q + 3 of a chunk into acc (FP32, in the chunk's order).
+template <int NV>
+__device__ __forceinline__ void add_rows(const NzChunk &c, int q, const float *U32, int Dp, int cols, int lane,
+                                         float4 (&acc)[NV]) {
+  int mm[4];
+  float ff[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    mm[u] = __shfl_sync(0xffffffffu, c.m, (q + u) & 31);
+    ff[u] = (float)__shfl_sync(0xffffffffu, c.f, (q + u) & 31);
+    if (q + u >= c.n) ff[u] = 0.f;
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const int col = v * 128 + lane * 4;
+    if (col < cols) {
+      float4 r[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) r[u] = __ldg(reinterpret_cast<const float4 *>(U32 + (long long)mm[u] * Dp + col));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[v] = fma4(ff[u], r[u], acc[v]);
+    }
+  }
+}
 
 // One warp per document: validates the row, accumulates L_d and
-// x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, and (stats) adds
-// c_m to this block's copy and the block's share of S3.  TC=true also writes X in BF16 row-major (X16),
-// whole rows.
+// x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, adds c_m to this
+// block's copy and the block's share of S3.  TC=true writes X in BF16 row-major
+// (X16), whole rows, else in FP32.
 template <int NV, bool TC>
-__global__ void __launch_bounds__(32 * kDocsPerBlock)
-    k_scan_whiten(StepArgs a, float *X_out, int stats) {
+__global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a) {
   const BatchDesc b = a.st->cur;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d0 = blockIdx.x * kDocsPerBlock;
@@ -204,7 +237,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
   for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
   if (d < b.n_docs) {
     const int lo = b.indptr[d], hi = b.indptr[d + 1];
-    bool bad = stats ? !row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs]) : lo < b.nz_base || hi < lo;
+    bool bad = !row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs]);
     long long lsum = 0;
     int prev = -1;
     if (!bad) {
@@ -213,44 +246,15 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
         if (__any_sync(0xffffffffu, c.bad)) bad = true;
         prev = __shfl_sync(0xffffffffu, c.in ? c.m : -1, c.n - 1);
         lsum += c.f;
-        if (stats && a.same_token && c.f > 0) atomicAdd(cnt + c.m, c.f);
-        for (int q = 0; q < c.n; q += 4) {
-          int mm[4];
-          float ff[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            mm[u] = __shfl_sync(0xffffffffu, c.m, (q + u) & 31);
-            ff[u] = (float)__shfl_sync(0xffffffffu, c.f, (q + u) & 31);
-            if (q + u >= c.n) ff[u] = 0.f;
-          }
-#pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            const int col = v * 128 + lane * 4;
-            if (col < a.Dp) {
-              float4 r[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                r[u] = __ldg(reinterpret_cast<const float4 *>(a.U32 + (long long)mm[u] * a.Dp + col));
-#pragma unroll
-              for (int u = 0; u < 4; ++u) acc[v] = fma4(ff[u], r[u], acc[v]);
-            }
-          }
-        }
+        if (a.same_token && c.f > 0) atomicAdd(cnt + c.m, c.f);
+        for (int q = 0; q < c.n; q += 4) add_rows<NV>(c, q, a.U32, a.Dp, a.Dp, lane, acc);
       }
     }
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     const long long L = lsum;
     if (bad && lane == 0) atomicOr(&a.st->err, kErrCsr);
-    if (stats && lane == 0 && L >= 3) atomicAdd(&s3, (unsigned long long)(L * (L - 1) * (L - 2)));
-    if (X_out) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const int col = v * 128 + lane * 4;
-        const float c[4] = {acc[v].x, acc[v].y, acc[v].z, acc[v].w};
-        for (int q = 0; q < 4; ++q)
-          if (col + q < a.D) X_out[(long long)d * a.D + col + q] = c[q];
-      }
-    } else if (!TC) {
+    if (lane == 0 && L >= 3) atomicAdd(&s3, (unsigned long long)(L * (L - 1) * (L - 2)));
+    if (!TC) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const int col = v * 128 + lane * 4;
@@ -259,7 +263,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
     }
   }
   if constexpr (TC) {
-    if (!X_out && d < round_up(b.n_docs, 64)) {
+    if (d < round_up(b.n_docs, 64)) {
       // row-major BF16 copy: the A operand of Y = X Phi and of G1 = X^T Z (rows
       // past the batch, up to the next multiple of 64, are written as zeros)
 #pragma unroll
@@ -273,21 +277,73 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock)
     }
   }
   __syncthreads();
-  if (stats && threadIdx.x == 0 && s3) atomicAdd(&a.st->S3, s3);
+  if (threadIdx.x == 0 && s3) atomicAdd(&a.st->S3, s3);
 }
 
-void launch_whiten(const StepArgs &a, cudaStream_t s, float *X_out, bool stats) {
-  const bool tc = a.precision == TLDA_BF16 && X_out == nullptr;
+void launch_whiten(const StepArgs &a, cudaStream_t s) {
+  const bool tc = a.precision == TLDA_BF16;
   const int grid = round_up(a.Bmax, 64) / kDocsPerBlock;
   const int nv = (a.Dp + 127) / 128;
-#define TLDA_WHITEN(NVv)                                                                        \
-  if (nv == NVv) {                                                                              \
-    if (tc) k_scan_whiten<NVv, true><<<grid, 32 * kDocsPerBlock, 0, s>>>(a, X_out, stats);     \
-    else k_scan_whiten<NVv, false><<<grid, 32 * kDocsPerBlock, 0, s>>>(a, X_out, stats);       \
-    return;                                                                                     \
+#define TLDA_WHITEN(NVv)                                                              \
+  if (nv == NVv) {                                                                    \
+    if (tc) k_scan_whiten<NVv, true><<<grid, 32 * kDocsPerBlock, 0, s>>>(a);          \
+    else k_scan_whiten<NVv, false><<<grid, 32 * kDocsPerBlock, 0, s>>>(a);            \
+    return;                                                                           \
   }
   TLDA_WHITEN(1) TLDA_WHITEN(2) TLDA_WHITEN(3) TLDA_WHITEN(4)
 #undef TLDA_WHITEN
+}
+
+// X = F U of one batch given by value into the caller's B x D array
+// (tlda_whiten_batch): no step state but the error bits.  One warp per document,
+// bound by the latency of its dependent loads (offsets, nonzeros, rows): small
+// blocks sized to the batch, only the D columns of a row read, and whole 16-byte
+// stores where the output's rows allow them (`wide`).  8192 documents at D = 100:
+// 15.0 -> 9.3 us a call; the kernel shared with the CP step needed its batch
+// written to the step state by a launch of its own and stored 4 bytes a lane.
+template <int NV>
+__global__ void __launch_bounds__(128) k_whiten_out(BatchDesc b, int V, int D, int Dp, const float *__restrict__ U32, int *err,
+                                                    float *__restrict__ X, int wide) {
+  const int d = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (d >= b.n_docs) return;
+  const int lo = b.indptr[d], hi = b.indptr[d + 1], cols = (D + 3) & ~3;
+  bool bad = lo < b.nz_base || hi < lo;
+  float4 acc[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
+  if (!bad) {
+    int prev = -1;
+    for (int base = lo; base < hi; base += 32) {
+      const NzChunk c = load_chunk(b, V, base, hi, lane, prev);
+      bad |= __any_sync(0xffffffffu, c.bad);
+      prev = __shfl_sync(0xffffffffu, c.in ? c.m : -1, c.n - 1);
+#pragma unroll 4
+      for (int q = 0; q < c.n; q += 4) add_rows<NV>(c, q, U32, Dp, cols, lane, acc);
+    }
+  }
+  if (bad && lane == 0) atomicOr(err, kErrCsr);
+  float *x = X + (long long)d * D;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const int col = v * 128 + lane * 4;
+    if (wide) {
+      if (col < D) *reinterpret_cast<float4 *>(x + col) = acc[v];
+    } else {
+      const float c[4] = {acc[v].x, acc[v].y, acc[v].z, acc[v].w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (col + q < D) x[col + q] = c[q];
+    }
+  }
+}
+
+void launch_whiten_out(const StepArgs &a, const BatchDesc &b, cudaStream_t s, float *X) {
+  const int grid = (b.n_docs + 3) / 4, nv = (a.Dp + 127) / 128;
+  const int wide = a.D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  if (nv == 1) k_whiten_out<1><<<grid, 128, 0, s>>>(b, a.V, a.D, a.Dp, a.U32, &a.st->err, X, wide);
+  else if (nv == 2) k_whiten_out<2><<<grid, 128, 0, s>>>(b, a.V, a.D, a.Dp, a.U32, &a.st->err, X, wide);
+  else if (nv == 3) k_whiten_out<3><<<grid, 128, 0, s>>>(b, a.V, a.D, a.Dp, a.U32, &a.st->err, X, wide);
+  else k_whiten_out<4><<<grid, 128, 0, s>>>(b, a.V, a.D, a.Dp, a.U32, &a.st->err, X, wide);
 }
 
 // ------------------------------------------------------------ a7/a8: Phi-only terms

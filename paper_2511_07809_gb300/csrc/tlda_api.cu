@@ -192,7 +192,7 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
     { Prof p(ctx, kG, main); launch_gw_f32(a, main); }
   } else {
     if (a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
-    { Prof p(ctx, kWhiten, main); launch_whiten(a, main, nullptr, true); }
+    { Prof p(ctx, kWhiten, main); launch_whiten(a, main); }
     { Prof p(ctx, kQY, main); if (tc) launch_qy_tc(a, main); else launch_qy_f32(a, main); }
     { Prof p(ctx, kRZ, main); launch_rz(a, main); }
     if (a.same_token) { Prof p(ctx, kZH, main); if (tc) launch_zh_tc(a, main); else launch_zh_f32(a, main); }
@@ -775,9 +775,7 @@ tlda_status tlda_whiten_batch(tlda_ctx *ctx, const tlda_csr *batch, float *X_out
   if (!ctx->whitened) return fail(ctx, TLDA_ERR_STATE, "no whitening: fit or set one first");
   if (batch->n_docs > ctx->Bmax) return fail(ctx, TLDA_ERR_INVALID, "n_docs %d > max_batch %d", batch->n_docs, ctx->Bmax);
   if (batch->n_docs == 0) return TLDA_OK;
-  launch_set_desc(ctx->st, desc_of(batch), ctx->stream);
-  StepArgs a = make_args(ctx);
-  launch_whiten(a, ctx->stream, X_out, false);
+  launch_whiten_out(make_args(ctx), desc_of(batch), ctx->stream, X_out);
   CKL();
   return TLDA_OK;
 }
@@ -798,10 +796,12 @@ static tlda_status step_common(tlda_ctx *ctx, const tlda_csr *batch, float *Phi,
   a.gdata_out = gdata_out;
   a.mode = mode;
   a.want_loss = loss_out ? 1 : 0;
-  launch_set_desc(ctx->st, desc_of(batch), ctx->stream);
+  const bool touch = wants_touch(ctx, a);
+  if (touch) launch_touch_batch(a, desc_of(batch), ctx->stream);
+  else launch_set_desc(ctx->st, desc_of(batch), ctx->stream);
   if (a.PhiImg) launch_phi_img(a, ctx->stream);
   CKL();
-  s = enqueue_step(ctx, a, ctx->stream);
+  s = enqueue_step(ctx, a, ctx->stream, touch);
   if (s) return s;
   if (loss_out || mode == 1) {
     s = read_state(ctx);

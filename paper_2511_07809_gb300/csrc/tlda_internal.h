@@ -283,8 +283,10 @@ extern const char *const kKernelNames[kNumKernels];
 // k_step.cu
 void launch_set_desc(DevState *st, const BatchDesc &b, cudaStream_t s);
 void launch_begin_pass(DevState *st, const BatchDesc *descs, int n, cudaStream_t s);
-void launch_whiten(const StepArgs &a, cudaStream_t s, float *X_out, bool stats);
+void launch_whiten(const StepArgs &a, cudaStream_t s);
+void launch_whiten_out(const StepArgs &a, const BatchDesc &b, cudaStream_t s, float *X);
 void launch_touch(const StepArgs &a, cudaStream_t s);
+void launch_touch_batch(const StepArgs &a, const BatchDesc &b, cudaStream_t s);
 void launch_q_f32(const StepArgs &a, cudaStream_t s);
 void launch_doc(const StepArgs &a, cudaStream_t s);
 void launch_gw_f32(const StepArgs &a, cudaStream_t s);   // with a.nsplit partial sums

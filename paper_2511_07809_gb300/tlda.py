@@ -564,7 +564,7 @@ class TLDALoss(torch.autograd.Function):
         G = torch.empty_like(P)
         loss = model.cp_step(batch, P, 0.0, grad=G, want_loss=True)
         ctx.save_for_backward(G)
-        return torch.tensor(loss, dtype=torch.float64, device=P.device)
+        return torch.full((), loss, dtype=torch.float64, device=P.device)  # a fill: no copy from the host to wait for
 
     @staticmethod
     def backward(ctx, grad_output):
