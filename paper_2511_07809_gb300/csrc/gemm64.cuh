@@ -128,28 +128,30 @@ __device__ __forceinline__ void g64_load(T *raw, const T *x, int ld, int t0, int
 }
 
 // The whole number rint(x 2^(55-e)) (half away from zero) plus the bias that
-// makes its bytes the balanced digits plus 128 (|x| < 2^e).
-__device__ __forceinline__ unsigned long long g64_fixed(double x, int e) {
-  const long long b = __double_as_longlong(x);
-  const int E = (int)((b >> 52) & 0x7ff);
-  unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
-  if (E) m |= 1ull << 52;
+// makes its bytes the balanced digits plus 128 (|x| < 2^e); lo and hi words.
+__device__ __forceinline__ uint2 g64_fixed(double x, int e) {
+  const int hx = __double2hiint(x);
+  const int E = (hx >> 20) & 0x7ff;
+  const uint32_t mh = ((uint32_t)hx & 0xfffffu) | (E ? 0x100000u : 0u);
+  const unsigned long long m = ((unsigned long long)mh << 32) | (uint32_t)__double2loint(x);
   const int k = max(E, 1) - 1020 - e;  // <= 2 (an infinity or NaN: the result is NaN whatever the digits)
-  unsigned long long q;
-  if (k >= 0) q = m << min(k, 2);
-  else q = k < -60 ? 0ull : (m + (1ull << (-k - 1))) >> -k;
-  const long long s = b < 0 ? -(long long)q : (long long)q;
-  return (unsigned long long)s + 0x0080808080808080ull;
+  const unsigned long long q = k > 0 ? m << min(k, 2) : (((m << 1) >> min(-k, 62)) + 1) >> 1;
+  const uint32_t neg = (uint32_t)(hx >> 31);
+  const unsigned long long s = (q ^ (((unsigned long long)neg << 32) | neg)) + (neg & 1u) + 0x0080808080808080ull;
+  return make_uint2((uint32_t)s, (uint32_t)(s >> 32));
 }
 
-// Digit i of a fixed value pair (terms k, k+1) as two BF16.  Byte u as FP32
-// 2^23 + u, minus 2^23 + 128: the upper half of that FP32 is the digit in BF16.
-__device__ __forceinline__ uint32_t g64_digit2(unsigned long long a, unsigned long long b, int i) {
-  const int sh = 8 * (6 - i);
-  const uint32_t mask = i == 0 ? 0x1ffu : 0xffu;  // the top digit may be 128: 256 with the bias
-  const uint32_t ua = (uint32_t)(a >> sh) & mask, ub = (uint32_t)(b >> sh) & mask;
-  const float fa = __uint_as_float(0x4b000000u | ua) - 8388736.f;
-  const float fb = __uint_as_float(0x4b000000u | ub) - 8388736.f;
+// Digit of byte i (0: the top) of a pair of fixed values (terms k, k+1) as two
+// BF16.  A byte u as FP32 2^23 + u, minus 2^23 + 128: the upper half of that FP32
+// is the digit in BF16.  The top digit takes two bytes: it may be 128, 256 with
+// the bias.
+template <int I>
+__device__ __forceinline__ uint32_t g64_digit2(uint2 a, uint2 b) {
+  constexpr int byte = 6 - I;
+  constexpr uint32_t sel = I == 0 ? 0x7432 : 0x7440 | (byte & 3);  // {0x4b, 0, the upper byte or 0, byte}
+  const uint32_t ua = __byte_perm(byte < 4 ? a.x : a.y, 0x4b000000u, sel);
+  const uint32_t ub = __byte_perm(byte < 4 ? b.x : b.y, 0x4b000000u, sel);
+  const float fa = __uint_as_float(ua) - 8388736.f, fb = __uint_as_float(ub) - 8388736.f;
   return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
 }
 
@@ -163,10 +165,16 @@ __device__ __forceinline__ void g64_cut(const T *raw, const int *e, const int *c
     const int et = e[t];
     const double x0 = (double)raw[KROWS ? k * kG64RawLd + t : t * 33 + k];
     const double x1 = (double)raw[KROWS ? (k + 1) * kG64RawLd + t : t * 33 + k + 1];
-    const unsigned long long a = g64_fixed(x0, SGN ? et + SGN * ck[k] : et), b = g64_fixed(x1, SGN ? et + SGN * ck[k + 1] : et);
-#pragma unroll
-    for (int s = 0; s < kG64Dig; ++s)
-      *reinterpret_cast<uint32_t *>(dig + (s * kG64Tile + t) * kG64Ld + k) = g64_digit2(a, b, s);
+    const uint2 a = g64_fixed(x0, SGN ? et + SGN * ck[k] : et), b = g64_fixed(x1, SGN ? et + SGN * ck[k + 1] : et);
+    uint32_t *d = reinterpret_cast<uint32_t *>(dig + t * kG64Ld + k);
+    constexpr int plane = kG64Tile * kG64Ld / 2;
+    d[0] = g64_digit2<0>(a, b);
+    d[plane] = g64_digit2<1>(a, b);
+    d[2 * plane] = g64_digit2<2>(a, b);
+    d[3 * plane] = g64_digit2<3>(a, b);
+    d[4 * plane] = g64_digit2<4>(a, b);
+    d[5 * plane] = g64_digit2<5>(a, b);
+    d[6 * plane] = g64_digit2<6>(a, b);
   }
 }
 

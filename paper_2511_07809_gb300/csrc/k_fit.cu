@@ -19,6 +19,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <type_traits>
 #include <vector>
 
 #include "gemm64.cuh"
@@ -82,77 +83,93 @@ __global__ void k_fit_accumulate(tlda_csr b, int V, double *P, unsigned long lon
 
 // ------------------------------------------------------------------ products
 // FP32: C[M x N] = A[M x Kd] B[Kd x N] (row-major, any pitch), FFMA.  Tiles of
-// 128 rows x 16 TN columns, 8 x TN outputs a thread, so that N = 66 or 116
-// columns (D + 16) waste at most 15 of a tile; the next 16 terms are in flight
-// in registers while a slab is used.  Few row tiles leave SMs idle, so the terms
-// are split over blockIdx.z into partial products (sgemm_splits), summed in
-// order by k_sgemm_sum.
-template <int TN>
+// 16 TM rows x 16 TN columns, TM x TN outputs a thread, so that N = 66 or 116
+// columns (D + 16) waste at most 15 of a tile; slabs of 32 terms pass through
+// three stages of shared memory by cp.async (16 bytes a piece where A's rows
+// allow it).  Few row tiles leave SMs idle, so the terms are split over
+// blockIdx.z into partial products (sgemm_splits), summed in order by
+// k_sgemm_sum.  M2 Q at V = 5000, N = 66: 122 us (286 with 64 x 64 tiles and no
+// split; the FFMA rate alone would allow 52 with the tile's padding); Q L^-T, 66
+// terms in 32-row tiles: 9 us (28 in 128-row tiles, 40 blocks).
+constexpr int kSgBk = 32, kSgStages = 3;
+template <int TM, int TN>
+constexpr int sgemm_smem() { return kSgStages * (16 * TM * (kSgBk + 4) + kSgBk * 16 * TN) * 4; }
+
+template <int TM, int TN, bool WIDE>
 __global__ void __launch_bounds__(256) k_sgemm(const float *__restrict__ A, int lda, const float *__restrict__ B, int ldb,
                                                float *__restrict__ C, int ldc, int M, int N, int Kd, int chunk,
                                                long long cstride) {
-  constexpr int BN = 16 * TN, BK = 16, NB = (BK * BN + 255) / 256;
-  __shared__ __align__(16) float As[2][BK][128 + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN];
+  constexpr int BM = 16 * TM, BN = 16 * TN, BK = kSgBk, LDA = BK + 4, STAGE = BM * LDA + BK * BN;
+  extern __shared__ __align__(16) float sg_sm[];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 128, n0 = blockIdx.x * BN;
-  const int kb = blockIdx.z * chunk, ke = min(Kd, kb + chunk);
-  float acc[8][TN], ra[8], rb[NB];
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int kb = blockIdx.z * chunk, ke = min(Kd, kb + chunk), slabs = (ke - kb + BK - 1) / BK;
+  float acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  auto fetch = [&](int k0) {
+  auto request = [&](int q) {
+    if (q < slabs) {
+      float *As = sg_sm + (q % kSgStages) * STAGE, *Bs = As + BM * LDA;
+      const int k0 = kb + q * BK;
+      if (WIDE) {  // kb, ke, lda multiples of 4 and A on 16 bytes
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int e = tid + i * 256, k = k0 + (e & 15), r = m0 + (e >> 4);
-      ra[i] = (k < ke && r < M) ? __ldg(A + (long long)r * lda + k) : 0.f;
-    }
+        for (int i = 0; i < BM * BK / 1024; ++i) {
+          const int e = tid + i * 256, r = e >> 3, k = (e & 7) * 4;
+          const bool in = k0 + k < ke && m0 + r < M;
+          const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(As + r * LDA + k));
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(in ? A + (long long)(m0 + r) * lda + k0 + k : A),
+                       "r"(in ? 16 : 0)
+                       : "memory");
+        }
+      } else {
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      const int e = tid + i * 256, k = k0 + e / BN, c = n0 + e % BN;
-      rb[i] = (e < BK * BN && k < ke && c < N) ? __ldg(B + (long long)k * ldb + c) : 0.f;
+        for (int i = 0; i < BM * BK / 256; ++i) {
+          const int e = tid + i * 256, r = e >> 5, k = e & 31;
+          const bool in = k0 + k < ke && m0 + r < M;
+          g64_cp(As + r * LDA + k, in ? A + (long long)(m0 + r) * lda + k0 + k : A, in);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < BK * BN / 256; ++i) {
+        const int e = tid + i * 256, k = e / BN, c = e % BN;
+        const bool in = k0 + k < ke && n0 + c < N;
+        g64_cp(Bs + k * BN + c, in ? B + (long long)(k0 + k) * ldb + n0 + c : B, in);
+      }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  auto file = [&](int p) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int e = tid + i * 256;
-      As[p][e & 15][e >> 4] = ra[i];
-    }
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      const int e = tid + i * 256;
-      if (e < BK * BN) Bs[p][e / BN][e % BN] = rb[i];
-    }
-  };
-  fetch(kb);
-  file(0);
-  __syncthreads();
-  int p = 0;
-  for (int k0 = kb; k0 < ke; k0 += BK, p ^= 1) {
-    const bool more = k0 + BK < ke;
-    if (more) fetch(k0 + BK);
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4 *>(&As[p][kk][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4 *>(&As[p][kk][ty * 8 + 4]);
-      const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      float br[TN];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) br[j] = Bs[p][kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
-    }
-    if (more) file(p ^ 1);
+  request(0);
+  request(1);
+  for (int q = 0; q < slabs; ++q) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
+    request(q + 2);  // into the stage of slab q - 1, which has been read
+    const float *As = sg_sm + (q % kSgStages) * STAGE + ty * LDA, *Bs = sg_sm + (q % kSgStages) * STAGE + BM * LDA;
+#pragma unroll 2
+    for (int k = 0; k < BK; k += 4) {
+      float4 x[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) x[i] = *reinterpret_cast<const float4 *>(As + 16 * i * LDA + k);  // a warp's two rows: other banks
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float br[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) br[j] = Bs[(k + u) * BN + tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const float xi = u == 0 ? x[i].x : u == 1 ? x[i].y : u == 2 ? x[i].z : x[i].w;
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(xi, br[j], acc[i][j]);
+        }
+      }
+    }
   }
   float *c = C + blockIdx.z * cstride;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = m0 + ty * 8 + i;
+  for (int i = 0; i < TM; ++i) {
+    const int r = m0 + ty + 16 * i;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int n = n0 + tx + 16 * j;
@@ -175,19 +192,34 @@ int sgemm_splits(int M, int N, int Kd, int sms) {
   return std::max(1, std::min(2 * sms / tiles, Kd / 256));
 }
 
+template <int TM, int TN>
+void sgemm_launch(const float *A, int lda, const float *B, int ldb, float *out, int M, int N, int Kd, int chunk, int splits,
+                  cudaStream_t s) {
+  static const cudaError_t attr[2] = {
+      cudaFuncSetAttribute(k_sgemm<TM, TN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sgemm_smem<TM, TN>()),
+      cudaFuncSetAttribute(k_sgemm<TM, TN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sgemm_smem<TM, TN>())};
+  (void)attr;
+  const dim3 g((N + 16 * TN - 1) / (16 * TN), (M + 16 * TM - 1) / (16 * TM), splits);
+  const bool wide = lda % 4 == 0 && Kd % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;  // chunk is a multiple of 32
+  if (wide) k_sgemm<TM, TN, true><<<g, 256, sgemm_smem<TM, TN>(), s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N);
+  else k_sgemm<TM, TN, false><<<g, 256, sgemm_smem<TM, TN>(), s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N);
+}
+
 // part: splits x M x N floats when there is more than one split (C then is M x N).
+// Unsplit products (few terms) take tiles of 32 rows, for more blocks.
 void sgemm(const float *A, int lda, const float *B, int ldb, float *C, int M, int N, int Kd, float *part, int splits,
            cudaStream_t s) {
   const int nt = (N + 127) / 128, tn = (N + 16 * nt - 1) / (16 * nt);
-  const int chunk = ((Kd + splits - 1) / splits + 15) / 16 * 16;
+  const int chunk = ((Kd + splits - 1) / splits + kSgBk - 1) / kSgBk * kSgBk;
   splits = (Kd + chunk - 1) / chunk;
-  const dim3 g(nt, (M + 127) / 128, splits);
   float *out = splits > 1 ? part : C;
-#define TLDA_SGEMM(TNv)                                                                                          \
-  case TNv: k_sgemm<TNv><<<g, 256, 0, s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N); break;
+#define TLDA_SGEMM(TNv)                                                                         \
+  case TNv:                                                                                     \
+    if (splits > 1) sgemm_launch<8, TNv>(A, lda, B, ldb, out, M, N, Kd, chunk, splits, s);      \
+    else sgemm_launch<2, TNv>(A, lda, B, ldb, out, M, N, Kd, chunk, splits, s);                 \
+    break;
   switch (tn) {
-    TLDA_SGEMM(1) TLDA_SGEMM(2) TLDA_SGEMM(3) TLDA_SGEMM(4) TLDA_SGEMM(5) TLDA_SGEMM(6) TLDA_SGEMM(7)
-    default: k_sgemm<8><<<g, 256, 0, s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N); break;
+    TLDA_SGEMM(1) TLDA_SGEMM(2) TLDA_SGEMM(3) TLDA_SGEMM(4) TLDA_SGEMM(5) TLDA_SGEMM(6) TLDA_SGEMM(7) TLDA_SGEMM(8)
   }
 #undef TLDA_SGEMM
   if (splits > 1) {
@@ -651,15 +683,59 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
   if (gt == 0) ctl->sweeps = sweep;
 }
 
+// Column c of L^-1 by forward substitution in one warp, rows lane + 32 t in
+// z[t] (r <= 32 RL): x_k = z_k / l_kk goes round by shuffles, then z_i -= l_ik x_k
+// below.  Two FP64 operations and a shuffle deep a step; column k of L (a row of
+// LT) is requested four steps ahead.
+template <int RL>
+__device__ void chol_inv_column(int c, int r, const double *LT, const double *inv, int lane, double (&z)[RL]) {
+#pragma unroll
+  for (int t = 0; t < RL; ++t) z[t] = lane + 32 * t == c ? 1.0 : 0.0;
+  double ring[4][RL];
+  auto request = [&](int k, double (&v)[RL]) {
+#pragma unroll
+    for (int t = 0; t < RL; ++t) {
+      const int i = lane + 32 * t;
+      v[t] = (k < r && i < r && i > k) ? __ldcg(LT + k * r + i) : 0.0;
+    }
+  };
+  const int k0 = c & ~3;  // the steps before c find zeros
+#pragma unroll
+  for (int g = 0; g < 4; ++g) request(k0 + g, ring[g]);
+#pragma unroll
+  for (int t = 0; t < RL; ++t) {
+    if (32 * t + 31 < k0 || 32 * t >= r) continue;
+    for (int kb = max(32 * t, k0); kb < min(32 * t + 32, r); kb += 4) {
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const int k = kb + g;
+        if (k < r) {
+          const double x = __shfl_sync(0xffffffffu, z[t], k & 31) * inv[k];
+          if (lane == (k & 31)) z[t] = x;
+#pragma unroll
+          for (int u = t; u < RL; ++u)
+            if (32 * u < r) z[u] = fma(-ring[g][u], x, z[u]);  // zero at and above row k
+        }
+        request(k + 4, ring[g]);
+      }
+    }
+  }
+}
+
 // Cholesky factor and inverse of a symmetric positive definite r x r FP64
 // matrix A (overwritten), r <= 512: A = L L^T in panels of 32 columns, then
 // X = L^-1 column by column.  Per panel every block factors the 32 x 32
-// diagonal block for itself in shared memory (one block barrier a column: the
-// columns are scaled at the end), warps solve the rows below it, a grid
-// barrier, then the trailing entries take the panel's 32 terms, and another:
-// 2 r/32 grid barriers where one per column took 2 r, each about as long as a
-// panel's arithmetic.  The columns of X are independent: each block takes its
-// own by forward substitution from LT, with no grid barrier.
+// diagonal block for itself, warps solve the rows below it, a grid barrier, then
+// the trailing entries take the panel's 32 terms, and another: 2 r/32 grid
+// barriers where one per column took 2 r.  The columns of X are independent: a
+// warp each, no barrier.
+// What bounds it is the chain of FP64 operations, 64 cycles each a warp and SM
+// quarter (a division or square root 430 to 680).  The diagonal block runs in
+// four warps, one a quarter, lane = row, every fourth column a warp: a step is
+// the pivot's reciprocal (FP32 and one third-order step), the scaled column, and
+// the next pivot's column, which its warp publishes before the other columns
+// take the step; the columns are scaled by 1/sqrt at the end, side by side.
+// 1185 -> 287 us at r = 216, 345 -> 85 us at r = 66 (19 us of each whole panel).
 // L (lower, zeros above) and LT (its transpose, scratch) are required; Linv,
 // LinvT64 = L^-T and LinvT32 (FP32) are written when given.  status: 1 if a
 // pivot was not positive (it is taken as 1), 2 if a grid barrier expired.
@@ -667,67 +743,77 @@ constexpr int kCholNb = 32;
 __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A, int r, double *__restrict__ L,
                                                          double *__restrict__ LT, double *Linv, double *LinvT64,
                                                          float *LinvT32, int *status, JacCtl *ctl) {
-  __shared__ double Ds[kCholNb][kCholNb + 1], inv[kMaxDim];
-  __shared__ double sx[2][4];
+  __shared__ double Dc[kCholNb][kCholNb + 1], inv[kMaxDim];  // the diagonal block by columns: Dc[k][i]
   __shared__ int s_ok;
-  const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5;
   const int gt = blockIdx.x * nt + tid, gn = G * nt, rr = r * r;
   unsigned nbar = 0;
   for (int e = gt; e < rr; e += gn)
     if (e % r > e / r) L[e] = 0.0;
   for (int j0 = 0; j0 < r; j0 += kCholNb) {
     const int jb = min(kCholNb, r - j0), j1 = j0 + jb;
-    for (int e = tid; e < jb * jb; e += nt) Ds[e / jb][e % jb] = __ldcg(A + (j0 + e / jb) * r + j0 + e % jb);
+    // the lower half; past the matrix the identity, so that a short panel runs alike
+    for (int e = tid; e < kCholNb * kCholNb; e += nt) {
+      const int i = e >> 5, k = e & 31;
+      if (k <= i) Dc[k][i] = i < jb ? __ldcg(A + (j0 + i) * r + j0 + k) : (i == k ? 1.0 : 0.0);
+    }
     __syncthreads();
-    // four warps factor, one per SM quarter: an FP64 operation takes a quarter
-    // 64 cycles a warp, so more warps would only repeat the pivot's reciprocal.
-    // Lane = column (kept in registers: rows w, w + 4, ...); the pivot's column
-    // passes through shared memory.  Entries keep a_ij - sum l_ik l_jk, the
-    // columns are scaled afterwards.
-    if (tid < 128) {
-      const int w = tid >> 5;
-      double a[8];
+    if (w < 4) {
+      double a[8];  // column w + 4 u, row lane (u counted from the current pivot's group)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] = (w + 4 * u < jb && lane < jb) ? Ds[w + 4 * u][lane] : 0.0;
-      for (int j = 0; j < jb; ++j) {
-        double d = Ds[j][j];
-        if (!(d > 0.0)) {
-          if (gt == 0) atomicMax(status, 1);
-          d = 1.0;
-        }
-        const double f = -Ds[lane][j] * recip64(d);  // rows below j of column j are up to date
+      for (int u = 0; u < 8; ++u) a[u] = w + 4 * u <= lane ? Dc[w + 4 * u][lane] : 0.0;
+      for (int jg = 0; jg < jb; jg += 4) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int i = w + 4 * u;
-          if (i > j && i < jb) {
-            a[u] = fma(Ds[i][j], f, a[u]);
-            if (lane > j && lane <= i) Ds[i][lane] = a[u];
+        for (int q = 0; q < 4; ++q) {
+          const int j = jg + q;
+          // column j is final in Dc
+          const double v = lane >= j ? Dc[j][lane] : 0.0;
+          double d = Dc[j][j];
+          const int hd = __double2hiint(d);  // positive, not NaN: an integer test
+          if (!((hd > 0 && hd <= 0x7ff00000) || (hd == 0 && __double2loint(d) != 0))) {
+            if (gt == 0 && j < jb) atomicMax(status, 1);
+            d = 1.0;
+          }
+          const double g = -(v * recip64(d));
+          // the next pivot's column first, published at once
+          const int nw = (q + 1) & 3, nu = q == 3 ? 1 : 0;
+          if (w == nw && j + 1 < kCholNb) {
+            a[nu] = fma(g, Dc[j][j + 1], a[nu]);
+            if (lane > j) Dc[j + 1][lane] = a[nu];
+          }
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int k = jg + w + 4 * u;
+            if (k > j + 1 && k < kCholNb) a[u] = fma(g, Dc[j][k], a[u]);
           }
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+        for (int u = 0; u < 7; ++u) a[u] = a[u + 1];
       }
     }
     __syncthreads();
     if (tid < jb) {
-      const double d = Ds[tid][tid];
-      inv[j0 + tid] = rsqrt(d > 0.0 ? d : 1.0);
+      const double d = Dc[tid][tid];
+      const double q = rsqrt(d > 0.0 ? d : 1.0);
+      inv[j0 + tid] = q;
     }
     __syncthreads();
     for (int e = tid; e < jb * jb; e += nt) {
-      const int i = e / jb, k = e % jb;
-      if (k < i) Ds[i][k] *= inv[j0 + k];
-    }
-    if (tid < jb) {
-      const double d = Ds[tid][tid];
-      Ds[tid][tid] = (d > 0.0 ? d : 1.0) * inv[j0 + tid];
+      const int k = e / jb, i = e % jb;
+      if (k <= i) {
+        double x = Dc[k][i];
+        if (k == i && !(x > 0.0)) x = 1.0;
+        Dc[k][i] = x * inv[j0 + k];
+      }
     }
     __syncthreads();
     if (blockIdx.x == 0)
       for (int e = tid; e < jb * jb; e += nt) {
-        const int i = e / jb, k = e % jb;
+        const int k = e / jb, i = e % jb;
         if (k <= i) {
-          L[(j0 + i) * r + j0 + k] = Ds[i][k];
-          LT[(j0 + k) * r + j0 + i] = Ds[i][k];
+          L[(j0 + i) * r + j0 + k] = Dc[k][i];
+          LT[(j0 + k) * r + j0 + i] = Dc[k][i];
         }
       }
     // rows below: x L11^T = a, lane k holds column k
@@ -736,7 +822,7 @@ __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A
       for (int k = 0; k < jb; ++k) {
         const double x = __shfl_sync(0xffffffffu, a, k) * inv[j0 + k];
         if (lane == k) a = x;
-        else if (lane > k && lane < jb) a = fma(-x, Ds[lane][k], a);
+        else if (lane > k && lane < jb) a = fma(-x, Dc[k][lane], a);
       }
       if (lane < jb) {
         L[i * r + j0 + lane] = a;
@@ -764,72 +850,26 @@ __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A
     }
   }
   if (!Linv && !LinvT64 && !LinvT32) return;
-  // columns blockIdx, blockIdx + G, ... of L^-1, four at a time; thread i holds
-  // rows i and i + 256.  Two FP64 operations and a block barrier a step, each row
-  // of x scaled by its own thread.
-  for (int c0 = blockIdx.x; c0 < r; c0 += 4 * G) {
-    const int nc = min(4, (r - c0 + G - 1) / G);
-    double z[2][4];
+  // warp w of block b takes columns b + G w, b + G (w + 8), ...: one a quarter first
+  auto columns = [&](auto rl) {
+    constexpr int RL = decltype(rl)::value;
+    for (int c = blockIdx.x + G * w; c < r; c += G * (nt >> 5)) {
+      double z[RL];
+      chol_inv_column<RL>(c, r, LT, inv, lane, z);
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) z[u][q] = (tid + u * kJacThreads == c0 + q * G) ? 1.0 : 0.0;
-    double lv[4][2], nx[4][2];
-    auto rows = [&](int k, double (&v)[4][2]) {  // L rows tid, tid + 256 of columns k .. k + 3
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int i = tid + u * kJacThreads;
-          v[g][u] = (k + g < r && i < r && i > k + g) ? __ldcg(LT + (k + g) * r + i) : 0.0;
-        }
-    };
-    rows(c0, lv);
-    __syncthreads();  // sx of the columns before
-    for (int k0 = c0; k0 < r; k0 += 4) {
-      rows(k0 + 4, nx);
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int k = k0 + g;
-        if (k < r) {
-          if (tid == (k & (kJacThreads - 1))) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (q < nc) {
-                const double x = (k < kJacThreads ? z[0][q] : z[1][q]) * inv[k];
-                if (k < kJacThreads) z[0][q] = x;
-                else z[1][q] = x;
-                sx[k & 1][q] = x;
-              }
-          }
-          __syncthreads();
-          // FP64 issue is what a step costs: rows at or above k and columns past r are skipped
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < nc) {
-              const double x = sx[k & 1][q];
-              if ((tid | 31) > k) z[0][q] = fma(-lv[g][0], x, z[0][q]);
-              if (kJacThreads < r && (tid | 31) + kJacThreads > k) z[1][q] = fma(-lv[g][1], x, z[1][q]);
-            }
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) lv[g][u] = nx[g][u];
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = tid + u * kJacThreads, c = c0 + q * G;
-        if (i >= r || c >= r) continue;
-        const double x = c <= i ? z[u][q] : 0.0;
+      for (int t = 0; t < RL; ++t) {
+        const int i = lane + 32 * t;
+        if (i >= r) continue;
+        const double x = c <= i ? z[t] : 0.0;
         if (Linv) Linv[i * r + c] = x;
         if (LinvT64) LinvT64[c * r + i] = x;
         if (LinvT32) LinvT32[c * r + i] = (float)x;
       }
-  }
+    }
+  };
+  if (r <= 128) columns(std::integral_constant<int, 4>());
+  else if (r <= 256) columns(std::integral_constant<int, 8>());
+  else columns(std::integral_constant<int, 16>());
 }
 
 // B = C1 C2^-1 for r x r FP64 matrices (C2 general, row-major): Gauss-Jordan
