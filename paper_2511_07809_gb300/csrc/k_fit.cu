@@ -395,13 +395,11 @@ __global__ void k_d2f(const double *x, float *y, long long n) {
 }
 
 // ------------------------------------------------------------------ small dense FP64
-// Transpose r x r (FP64 -> FP32 for the Y Linv^T product).
-__global__ void k_transpose_rr(const double *A, int r, float *AT32, double *AT64) {
+__global__ void k_transpose_rr(const double *A, int r, double *AT) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= r * r) return;
   const int i = e / r, j = e % r;
-  if (AT32) AT32[j * r + i] = (float)A[e];
-  if (AT64) AT64[j * r + i] = A[e];
+  AT[j * r + i] = A[e];
 }
 
 // Control block of the grid-wide Jacobi: the grid barrier's arrival counter,
@@ -503,11 +501,13 @@ __device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q
 // FP64 pipe, which takes 2 operations a clock per SM.  So the 2 x 2 blocks are
 // dealt as tiles of bt x bt pairs over T x T thread blocks: a block needs the
 // rotations of its 2 bt pairs only, not of all r/2; its entries are requested
-// before the rotations are computed; and the angle is found in FP32, with c =
-// (1 - h^2)/(1 + h^2) and s = 2 h/(1 + h^2) in FP64 for the h that FP32 gives
-// (an FP64 division or square root takes 430 to 680 cycles here): the rotation
-// is orthogonal to FP64 rounding, and the annihilated entry keeps its computed
-// rest, 1e-7 of what it was.
+// before the rotations are computed; and the angle is found in FP32 and made good
+// to 1e-14 by one Newton step whose rest is FP64, with c = (1 - h^2)/(1 + h^2) and
+// s = 2 h/(1 + h^2) for the tangent h of its half (an FP64 division or square root
+// takes 430 to 680 cycles here): the rotation is orthogonal to FP64 rounding.
+// Without the step an r = 216 solve takes 0.45 ms less of 6.9, but then the entries
+// that the last sweep leaves under the stopping rule, and with them the
+// eigenvectors at 1e-8, are others than with exact angles.
 __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, int r, double *__restrict__ Et,
                                                        double *__restrict__ eval, int max_sweeps,
                                                        JacCtl *ctl) {
@@ -633,7 +633,13 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
           const float tau = __fdividef(0.5f * fd, fp), f = fabsf(tau);
           const float t = __frcp_rn(f + __fsqrt_rn(fmaf(f, f, 1.f)));
           const float h1 = __fdividef(t, 1.f + __fsqrt_rn(fmaf(t, t, 1.f)));  // tan of half the angle, at most 0.42
-          const double hh = widen_f32(tau < 0.f ? -h1 : h1), w = fma(hh, hh, 1.0);
+          double hh = widen_f32(tau < 0.f ? -h1 : h1);
+          // Newton from the rest that this angle would leave (times (1 + h^2)^2)
+          const double u = fma(-hh, hh, 1.0), v = 2.0 * hh, uv = u * v, uu = fma(u, u, -v * v);
+          const float rest = seed_f32(fma(uu, apq, -uv * (aqq - app)));
+          const float slope = fmaf(seed_f32(uu), fd, 4.f * seed_f32(uv) * fp);
+          hh += widen_f32(__fdividef(0.5f * fmaf(h1, h1, 1.f) * rest, slope));
+          const double w = fma(hh, hh, 1.0);
           const double q = recip64(w);
           c = fma(2.0, q, -1.0);
           sv = 2.0 * hh * q;
@@ -1703,7 +1709,7 @@ tlda_status online_rewhiten(tlda_ctx *ctx) {
   if (tlda_status st = cholqr_pass(w.Q1, w.Q2, w.L2)) return st;
   gemm_tn64(w.Q2, r, ctx->on_Om, r, w.C2, r, r, r, V, ex, V, sms, s);  // Q^T Omega
   // Q^T Y = R = (L1 L2)^T = L2^T L1^T
-  k_transpose_rr<<<(r * r + 255) / 256, 256, 0, s>>>(w.L1, r, nullptr, w.L1T);
+  k_transpose_rr<<<(r * r + 255) / 256, 256, 0, s>>>(w.L1, r, w.L1T);
   gemm_tn64(w.L2, r, w.L1T, r, w.C1, r, r, r, r, ex, V, sms, s);
   // B = (Q^T Y)(Q^T Omega)^-1, symmetrised by the eigensolver
   if (tlda_status st = run_solve_right(ctx, w.C1, w.C2, r, w.Ms, w.Rs, w.Bm, status + 1, s)) return st;
