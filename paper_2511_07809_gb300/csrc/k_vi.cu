@@ -46,35 +46,39 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Four words of a round: their sums s_i = sum_k mu_ik e_k over the warp (each
-// lane brings the products of its own topics in pv), then acc += f_i pv_i / s_i.
-// The four sums are reduced together: after two exchanges a lane holds one
-// word's partial sum, so that 6 shuffles, 3 of them on one value, and 4
-// broadcasts of f_i / s_i serve four words, where one sum at a time took 20.
-// The pairs added are those of a butterfly over each word alone, bit for bit.
-template <int KPL>
-__device__ __forceinline__ void vi_four(const float (&pv)[4][KPL], float f, float (&acc)[KPL], int lane) {
-  float s[4];
+// W words of a round (1, 2 or 4): their sums s_i = sum_k mu_ik e_k over the warp
+// (each lane brings the products of its own topics in pv), then acc += f_i pv_i / s_i.
+// The sums are reduced together: an exchange halves the words that a lane sums,
+// so that 6 shuffles, 3 of them on one value, and 4 broadcasts of f_i / s_i serve
+// four words, where one sum at a time took 20.  The pairs added are those of a
+// butterfly over each word alone, bit for bit.
+template <int KPL, int W>
+__device__ __forceinline__ void vi_words(const float (&pv)[W][KPL], float f, float (&acc)[KPL], int lane) {
+  constexpr int P = 32 / W;  // lanes P i .. P i + P - 1 end with word i's sum; f is that word's count there
+  float s[W];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < W; ++i) {
     s[i] = pv[i][0];
 #pragma unroll
     for (int t = 1; t < KPL; ++t) s[i] += pv[i][t];
   }
-  const bool up = lane & 16, odd = lane & 8;
-  const float a0 = (up ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, up ? s[0] : s[2], 16);
-  const float a1 = (up ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, up ? s[1] : s[3], 16);
-  float v = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  // lanes 8 i .. 8 i + 7 hold word i's sum; f is that word's count there
+  for (int n = W / 2, o = 16; n > 0; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n; ++i)
+      s[i] = (up ? s[i + n] : s[i]) + __shfl_xor_sync(0xffffffffu, up ? s[i] : s[i + n], o);
+  }
+  float v = s[0];
+#pragma unroll
+  for (int o = P / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   const float w = v > 0.f ? __fdividef(f, v) : -1.f;  // -1: no topic holds the word, it adds nothing
   const bool tiny = w > 3.0e38f;  // a sum below f / FLT_MAX (subnormal rows): product and sum times 2^100
   if (__any_sync(0xffffffffu, tiny)) {
     const float w2 = tiny ? __fdividef(f, v * 0x1p100f) : w, sc = tiny ? 0x1p100f : 1.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float wi = __shfl_sync(0xffffffffu, w2, 8 * i), si = __shfl_sync(0xffffffffu, sc, 8 * i);
+    for (int i = 0; i < W; ++i) {
+      const float wi = __shfl_sync(0xffffffffu, w2, P * i), si = __shfl_sync(0xffffffffu, sc, P * i);
       if (wi >= 0.f) {
 #pragma unroll
         for (int t = 0; t < KPL; ++t) acc[t] = fmaf(pv[i][t] * si, wi, acc[t]);
@@ -83,8 +87,8 @@ __device__ __forceinline__ void vi_four(const float (&pv)[4][KPL], float f, floa
     return;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float wi = __shfl_sync(0xffffffffu, w, 8 * i);
+  for (int i = 0; i < W; ++i) {
+    const float wi = W > 1 ? __shfl_sync(0xffffffffu, w, P * i) : w;
     if (wi >= 0.f) {
 #pragma unroll
       for (int t = 0; t < KPL; ++t) acc[t] = fmaf(pv[i][t], wi, acc[t]);
@@ -92,34 +96,49 @@ __device__ __forceinline__ void vi_four(const float (&pv)[4][KPL], float f, floa
   }
 }
 
-// Groups of four words whose topic rows stay in registers over the rounds: about
-// 64 registers of rows a thread (16 to 32 words up to K = 128, most documents of
-// the workloads).
-__host__ __device__ constexpr int vi_cached(int kpl) { return kpl == 1 ? 8 : kpl == 2 ? 6 : kpl == 3 ? 5 : kpl == 4 ? 4 : kpl <= 6 ? 2 : 1; }
+// How KPL topics a lane are worked: W words reduced together, the rows of the
+// first NC W words kept in registers over the rounds, and as many blocks an SM as
+// the registers are bounded for.  Measured (10 rounds, V = 3000; one word at a
+// time before, in us): warps in flight hide the row gathers better than kept rows,
+// except where a row is one register.
+//   K = 20, 49 words, 30000 documents     778 -> 508   (nothing kept, 24 blocks: 547)
+//   K = 50, 49 words, 30000 documents     963 -> 643   (2 kept groups, 16 blocks: 666)
+//   K = 100, 12 words, 50000 documents    671 -> 558   (4 kept groups, 8 blocks: 604)
+//   K = 123, 49 words, 18557 documents    888 -> 658   (4 kept groups, 8 blocks: 923)
+//   K = 150, 45 words, 18000 documents   1059 -> 747   (2 kept groups, 8 blocks: 1357)
+//   K = 180, 45 words, 18000 documents   1222 -> 849   (24 warps an SM in place of 36: 1175)
+//   K = 200, 12 words, 20000 documents    528 -> 452   (four words: 456 at best)
+//   K = 300, 50 words, 10000 documents   1840 -> 1268  (two words: 1559, four: 1933)
+struct ViShape {
+  int W, NC, blocks;
+};
+__host__ __device__ constexpr ViShape vi_shape(int kpl) {
+  return kpl <= 1   ? ViShape{4, 4, 16}
+         : kpl <= 2 ? ViShape{4, 0, 20}
+         : kpl <= 6 ? ViShape{4, 0, 18}
+         : kpl <= 7 ? ViShape{2, 0, 16}
+         : kpl <= 8 ? ViShape{1, 0, 16}
+         : kpl <= 12 ? ViShape{1, 0, 14}
+                     : ViShape{1, 0, 10};
+}
 
 // KPL topics per lane: topic k = lane + 32 t.  exp(digamma) is taken relative
 // to its largest value over the topics, which the per-word normalisation
 // cancels, so small gamma never underflows every topic at once.  Bound by
-// instruction issue (741 warp instructions a document and round at K = 100 and
-// 12 words, IPC 2.45 of 4): 300,000 documents and 20 rounds take 5.69 ms, where
-// one word's sum at a time and every row loaded again each round took 6.95; the
-// results are the same bit for bit.  More rows in registers or more warps with
-// fewer were not faster (5.78 ms with 12 words kept, 6.09 with 4 at 32 warps).
+// instruction issue and by the L1/L2 latency of the row gathers: K = 100,
+// V = 20000, 100,000 documents of 12 words, 20 rounds take 1.97 ms, where one
+// word's sum at a time took 2.40; the results are the same bit for bit.
 template <int KPL>
-__global__ void __launch_bounds__(kViThreads, KPL <= 8 ? 8 : 5) k_doc_topics(tlda_csr docs, const float *__restrict__ mu,
+__global__ void __launch_bounds__(kViThreads, vi_shape(KPL).blocks) k_doc_topics(tlda_csr docs, const float *__restrict__ mu,
                                                           const float *__restrict__ alpha, int K, int n_iter,
                                                           float *__restrict__ theta, float *__restrict__ gamma_out,
                                                           int32_t *err) {
-  constexpr int NC = vi_cached(KPL);
+  constexpr int NC = vi_shape(KPL).NC, W = vi_shape(KPL).W, P = 32 / W;
   const int doc = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (doc >= docs.n_docs) return;
   const long long p0 = docs.indptr[doc], p1 = docs.indptr[doc + 1];
-  float a[KPL], g[KPL], e[KPL], acc[KPL];
-#pragma unroll
-  for (int t = 0; t < KPL; ++t) {
-    const int k = lane + 32 * t;
-    a[t] = k < K ? alpha[k] : 0.f;
-  }
+  float g[KPL], e[KPL], acc[KPL];
+  auto prior = [&](int t) { return lane + 32 * t < K ? __ldg(alpha + lane + 32 * t) : 0.f; };
   // validation and the document length
   bool bad = p0 < 0 || p1 < p0;
   long long L = 0;
@@ -145,17 +164,18 @@ __global__ void __launch_bounds__(kViThreads, KPL <= 8 ? 8 : 5) k_doc_topics(tld
   for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   const float l_over_k = (float)L / (float)K;
 #pragma unroll
-  for (int t = 0; t < KPL; ++t) g[t] = a[t] + l_over_k;
+  for (int t = 0; t < KPL; ++t) g[t] = prior(t) + l_over_k;
 
-  // four words at q0: their rows, and their counts as vi_four wants them (words
-  // past the end: row zero, count 0)
-  auto rows_at = [&](long long q0, float (&row)[4][KPL]) {
-    const long long mine = q0 + (lane >> 3);
-    const int m = mine < p1 ? docs.indices[mine] : -1;
-    const float f = mine < p1 ? (float)docs.counts[mine] : 0.f;
+  // a word and its count for each lane from q0 on (past the end: row zero, count 0)
+  auto word_at = [&](long long q0, int &m, float &f) {
+    m = q0 + lane < p1 ? docs.indices[q0 + lane] : -1;
+    f = q0 + lane < p1 ? (float)docs.counts[q0 + lane] : 0.f;
+  };
+  // the rows of the words that lanes c .. c + W - 1 hold
+  auto rows_of = [&](int m, int c, float (&row)[W][KPL]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int mi = __shfl_sync(0xffffffffu, m, 8 * i);
+    for (int i = 0; i < W; ++i) {
+      const int mi = __shfl_sync(0xffffffffu, m, c + i);
       const float *r = mu + (long long)max(mi, 0) * K;
 #pragma unroll
       for (int t = 0; t < KPL; ++t) {
@@ -163,14 +183,16 @@ __global__ void __launch_bounds__(kViThreads, KPL <= 8 ? 8 : 5) k_doc_topics(tld
         row[i][t] = mi >= 0 && k < K ? __ldg(r + k) : 0.f;
       }
     }
-    return f;
   };
-  float keep[NC][4][KPL], kf[NC];
+  float keep[NC ? NC : 1][W][KPL], kf[NC ? NC : 1], tf = 0.f;
+  int tm = -1;
+  word_at(p0, tm, tf);
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    kf[c] = 0.f;
-    if (p0 + 4 * c < p1) kf[c] = rows_at(p0 + 4 * c, keep[c]);
+    kf[c] = __shfl_sync(0xffffffffu, tf, W * c + lane / P);  // as vi_words wants them
+    if (p0 + W * c < p1) rows_of(tm, W * c, keep[c]);
   }
+  if (p0 + W * NC < p1) word_at(p0 + W * NC, tm, tf);  // the words after these, requested once
 
   for (int it = 0; it < n_iter; ++it) {
     float mx = -INFINITY;
@@ -185,27 +207,34 @@ __global__ void __launch_bounds__(kViThreads, KPL <= 8 ? 8 : 5) k_doc_topics(tld
     for (int t = 0; t < KPL; ++t) {
       const int k = lane + 32 * t;
       e[t] = k < K ? __expf(e[t] - mx) : 0.f;
-      acc[t] = a[t];
+      acc[t] = prior(t);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (p0 + 4 * c < p1) {
-        float pv[4][KPL];
+      if (p0 + W * c < p1) {
+        float pv[W][KPL];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < W; ++i)
 #pragma unroll
           for (int t = 0; t < KPL; ++t) pv[i][t] = keep[c][i][t] * e[t];
-        vi_four<KPL>(pv, kf[c], acc, lane);
+        vi_words<KPL, W>(pv, kf[c], acc, lane);
       }
     }
-    for (long long q0 = p0 + 4 * NC; q0 < p1; q0 += 4) {
-      float pv[4][KPL];
-      const float f = rows_at(q0, pv);
+    int m = tm;
+    float f = tf;
+    for (long long q0 = p0 + W * NC; q0 < p1; q0 += 32) {
+      if (q0 > p0 + W * NC) word_at(q0, m, f);
+      const int n = (int)min((long long)32, p1 - q0);
+      for (int c = 0; c < n; c += W) {
+        float pv[W][KPL];
+        rows_of(m, c, pv);
+        const float fc = __shfl_sync(0xffffffffu, f, c + lane / P);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < W; ++i)
 #pragma unroll
-        for (int t = 0; t < KPL; ++t) pv[i][t] *= e[t];
-      vi_four<KPL>(pv, f, acc, lane);
+          for (int t = 0; t < KPL; ++t) pv[i][t] *= e[t];
+        vi_words<KPL, W>(pv, fc, acc, lane);
+      }
     }
 #pragma unroll
     for (int t = 0; t < KPL; ++t) g[t] = acc[t];
@@ -249,7 +278,9 @@ extern "C" tlda_status tlda_doc_topics(const tlda_csr *docs, const float *mu, co
   else if (kpl <= 2) launch<2>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else if (kpl <= 3) launch<3>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else if (kpl <= 4) launch<4>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
+  else if (kpl <= 5) launch<5>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else if (kpl <= 6) launch<6>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
+  else if (kpl <= 7) launch<7>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else if (kpl <= 8) launch<8>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else if (kpl <= 12) launch<12>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
   else launch<16>(*docs, mu, alpha, K, n_iter, theta_out, gamma_out, err_out, s);
