@@ -918,12 +918,15 @@ void launch_q_f32(const StepArgs &a, cudaStream_t s) {
 // into this block's copy.  The rows come by cp.async into the warp's shared
 // memory, R of them at once: all of a short document's rows are in flight
 // together and are read twice there; a longer one gathers its rows again.
-template <int NK>
+// LW lanes hold a row (8 or 16 up to 32 or 64 topics, else the warp): a narrow
+// model's warp takes 32 / LW rows at a time and adds the parts at the end.
+template <int NK, int LW>
 __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R) {
+  constexpr int SUB = 32 / LW, UN = SUB < 4 ? 4 / SUB : 1;  // rows at a time, turns unrolled
   extern __shared__ __align__(16) float doc_rows[];
   const BatchDesc b = a.st->cur;
   if (b.n_docs <= 0) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LW, sl = lane % LW;
   const int K4 = (a.K + 3) & ~3;  // the padding columns are zero and stay so
   float *rows = doc_rows + (long long)warp * R * K4;
   float *B = a.H32 + (long long)(blockIdx.x % a.nrep) * a.V * a.Kp;
@@ -944,15 +947,15 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
     for (int v = 0; v < NK; ++v) y[v] = r[v] = f4(0.f);
     // rows [s0, s0 + n) of a chunk of nonzeros into shared memory
     auto stage = [&](const NzChunk &c, int s0, int n) {
-      for (int j0 = 0; j0 < n; j0 += 4)
+      for (int j0 = 0; j0 < n; j0 += UN * SUB)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = min(j0 + u, n - 1);
-          const float *src = a.Q32 + (long long)__shfl_sync(0xffffffffu, c.m, s0 + j) * a.Kp + lane * 4;
-          const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(rows + j * K4 + lane * 4));
+        for (int u = 0; u < UN; ++u) {
+          const int jj = j0 + u * SUB + sub, j = min(jj, n - 1);
+          const float *src = a.Q32 + (long long)__shfl_sync(0xffffffffu, c.m, s0 + j) * a.Kp + sl * 4;
+          const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(rows + j * K4 + sl * 4));
 #pragma unroll
           for (int v = 0; v < NK; ++v)
-            if (j0 + u < n && v * 128 + lane * 4 < K4)
+            if (jj < n && v * 128 + sl * 4 < K4)
               asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + v * 512), "l"(src + v * 128) : "memory");
         }
       asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
@@ -970,14 +973,14 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
         const int n = min(R, c.n - s0);
         __syncwarp();  // the rows before have been read
         stage(c, s0, n);
-        for (int j0 = 0; j0 < n; j0 += 4)
+        for (int j0 = 0; j0 < n; j0 += UN * SUB)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {  // past the end: the last row with count 0
-            const int j = min(j0 + u, n - 1);
-            const float f = j0 + u < n ? (float)__shfl_sync(0xffffffffu, c.f, s0 + j) : 0.f;
+          for (int u = 0; u < UN; ++u) {  // past the end: the last row with count 0
+            const int jj = j0 + u * SUB + sub, j = min(jj, n - 1);
+            const float fj = (float)__shfl_sync(0xffffffffu, c.f, s0 + j), f = jj < n ? fj : 0.f;
 #pragma unroll
             for (int v = 0; v < NK; ++v) {
-              const int col = v * 128 + lane * 4;
+              const int col = v * 128 + sl * 4;
               if (col < K4) {
                 const float4 q = *reinterpret_cast<const float4 *>(rows + j * K4 + col);
                 y[v] = fma4(f, q, y[v]);
@@ -996,6 +999,14 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
       if (bad) atomicOr(&a.st->err, kErrCsr);
       if (L >= 3) atomicAdd(&s3, (unsigned long long)(L * (L - 1) * (L - 2)));
     }
+#pragma unroll
+    for (int o = LW; o < 32; o <<= 1) {  // the parts of a narrow model's rows
+      const float4 py = y[0], pr = r[0];
+      y[0] = make_float4(py.x + __shfl_xor_sync(0xffffffffu, py.x, o), py.y + __shfl_xor_sync(0xffffffffu, py.y, o),
+                         py.z + __shfl_xor_sync(0xffffffffu, py.z, o), py.w + __shfl_xor_sync(0xffffffffu, py.w, o));
+      r[0] = make_float4(pr.x + __shfl_xor_sync(0xffffffffu, pr.x, o), pr.y + __shfl_xor_sync(0xffffffffu, pr.y, o),
+                         pr.z + __shfl_xor_sync(0xffffffffu, pr.z, o), pr.w + __shfl_xor_sync(0xffffffffu, pr.w, o));
+    }
     const float on = a.same_token ? 1.f : 0.f;
     float4 z[NK];
 #pragma unroll
@@ -1011,16 +1022,16 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
           __syncwarp();
           stage(c, s0, n);
         }
-        for (int j0 = 0; j0 < n; j0 += 4)
+        for (int j0 = 0; j0 < n; j0 += UN * SUB)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int j = min(j0 + u, n - 1);
+          for (int u = 0; u < UN; ++u) {
+            const int jj = j0 + u * SUB + sub, j = min(jj, n - 1);
             const int m = __shfl_sync(0xffffffffu, c.m, s0 + j);
-            const float f = j0 + u < n ? (float)__shfl_sync(0xffffffffu, c.f, s0 + j) : 0.f;
-            if (f == 0.f) continue;
+            const float f = (float)__shfl_sync(0xffffffffu, c.f, s0 + j);
+            if (jj >= n || f == 0.f) continue;
 #pragma unroll
             for (int v = 0; v < NK; ++v) {
-              const int col = v * 128 + lane * 4;
+              const int col = v * 128 + sl * 4;
               if (col < K4) {
                 const float4 q = *reinterpret_cast<const float4 *>(rows + j * K4 + col);
                 atomicAdd(reinterpret_cast<float4 *>(B + (long long)m * a.Kp + col),
@@ -1045,15 +1056,19 @@ void launch_doc(const StepArgs &a, cudaStream_t s) {
   const int R = std::max(3, std::min(32, kDocBytes / (K4 * 4)));
   const int smem = 8 * R * K4 * (int)sizeof(float);
   const int grid = std::max(1, std::min((a.Bmax + 7) / 8, 4 * a.sms));
-#define TLDA_DOC(NKv)                                                                                  \
-  if (nk == NKv) {                                                                                     \
-    static const cudaError_t attr =                                                                    \
-        cudaFuncSetAttribute(k_doc<NKv>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kDocBytes);       \
-    (void)attr;                                                                                        \
-    k_doc<NKv><<<grid, 256, smem, s>>>(a, R);                                                          \
-    return;                                                                                            \
+#define TLDA_DOC(NKv, LWv)                                                                                     \
+  {                                                                                                            \
+    static const cudaError_t attr =                                                                            \
+        cudaFuncSetAttribute(k_doc<NKv, LWv>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kDocBytes);     \
+    (void)attr;                                                                                                \
+    k_doc<NKv, LWv><<<grid, 256, smem, s>>>(a, R);                                                             \
   }
-  TLDA_DOC(1) TLDA_DOC(2) TLDA_DOC(3) TLDA_DOC(4)
+  if (K4 <= 32) TLDA_DOC(1, 8)
+  else if (K4 <= 64) TLDA_DOC(1, 16)
+  else if (nk == 1) TLDA_DOC(1, 32)
+  else if (nk == 2) TLDA_DOC(2, 32)
+  else if (nk == 3) TLDA_DOC(3, 32)
+  else TLDA_DOC(4, 32)
 #undef TLDA_DOC
 }
 
@@ -1177,10 +1192,11 @@ __global__ void __launch_bounds__(BI / TM * (BN / 4)) k_gw_f32(StepArgs a, int s
   }
 }
 
-// Partial sums: one block an SM over the tiles, at least 8.
+// Partial sums: one block an SM over the tiles, at least 8; two an SM for the 64 x
+// 64 tile, whose block waits more than it computes and whose partial is small.
 int gw_splits(int Dp, int Kp, int sms) {
   const int tiles = ((Dp + 127) / 128) * ((Kp + 127) / 128);
-  return std::max(8, sms / tiles);
+  return Dp <= 64 ? 2 * sms : std::max(8, sms / tiles);
 }
 
 template <int BI, int BN, int TM, bool FOLD>

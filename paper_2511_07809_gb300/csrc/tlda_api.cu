@@ -162,8 +162,9 @@ bool wants_touch(const tlda_ctx *ctx, const StepArgs &a) {
 // terms on the side stream, the data-term chain on the main stream, then the
 // reduction and update once both are done.
 // With `touched`, the batch's touched words are there already (an earlier step's
-// reduction kernel or the caller found them).
-tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false) {
+// reduction kernel or the caller found them); with `host`, the batch was copied
+// from the host just before.
+tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false, bool host = false) {
   const bool tc = a.precision == TLDA_BF16;
   auto fork_phi = [&]() -> tlda_status {
     CK(cudaEventRecord(ctx->ev_fork, main));
@@ -174,9 +175,33 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
     CK(cudaEventRecord(ctx->ev_join, ctx->side));
     return TLDA_OK;
   };
+  const bool tc_chain = tc && !ctx->fused;
   // beside k_doc in the FP32 form by word (its warps wait for memory), not beside
-  // the product before it
-  if (tc || !by_word(a))
+  // the product before it; behind Q in the BF16 chain
+  if (!tc_chain && !by_word(a))
+    if (tlda_status s = fork_phi()) return s;
+  // Q = U Phi needs no document: on the side stream beside the whitening (57 of the
+  // 95 us of [Q; Y] at V = 100,000 and K = 300), but for wide steps on copied input,
+  // which it slows (us a pass, beside the whitening against before Y: 4 batches of
+  // 33781 documents at V = 98359, K = 250 from the host 2873 against 2612, from the
+  // device 1610 against 1621; 103 batches of 1936 to 3873 at V = 1341, K = 26 from
+  // the host 6272 against 6375, from the device 3998 against 4243)
+  const bool q_side = tc_chain && a.same_token && !(host && a.Kp > 64);
+  if (tc_chain && a.same_token) {
+    CK(cudaEventRecord(ctx->ev_fork, main));
+    CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+    if (q_side) {
+      Prof p(ctx, kQY, ctx->side);
+      launch_qy_tc(a, ctx->side, 0);
+      CK(cudaEventRecord(ctx->ev_q, ctx->side));
+    }
+    if (!touched) {  // the touched words are read by zh only
+      Prof p(ctx, kWhiten, ctx->side);
+      launch_touch(a, ctx->side);
+    }
+    CK(cudaEventRecord(ctx->ev_touch, ctx->side));
+  }
+  if (tc_chain)
     if (tlda_status s = fork_phi()) return s;
   if (tc && ctx->fused) {
     // the fused kernel fills its SMs' shared memory: it leaves kPhiSMs SMs
@@ -191,11 +216,24 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
     { Prof p(ctx, kRZ, main); launch_doc(a, main); }
     { Prof p(ctx, kG, main); launch_gw_f32(a, main); }
   } else {
-    if (a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
+    if (!tc && a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
     { Prof p(ctx, kWhiten, main); launch_whiten(a, main); }
-    { Prof p(ctx, kQY, main); if (tc) launch_qy_tc(a, main); else launch_qy_f32(a, main); }
+    {
+      Prof p(ctx, kQY, main);
+      if (tc && a.same_token && !q_side) launch_qy_tc(a, main, 0);
+      if (tc) launch_qy_tc(a, main, 1);
+      else launch_qy_f32(a, main);
+    }
+    if (q_side) CK(cudaStreamWaitEvent(main, ctx->ev_q, 0));
     { Prof p(ctx, kRZ, main); launch_rz(a, main); }
+    if (tc && a.same_token) CK(cudaStreamWaitEvent(main, ctx->ev_touch, 0));
     if (a.same_token) { Prof p(ctx, kZH, main); if (tc) launch_zh_tc(a, main); else launch_zh_f32(a, main); }
+    if (tc && a.same_token) {  // H and c are cleared beside the last product
+      CK(cudaEventRecord(ctx->ev_zc, main));
+      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_zc, 0));
+      { Prof p(ctx, kZH, ctx->side); launch_h_clear(a, ctx->side); }
+      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+    }
     { Prof p(ctx, kG, main); if (tc) launch_g_tc(a, main); else launch_g_f32(a, main); }
   }
   CKL();
@@ -635,6 +673,9 @@ tlda_status tlda_create(tlda_ctx **out, int32_t vocab, const tlda_params *p, voi
   CA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
   CA(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   CA(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+  CA(cudaEventCreateWithFlags(&ctx->ev_q, cudaEventDisableTiming));
+  CA(cudaEventCreateWithFlags(&ctx->ev_zc, cudaEventDisableTiming));
+  CA(cudaEventCreateWithFlags(&ctx->ev_touch, cudaEventDisableTiming));
   CA(cudaStreamCreateWithFlags(&ctx->pstream, cudaStreamNonBlocking));
   CA(cudaEventCreateWithFlags(&ctx->ev_pass0, cudaEventDisableTiming));
   CA(cudaEventCreateWithFlags(&ctx->ev_pass1, cudaEventDisableTiming));
@@ -726,6 +767,9 @@ tlda_status tlda_destroy(tlda_ctx *ctx) {
   for (cudaEvent_t e : ctx->prof_pool) cudaEventDestroy(e);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+  if (ctx->ev_q) cudaEventDestroy(ctx->ev_q);
+  if (ctx->ev_zc) cudaEventDestroy(ctx->ev_zc);
+  if (ctx->ev_touch) cudaEventDestroy(ctx->ev_touch);
   if (ctx->side) cudaStreamDestroy(ctx->side);
   if (ctx->step_exec) cudaGraphExecDestroy(ctx->step_exec);
   if (ctx->pstream) cudaStreamDestroy(ctx->pstream);
@@ -796,7 +840,7 @@ static tlda_status step_common(tlda_ctx *ctx, const tlda_csr *batch, float *Phi,
   a.gdata_out = gdata_out;
   a.mode = mode;
   a.want_loss = loss_out ? 1 : 0;
-  const bool touch = wants_touch(ctx, a);
+  const bool touch = a.precision == TLDA_FP32 && wants_touch(ctx, a);  // the BF16 chain finds them beside its other work
   if (touch) launch_touch_batch(a, desc_of(batch), ctx->stream);
   else launch_set_desc(ctx->st, desc_of(batch), ctx->stream);
   if (a.PhiImg) launch_phi_img(a, ctx->stream);
@@ -901,26 +945,28 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
   if (loss_out && !no_wait) CK(cudaMallocHost(reinterpret_cast<void **>(&losses), sizeof(double) * n_batches));
   launch_begin_pass(ctx->st, ctx->descs, n_batches, ps);
   if (a.PhiImg) launch_phi_img(a, ps);
-  // device input: each step's reduction kernel finds the next batch's touched
-  // words beside its own work, the first batch's are found here (with host input
-  // the next batch is copied only after the step)
-  const bool ahead = !host && wants_touch(ctx, a);
+  // FP32, device input: each step's reduction kernel finds the next batch's
+  // touched words beside its own work, the first batch's are found here (with host
+  // input the next batch is copied only after the step; the BF16 chain has a side
+  // stream to find them on, where the reduction would wait for them: 4.26 against
+  // 3.98 ms a pass of 103 batches of 1936 to 3873 documents at K = 26)
+  const bool ahead = !host && by_word(a);
   if (ahead) {
-    a.touch_next = std::max(32, std::min(2 * ctx->num_sms, ctx->Bmax / 64));  // 16 nonzeros a document: one turn each
+    a.touch_next = std::max(64, std::min(2 * ctx->num_sms, ctx->Bmax / 32));  // 32 nonzeros a document: one turn each
     launch_touch(a, ps);
   }
   CKL();
   // one captured step, replayed per batch (not while the event profiler is on)
   const bool use_graph = ctx->prof_mask == 0;
   if (use_graph && !(ctx->step_exec && ctx->g_lr == lr && ctx->g_phi == Phi && ctx->g_loss == a.want_loss &&
-                     ctx->g_touch == a.touch_next)) {
+                     ctx->g_touch == a.touch_next && ctx->g_host == host)) {
     if (ctx->step_exec) {
       cudaGraphExecDestroy(ctx->step_exec);
       ctx->step_exec = nullptr;
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(ps, cudaStreamCaptureModeThreadLocal));
-    tlda_status cs = enqueue_step(ctx, a, ps, ahead);
+    tlda_status cs = enqueue_step(ctx, a, ps, ahead, host);
     cudaError_t ce = cudaStreamEndCapture(ps, &g);
     if (cs) {
       if (g) cudaGraphDestroy(g);
@@ -934,6 +980,7 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
     ctx->g_phi = Phi;
     ctx->g_loss = a.want_loss;
     ctx->g_touch = a.touch_next;
+    ctx->g_host = host;
   }
   for (int b = 0; b < n_batches && s == TLDA_OK; ++b) {
     if (host) {
@@ -951,7 +998,7 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
       }
     }
     if (use_graph) CK(cudaGraphLaunch(ctx->step_exec, ps));
-    else s = enqueue_step(ctx, a, ps, ahead);
+    else s = enqueue_step(ctx, a, ps, ahead, host);
     if (loss_out && s == TLDA_OK)
       CK(cudaMemcpyAsync(no_wait ? loss_out + b : losses + b, &ctx->st->loss, sizeof(double),
                          no_wait ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ps));
