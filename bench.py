@@ -868,10 +868,11 @@ def billion_main(args):
 
     def kernel_profile(c_, prec):
         """Per-kernel device times of one more pass over the first chunk (on a
-        copy of Phi, after the timed region), and the roofline of the two
-        dense contractions: [Q; Y] = [U; X] Phi, algorithmic 2 (n_t + B) D K
-        flop (Q is needed for the n_t touched words only), and
-        [X; U_t]^T [Z; Zc], 2 (B + n_t) D K flop."""
+        copy of Phi, after the timed region; a step has several launches of
+        some kinds), and the roofline of the two dense contractions: BF16
+        [Q; Y] = [U; X] Phi, algorithmic 2 (n_t + B) D K flop (Q is needed for
+        the n_t touched words only), and [X; U_t]^T [Z; Zc], 2 (B + n_t) D K;
+        FP32, by word, Q = U_t Phi and G = U_t^T (B + Zc), 2 n_t D K each."""
         n = min(chunk, args.billion_docs)
         c = gen.generate(0, n, out=buf)
         offs = list(range(0, n, B)) + [n]
@@ -892,12 +893,13 @@ def billion_main(args):
             pk, bound = peaks.get("bf16_tflops_sustained", PEAKS_FALLBACK["bf16_tflops_sustained"]), "tensor"
         else:
             pk, bound = alu_peak()["tflops"], "alu"
-        fl = 2.0 * float(np.sum(np.array(bt) + np.array(nt))) * sp.K * sp.K / len(bt)
-        out = {"ms_per_step": {k: v[1] / v[0] for k, v in pr.items() if v[0] > 0}, "peak_source": src,
+        rows = np.array(nt) + (np.array(bt) if prec == "bf16" else 0)
+        fl = 2.0 * float(np.sum(rows)) * sp.K * sp.K / len(bt)
+        out = {"ms_per_step": {k: v[1] / len(bt) for k, v in pr.items() if v[0] > 0}, "peak_source": src,
                "mean_touched_words": float(np.mean(nt))}
         for k in ("qy", "g_reduce"):
             if pr.get(k, (0, 0))[0] > 0:
-                ach = fl / (pr[k][1] / pr[k][0] / 1e3) / 1e12
+                ach = fl / (pr[k][1] / len(bt) / 1e3) / 1e12
                 out[k] = {"bound": bound, "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
                           "algorithmic_flop_per_launch": fl}
         return out
@@ -1107,9 +1109,9 @@ def main():
             # G1 = X^T Z, H = F^T Y, G2 = U_t^T Zc
             flops = float((2.0 * nnz_all * D + 4.0 * B_all * D * K + 4.0 * nt * D * K
                            + 4.0 * nnz_all * K).sum()) / len(B_all)
-        else:
-            flops = 2.0 * float((B_all + nt).sum()) * D * K / len(B_all)
-        ach = flops / (kms / launches / 1e3) / 1e12
+        else:  # the FP32 form's products run over the touched words only
+            flops = 2.0 * float((nt + (B_all if primary == "bf16" else 0)).sum()) * D * K / len(B_all)
+        ach = flops / (kms / (launches if dominant == "pass" else len(B_all)) / 1e3) / 1e12
         if primary == "bf16":
             pk, unit, bound = peaks.get("bf16_tflops_sustained", PEAKS_FALLBACK["bf16_tflops_sustained"]), "TFLOP/s", "tensor"
         else:
@@ -1120,7 +1122,7 @@ def main():
         # HBM-bound kernels: algorithmic bytes = the batch's CSR stream + X written
         xbytes = D * 4 if primary == "fp32" else D * 2 * 2
         byts = float(((B_all + 1) * 4 + nnz_all * 8 + B_all * xbytes).sum()) / len(B_all)
-        ach = byts / (kms / launches / 1e3) / 1e9
+        ach = byts / (kms / len(B_all) / 1e3) / 1e9
         pk = peaks.get("hbm_gbs", PEAKS_FALLBACK["hbm_gbs"])
         roof = {"bound": "hbm", "achieved": ach, "peak": pk, "unit": "GB/s", "frac": ach / pk}
     if roof is not None:
@@ -1214,10 +1216,11 @@ def main():
 
     if rank == 0:
         # kernels per step: fused BF16 form (D, K padded to 128): Phi-only x2,
-        # fused, reduction, step end; otherwise Phi-only x2, scan/whiten, Q/Y,
-        # R/Z/H, Zc, reduction over rows, reduction, step end
+        # fused, reduction; BF16 multi-kernel form: Phi-only x2, touched words,
+        # Q, scan/whiten, Y, R/Z/H, Zc, clearing, reduction over rows, reduction;
+        # FP32: Phi-only x2, Q, documents, reduction over words, reduction
         fused = primary == "bf16" and sp.K <= 128 and sp.K > 64
-        per_step_kernels = 5 if fused else 9
+        per_step_kernels = 4 if fused else 11 if primary == "bf16" else 6
         # persistent form: per cp_pass call over a device-resident corpus, the
         # prologue kernel (split points, Phi^T image, control block) and one
         # pass kernel for all of its steps
