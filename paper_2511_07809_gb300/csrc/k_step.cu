@@ -1073,13 +1073,27 @@ void launch_doc(const StepArgs &a, cudaStream_t s) {
 }
 
 // Rows t of B summed over the copies into the compact Zc32 (D or K above 128:
-// several blocks of k_gw_f32 read a row); launch_h_clear clears them afterwards.
+// several blocks of k_gw_f32 read a row); k_b_clear clears them afterwards.
 __global__ void __launch_bounds__(256) k_b_fold(StepArgs a) {
   const int lane = threadIdx.x & 31;
   for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
     const int m = a.widx[t];
     for (int col = lane * 4; col < a.Kp; col += 128)
       *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = word_sum(a, m, col);
+  }
+}
+
+// Their rows of B and flags cleared for the next batch (c is not part of this
+// form, and need not exist).  A kernel of its own: a warp that loads a row and
+// then stores to it waits for the load.
+__global__ void __launch_bounds__(256) k_b_clear(StepArgs a) {
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
+    const int m = a.widx[t];
+    for (int r = 0; r < a.nrep; ++r)
+      for (int col = lane * 4; col < a.Kp; col += 128)
+        *reinterpret_cast<float4 *>(a.H32 + ((long long)r * a.V + m) * a.Kp + col) = f4(0.f);
+    if (lane == 0) a.flag[m] = 0;
   }
 }
 
@@ -1219,7 +1233,7 @@ void launch_gw_f32(const StepArgs &a, cudaStream_t s) {
   } else {
     k_b_fold<<<4 * a.sms, 256, 0, s>>>(a);
     gw_launch<128, 128, 8, false>(a, dim3(a.nsplit, (a.Dp + 127) / 128, (a.Kp + 127) / 128), s);
-    launch_h_clear(a, s);
+    k_b_clear<<<4 * a.sms, 256, 0, s>>>(a);
   }
 }
 
