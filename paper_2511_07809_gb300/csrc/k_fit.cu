@@ -31,6 +31,8 @@ using namespace tlda;
 namespace {
 
 constexpr int kMaxFitV = 65536;
+constexpr int kOversample = 16;                    // columns of the fit's subspace beyond D
+constexpr int kMaxRitz = kMaxDim + kOversample;    // largest order of the dense FP64 kernels
 
 // ------------------------------------------------------------------ scan + pairs
 // One warp per document.  Only the pairs on or below the diagonal of P are
@@ -511,7 +513,7 @@ __device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q
 __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, int r, double *__restrict__ Et,
                                                        double *__restrict__ eval, int max_sweeps,
                                                        JacCtl *ctl) {
-  __shared__ double cs[2][kMaxDim / 2], sn[2][kMaxDim / 2];  // rows' pairs, columns' pairs of this block
+  __shared__ double cs[2][kMaxRitz / 2], sn[2][kMaxRitz / 2];  // rows' pairs, columns' pairs of this block
   __shared__ double red_o[kJacThreads / 32], red_t[kJacThreads / 32];
   __shared__ int s_ok, s_done;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
@@ -626,7 +628,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
 #pragma unroll
           for (int v = 0; v < 2; ++v) ev[u][v] = __ldcg(Et + ei[u][v]);
         }
-      if (mine) {
+      auto put_rotation = [&](int at, double apq, double app, double aqq) {
         double c = 1.0, sv = 0.0;
         const float fp = seed_f32(apq), fd = seed_f32(aqq - app);
         if (fp != 0.f) {  // an entry below FP32's range is left as it is
@@ -644,9 +646,14 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
           c = fma(2.0, q, -1.0);
           sv = 2.0 * hh * q;
         }
-        const int side = tid < kn ? 0 : 1, at = tid < kn ? tid : tid - kn;
-        cs[side][at] = c;
-        sn[side][at] = sv;
+        const int side = at < kn ? 0 : 1, of = at < kn ? at : at - kn;
+        cs[side][of] = c;
+        sn[side][of] = sv;
+      };
+      if (mine) put_rotation(tid, apq, app, aqq);
+      for (int w = tid + nt; w < kn + ln; w += nt) {  // a small grid's tiles have more pairs than threads
+        jac_pair(w < kn ? ka + w : la + w - kn, round, r, p, q);
+        put_rotation(w, __ldcg(A + p * r + q), __ldcg(A + p * r + p), __ldcg(A + q * r + q));
       }
       __syncthreads();
       auto rotate_block = [&](int k, int l, const double (&v)[4], const int (&base)[4]) {
@@ -729,7 +736,7 @@ __device__ void chol_inv_column(int c, int r, const double *LT, const double *in
 }
 
 // Cholesky factor and inverse of a symmetric positive definite r x r FP64
-// matrix A (overwritten), r <= 512: A = L L^T in panels of 32 columns, then
+// matrix A (overwritten), r <= kMaxRitz: A = L L^T in panels of 32 columns, then
 // X = L^-1 column by column.  Per panel every block factors the 32 x 32
 // diagonal block for itself, warps solve the rows below it, a grid barrier, then
 // the trailing entries take the panel's 32 terms, and another: 2 r/32 grid
@@ -749,7 +756,7 @@ constexpr int kCholNb = 32;
 __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A, int r, double *__restrict__ L,
                                                          double *__restrict__ LT, double *Linv, double *LinvT64,
                                                          float *LinvT32, int *status, JacCtl *ctl) {
-  __shared__ double Dc[kCholNb][kCholNb + 1], inv[kMaxDim];  // the diagonal block by columns: Dc[k][i]
+  __shared__ double Dc[kCholNb][kCholNb + 1], inv[kMaxRitz];  // the diagonal block by columns: Dc[k][i]
   __shared__ int s_ok;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5;
   const int gt = blockIdx.x * nt + tid, gn = G * nt, rr = r * r;
@@ -875,7 +882,8 @@ __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A
   };
   if (r <= 128) columns(std::integral_constant<int, 4>());
   else if (r <= 256) columns(std::integral_constant<int, 8>());
-  else columns(std::integral_constant<int, 16>());
+  else if (r <= 512) columns(std::integral_constant<int, 16>());
+  else columns(std::integral_constant<int, (kMaxRitz + 31) / 32>());
 }
 
 // B = C1 C2^-1 for r x r FP64 matrices (C2 general, row-major): Gauss-Jordan
@@ -1247,6 +1255,7 @@ tlda_status g64_exps(tlda_ctx *ctx, int **out) {
 // Diagonalises the symmetric r x r matrix A (device, overwritten): eigenvalues
 // to ev, eigenvector rows to Et.  Synchronises.
 tlda_status run_jacobi(tlda_ctx *ctx, double *A, int r, double *Et, double *ev, cudaStream_t s) {
+  if (r > kMaxRitz) return fail(ctx, TLDA_ERR_INVALID, "eigenproblem above the solver's order");
   JacCtl *ctl = nullptr;
   if (tlda_status st = coop_ctl(ctx, &ctl, s)) return st;
   int ms = 40;
@@ -1263,6 +1272,7 @@ tlda_status run_jacobi(tlda_ctx *ctx, double *A, int r, double *Et, double *ev, 
 // Enqueues k_chol_inv (asynchronous; failures land in *status).
 tlda_status run_chol_inv(tlda_ctx *ctx, double *A, int r, double *L, double *Z, double *Linv, double *LinvT64,
                          float *LinvT32, int *status, cudaStream_t s) {
+  if (r > kMaxRitz) return fail(ctx, TLDA_ERR_INVALID, "matrix above the Cholesky kernel's order");
   JacCtl *ctl = nullptr;
   if (tlda_status st = coop_ctl(ctx, &ctl, s)) return st;
   void *args[] = {&A, &r, &L, &Z, &Linv, &LinvT64, &LinvT32, &status, &ctl};
@@ -1290,7 +1300,7 @@ tlda_status chol_status(tlda_ctx *ctx, int st, const char *breakdown) {
 tlda_status finalize(tlda_ctx *ctx) {
   cudaStream_t s = ctx->stream;
   const int V = ctx->V, D = ctx->D;
-  int r = round_up(D + 16, 2);
+  int r = round_up(D + kOversample, 2);
   if (r > V) r = V - (V & 1);
   if (r < D) return fail(ctx, TLDA_ERR_INVALID, "vocabulary too small for the whitening dimension");
   unsigned long long TS[3];
