@@ -487,15 +487,18 @@ __device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q
   q = max(a, b);
 }
 
-// Cyclic Jacobi for a symmetric r x r FP64 matrix A (r even, global memory,
-// overwritten), round-robin ordering so each round applies r/2 disjoint
+// Cyclic Jacobi for a symmetric r x r FP64 matrix A0 (r even, global memory,
+// overwritten; A1: as much scratch), round-robin ordering so each round applies r/2 disjoint
 // rotations in parallel (Golub & Van Loan, "Matrix Computations", sec. 8.5,
 // parallel ordering).  Rotation of pair (p, q): tau = (a_qq - a_pp)/(2 a_pq),
 // t = sign(tau)/(|tau| + sqrt(1 + tau^2)), c = 1/sqrt(1 + t^2), s = t c.
 // Because the rotations of one round are disjoint, A <- J^T A J is applied in
 // one pass over the 2 x 2 blocks (pair k rows, pair l columns), each block
 // rotated on the left by pair k and on the right by pair l; the eigenvectors
-// are kept as rows, Et <- J^T Et.  Et starts as I; on return eval[i] = A_ii and
+// are kept as rows, Et <- J^T Et.  The rotations' entries are read by every tile
+// that holds one of the pairs while the diagonal tiles rotate them, so a round
+// reads A from one copy and writes it, whole, to the other; an entry of Et has one
+// reader and writer a round.  Et starts as I; on return eval[i] = A_ii and
 // row i of Et is its eigenvector.  Sweeps stop when the off-diagonal mass is
 // below 1e-26 r^2 of the total, i.e. entries near 1e-13 of the scale (or after
 // max_sweeps).
@@ -510,7 +513,7 @@ __device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q
 // Without the step an r = 216 solve takes 0.45 ms less of 6.9, but then the entries
 // that the last sweep leaves under the stopping rule, and with them the
 // eigenvectors at 1e-8, are others than with exact angles.
-__global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, int r, double *__restrict__ Et,
+__global__ void __launch_bounds__(kJacThreads) k_jacobi(double *A0, double *A1, int r, double *__restrict__ Et,
                                                        double *__restrict__ eval, int max_sweeps,
                                                        JacCtl *ctl) {
   __shared__ double cs[2][kMaxRitz / 2], sn[2][kMaxRitz / 2];  // rows' pairs, columns' pairs of this block
@@ -535,6 +538,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
   for (int u = 0; u < 4; ++u)
     if (tid + u * nt < ne) ek[u] = (tid + u * nt) / jn, ej[u] = (tid + u * nt) % jn;
   unsigned nbar = 0;
+  double *A = A0, *An = A1;  // this round's copy, the next one's
   for (int e = gt; e < rr; e += gn) {
     const int i = e / r, j = e % r;
     if (i < j) {
@@ -660,10 +664,10 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
         const double ck = cs[0][k], sk = sn[0][k], cl = cs[1][l], sl = sn[1][l];
         const double a1 = ck * v[0] - sk * v[2], b1 = ck * v[1] - sk * v[3];
         const double c1 = sk * v[0] + ck * v[2], d1 = sk * v[1] + ck * v[3];
-        A[base[0]] = cl * a1 - sl * b1;
-        A[base[1]] = sl * a1 + cl * b1;
-        A[base[2]] = cl * c1 - sl * d1;
-        A[base[3]] = sl * c1 + cl * d1;
+        An[base[0]] = cl * a1 - sl * b1;
+        An[base[1]] = sl * a1 + cl * b1;
+        An[base[2]] = cl * c1 - sl * d1;
+        An[base[3]] = sl * c1 + cl * d1;
       };
       auto rotate_pair = [&](int k, const double (&v)[2], const int (&base)[2]) {
         const double c = cs[0][k], sv = sn[0][k];
@@ -690,6 +694,9 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *__restrict__ A, 
         rotate_pair(w / jn, ev[0], ei[0]);
       }
       if (!jac_sync(ctl, ++nbar * G, &s_ok)) return;
+      double *const done = An;
+      An = A;
+      A = done;
     }
   }
   for (int i = gt; i < r; i += gn) eval[i] = __ldcg(A + i * r + i);
@@ -1252,14 +1259,14 @@ tlda_status g64_exps(tlda_ctx *ctx, int **out) {
   return TLDA_OK;
 }
 
-// Diagonalises the symmetric r x r matrix A (device, overwritten): eigenvalues
-// to ev, eigenvector rows to Et.  Synchronises.
-tlda_status run_jacobi(tlda_ctx *ctx, double *A, int r, double *Et, double *ev, cudaStream_t s) {
+// Diagonalises the symmetric r x r matrix A (device, overwritten, as is the r x r
+// scratch): eigenvalues to ev, eigenvector rows to Et.  Synchronises.
+tlda_status run_jacobi(tlda_ctx *ctx, double *A, double *scratch, int r, double *Et, double *ev, cudaStream_t s) {
   if (r > kMaxRitz) return fail(ctx, TLDA_ERR_INVALID, "eigenproblem above the solver's order");
   JacCtl *ctl = nullptr;
   if (tlda_status st = coop_ctl(ctx, &ctl, s)) return st;
   int ms = 40;
-  void *args[] = {&A, &r, &Et, &ev, &ms, &ctl};
+  void *args[] = {&A, &scratch, &r, &Et, &ev, &ms, &ctl};
   CKF(cudaLaunchCooperativeKernel((const void *)k_jacobi, dim3(coop_grid()), dim3(kJacThreads), args, 0, s));
   int hs[3];
   CKF(cudaMemcpyAsync(hs, &ctl->bar, sizeof hs, cudaMemcpyDeviceToHost, s));
@@ -1380,7 +1387,7 @@ tlda_status finalize(tlda_ctx *ctx) {
   k_rank1_fix<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(Z64, M1, m1q, V, r, sP, a0);
   gemm_tn64(Q64, r, Z64, r, Bm, r, r, r, V, ex, V, sms, s);
   CKF(cudaGetLastError());
-  if (tlda_status js = run_jacobi(ctx, Bm, r, Ev, ev, s)) return js;
+  if (tlda_status js = run_jacobi(ctx, Bm, G, r, Ev, ev, s)) return js;
   std::vector<double> hev(r), hEv((size_t)r * r);
   int hstat[2];
   CKF(cudaMemcpyAsync(hev.data(), ev, sizeof(double) * r, cudaMemcpyDeviceToHost, s));
@@ -1729,7 +1736,7 @@ tlda_status online_rewhiten(tlda_ctx *ctx) {
   CKF(cudaStreamSynchronize(s));
   if (tlda_status st = chol_status(ctx, hstat[0], "sketch basis lost rank (CholeskyQR breakdown)")) return st;
   if (tlda_status st = chol_status(ctx, hstat[1], "Q^T Omega is singular")) return st;
-  if (tlda_status js = run_jacobi(ctx, w.Bm, r, w.Et, w.ev, s)) return js;
+  if (tlda_status js = run_jacobi(ctx, w.Bm, w.G, r, w.Et, w.ev, s)) return js;
   std::vector<double> hev(r), hEv((size_t)r * r);
   CKF(cudaMemcpyAsync(hev.data(), w.ev, sizeof(double) * r, cudaMemcpyDeviceToHost, s));
   CKF(cudaMemcpyAsync(hEv.data(), w.Et, sizeof(double) * r * r, cudaMemcpyDeviceToHost, s));
