@@ -107,9 +107,10 @@ __device__ __forceinline__ NzChunk load_chunk(const BatchDesc &b, int V, int bas
 
 // Whether document row [lo, hi) lies in the batch's nonzero range (the offsets
 // at its first and last document): outside it the row offsets decrease
-// somewhere, and k_touch has not seen the words.
+// somewhere, and k_touch has not seen the words.  Nor has it where the batch's
+// first offset is out of range: then no row is taken.
 __device__ __forceinline__ bool row_in_batch(const BatchDesc &b, int lo, int hi, int first, int last) {
-  return lo >= b.nz_base && hi >= lo && lo >= first && hi <= last;
+  return first >= b.nz_base && lo >= first && hi >= lo && hi <= last;
 }
 
 // Touched words of the batch into widx (compact, no fixed order) with flag set.
