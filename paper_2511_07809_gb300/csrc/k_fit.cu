@@ -758,11 +758,12 @@ __device__ void chol_inv_column(int c, int r, const double *LT, const double *in
 // 1185 -> 287 us at r = 216, 345 -> 85 us at r = 66 (19 us of each whole panel).
 // L (lower, zeros above) and LT (its transpose, scratch) are required; Linv,
 // LinvT64 = L^-T and LinvT32 (FP32) are written when given.  status: 1 if a
-// pivot was not positive (it is taken as 1), 2 if a grid barrier expired.
+// pivot was not positive (it is taken as 1), 2 if a grid barrier expired.  *ill,
+// when given: set to 1 if the diagonal of L spans more than 1e5.
 constexpr int kCholNb = 32;
 __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A, int r, double *__restrict__ L,
                                                          double *__restrict__ LT, double *Linv, double *LinvT64,
-                                                         float *LinvT32, int *status, JacCtl *ctl) {
+                                                         float *LinvT32, int *status, int *ill, JacCtl *ctl) {
   __shared__ double Dc[kCholNb][kCholNb + 1], inv[kMaxRitz];  // the diagonal block by columns: Dc[k][i]
   __shared__ int s_ok;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5;
@@ -868,6 +869,23 @@ __global__ void __launch_bounds__(kJacThreads) k_chol_inv(double *__restrict__ A
       if (tid == 0) atomicMax(status, 2);
       return;
     }
+  }
+  if (ill && blockIdx.x == 0 && w == 0) {  // every block has the whole of inv
+    double mn = inv[0], mx = inv[0];
+    bool num = true;
+    for (int i = lane; i < r; i += 32) {
+      const double v = inv[i];
+      num = num && v > 0.0;
+      mn = fmin(mn, v);
+      mx = fmax(mx, v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    num = __all_sync(0xffffffffu, num);
+    if (lane == 0 && !(num && mx <= 1e5 * mn)) *ill = 1;
   }
   if (!Linv && !LinvT64 && !LinvT32) return;
   // warp w of block b takes columns b + G w, b + G (w + 8), ...: one a quarter first
@@ -1278,11 +1296,11 @@ tlda_status run_jacobi(tlda_ctx *ctx, double *A, double *scratch, int r, double 
 
 // Enqueues k_chol_inv (asynchronous; failures land in *status).
 tlda_status run_chol_inv(tlda_ctx *ctx, double *A, int r, double *L, double *Z, double *Linv, double *LinvT64,
-                         float *LinvT32, int *status, cudaStream_t s) {
+                         float *LinvT32, int *status, cudaStream_t s, int *ill = nullptr) {
   if (r > kMaxRitz) return fail(ctx, TLDA_ERR_INVALID, "matrix above the Cholesky kernel's order");
   JacCtl *ctl = nullptr;
   if (tlda_status st = coop_ctl(ctx, &ctl, s)) return st;
-  void *args[] = {&A, &r, &L, &Z, &Linv, &LinvT64, &LinvT32, &status, &ctl};
+  void *args[] = {&A, &r, &L, &Z, &Linv, &LinvT64, &LinvT32, &status, &ill, &ctl};
   CKF(cudaLaunchCooperativeKernel((const void *)k_chol_inv, dim3(coop_grid()), dim3(kJacThreads), args, 0, s));
   return TLDA_OK;
 }
@@ -1356,27 +1374,43 @@ tlda_status finalize(tlda_ctx *ctx) {
     c.take(part, splits > 1 ? splits * Vr : 1);
     c.take(status, 2);
   }));
-  CKF(cudaMemsetAsync(status, 0, 2 * sizeof(int), s));
   k_m1<<<(V + 255) / 256, 256, 0, s>>>(ctx->Ccnt, ctx->TS, V, M1);
   k_m2_mirror<<<dim3((V + 31) / 32, (V + 31) / 32), 256, 0, s>>>(ctx->P64, M1, V, sP, a0, M2);
   k_gauss<<<(unsigned)(((long long)V * r + 255) / 256), 256, 0, s>>>(Om, (long long)V * r, ctx->p.seed * 0x100000001B3ull + 17);
   // one CholeskyQR pass: out = in L^-T with L L^T = in^T in (FP64 Gram)
   auto cholqr_pass = [&](const float *in, float *out) -> tlda_status {
     gemm_tn64(in, r, in, r, G, r, r, r, V, ex, V, sms, s);
-    if (tlda_status st = run_chol_inv(ctx, G, r, Linv, Zr, nullptr, nullptr, LinvT32, status, s)) return st;
+    if (tlda_status st = run_chol_inv(ctx, G, r, Linv, Zr, nullptr, nullptr, LinvT32, status, s, status + 1)) return st;
     sgemm(in, r, LinvT32, r, out, V, r, r, nullptr, 1, s);
     return TLDA_OK;
   };
-  // Y = M2 Q, then one CholeskyQR pass.  A single pass keeps the same span, and
-  // the columns orthonormal to 1e-16 times the squared condition of Y, which is
-  // all that the next product needs; a second one is taken at the end.
-  sgemm(M2, V, Om, r, Y, V, r, V, part, splits, s);
-  if (tlda_status st = cholqr_pass(Y, Qf)) return st;
+  // Y = M2 Q, then CholeskyQR.  A single pass keeps the same span, and the columns
+  // orthonormal to the FP32 rounding of Q times the condition of Y.  While that is
+  // small the next product needs no more, and a second pass is taken at the end
+  // only; where a factor's diagonal spans more than 1e5 (a spectrum that falls by
+  // as much within r columns) the loss would grow from product to product until
+  // the factor breaks down, and the iteration starts over with two passes each.
   const int n_iter = 24;
-  for (int it = 0; it < n_iter; ++it) {
-    sgemm(M2, V, Qf, r, Y, V, r, V, part, splits, s);
-    if (tlda_status st = cholqr_pass(Y, Qf)) return st;
+  auto iterate = [&](int passes) -> tlda_status {
+    CKF(cudaMemsetAsync(status, 0, 2 * sizeof(int), s));
+    for (int it = 0; it <= n_iter; ++it) {
+      sgemm(M2, V, it ? Qf : Om, r, Y, V, r, V, part, splits, s);
+      if (tlda_status st = cholqr_pass(Y, Qf)) return st;
+      if (passes == 2) {
+        if (tlda_status st = cholqr_pass(Qf, Y)) return st;
+        std::swap(Qf, Y);
+      }
+    }
+    return TLDA_OK;
+  };
+  int hstat[2];
+  for (int passes = 1; passes <= 2; ++passes) {
+    if (tlda_status st = iterate(passes)) return st;
+    CKF(cudaMemcpyAsync(hstat, status, sizeof hstat, cudaMemcpyDeviceToHost, s));
+    CKF(cudaStreamSynchronize(s));
+    if (!hstat[1] && hstat[0] != 1) break;
   }
+  if (tlda_status st = chol_status(ctx, hstat[0], "subspace basis lost rank (CholeskyQR breakdown)")) return st;
   // FP64 Rayleigh-Ritz on the exact M2 = sP P - a0 M1 M1^T
   // one FP64 CholeskyQR pass makes Q64 orthonormal to FP64 accuracy
   gemm_tn64(Qf, r, Qf, r, G, r, r, r, V, ex, V, sms, s);
@@ -1389,7 +1423,6 @@ tlda_status finalize(tlda_ctx *ctx) {
   CKF(cudaGetLastError());
   if (tlda_status js = run_jacobi(ctx, Bm, G, r, Ev, ev, s)) return js;
   std::vector<double> hev(r), hEv((size_t)r * r);
-  int hstat[2];
   CKF(cudaMemcpyAsync(hev.data(), ev, sizeof(double) * r, cudaMemcpyDeviceToHost, s));
   CKF(cudaMemcpyAsync(hEv.data(), Ev, sizeof(double) * r * r, cudaMemcpyDeviceToHost, s));
   CKF(cudaMemcpyAsync(hstat, status, sizeof hstat, cudaMemcpyDeviceToHost, s));
