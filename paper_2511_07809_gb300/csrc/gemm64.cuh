@@ -46,17 +46,19 @@ constexpr int kG64DigBytes = kG64Dig * kG64Tile * kG64Ld * 2;  // one operand's 
 constexpr int kG64RawLd = kG64Tile + 1;                    // raw slab row (terms x tile), in elements
 constexpr int kG64RawElems = 64 * 33 > kG64Slab * kG64RawLd ? 64 * 33 : kG64Slab * kG64RawLd;
 constexpr int kExpNan = 1 << 20;                           // exponent that marks an infinity or NaN
+constexpr int kExpZero = -(1 << 16);                       // below that of every number
 
 template <class TA, class TB>
 constexpr int g64_smem() {
   return 2 * kG64DigBytes + 2 * kG64RawElems * (int)(sizeof(TA) + sizeof(TB));
 }
 
-// Exponent e with |x| < 2^e (FP64 bits); kExpNan for an infinity or NaN, a
-// value below every other for zero.
+// Exponent e with |x| < 2^e (FP64 bits); kExpNan for an infinity or NaN,
+// kExpZero for zero.
 __device__ __forceinline__ int exp_above(double x) {
-  const int E = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
-  return E == 0x7ff ? kExpNan : E - 1022;
+  const long long b = __double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7ff);
+  return E == 0x7ff ? kExpNan : b << 1 == 0 ? kExpZero : E - 1022;  // integer units: an FP64 test takes 64 cycles
 }
 
 // e[c] = the largest exp_above over the rows of column c of a rows x cols matrix
@@ -68,11 +70,12 @@ __global__ void __launch_bounds__(256) k_col_exp(const T *x, int ld, int rows, i
   __shared__ int red[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
   const int r0 = blockIdx.y * slab, r1 = min(rows, r0 + slab);
-  int m = -(1 << 16);
+  int m = kExpZero;
   if (c < cols) {
 #pragma unroll 8
     for (int r = r0 + w; r < r1; r += 8) {
       const int v = exp_above((double)x[(long long)r * ld + c]);
+      if (v == kExpZero) continue;  // add[r] of a term without entries is kExpZero too
       if (v != kExpNan) m = max(m, v + (add ? add[r] : 0));
       else if (!FIN) m = kExpNan;
     }
@@ -92,11 +95,12 @@ template <class T>
 __global__ void __launch_bounds__(256) k_row_exp(const T *x, int ld, int rows, int cols, const int *sub, int *e) {
   const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (r >= rows) return;
-  int m = -(1 << 16);
+  int m = kExpZero;
 #pragma unroll 4
   for (int c = lane; c < cols; c += 32) {
     const int v = exp_above((double)x[(long long)r * ld + c]);
-    m = max(m, v == kExpNan ? v : v - sub[c]);
+    // a zero has no say in its row's exponent (in a column of zeros v - sub is 0)
+    if (v != kExpZero) m = max(m, v == kExpNan ? v : v - sub[c]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
