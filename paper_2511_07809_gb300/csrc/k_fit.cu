@@ -454,9 +454,10 @@ __device__ bool jac_sync(JacCtl *ctl, unsigned target, int *s_ok) {
 
 // FP64 to FP32 and back on the integer units, toward zero: a conversion takes
 // the FP64 pipe 65 cycles.  Outside FP32's normal range: 0 below, infinity above.
-__device__ __forceinline__ float seed_f32(double x) {
+// off: 896 plus the exponent of a power of two that x is divided by (positive).
+__device__ __forceinline__ float seed_f32(double x, int off = 896) {
   const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff) - 896;  // FP32 exponent field
+  const int e = (int)((b >> 52) & 0x7ff) - off;  // FP32 exponent field
   const uint32_t m = (uint32_t)(b >> 29) & 0x7fffffu, s = (uint32_t)(b >> 32) & 0x80000000u;
   return __uint_as_float(s | (e <= 0 ? 0u : e >= 255 ? 0x7f800000u : ((uint32_t)e << 23) | m));
 }
@@ -510,6 +511,8 @@ __device__ __forceinline__ void jac_pair(int k, int round, int r, int &p, int &q
 // to 1e-14 by one Newton step whose rest is FP64, with c = (1 - h^2)/(1 + h^2) and
 // s = 2 h/(1 + h^2) for the tangent h of its half (an FP64 division or square root
 // takes 430 to 680 cycles here): the rotation is orthogonal to FP64 rounding.
+// FP32 takes the entries relative to the norm of A, so that any scale will do: an
+// entry 2^-126 below the norm is left as it is, far under the stopping rule.
 // Without the step an r = 216 solve takes 0.45 ms less of 6.9, but then the entries
 // that the last sweep leaves under the stopping rule, and with them the
 // eigenvectors at 1e-8, are others than with exact angles.
@@ -518,7 +521,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *A0, double *A1, 
                                                        JacCtl *ctl) {
   __shared__ double cs[2][kMaxRitz / 2], sn[2][kMaxRitz / 2];  // rows' pairs, columns' pairs of this block
   __shared__ double red_o[kJacThreads / 32], red_t[kJacThreads / 32];
-  __shared__ int s_ok, s_done;
+  __shared__ int s_ok, s_done, s_off;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
   const int gt = blockIdx.x * nt + tid, gn = G * nt;
   const int h = r / 2, rr = r * r;
@@ -586,10 +589,14 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *A0, double *A1, 
         so += __shfl_xor_sync(0xffffffffu, so, m);
         st += __shfl_xor_sync(0xffffffffu, st, m);
       }
-      if (tid == 0) s_done = so <= 1e-26 * (double)r * r * st;
+      if (tid == 0) {
+        s_done = so <= 1e-26 * (double)r * r * st;
+        s_off = 896 + (((__double2hiint(st) >> 20) & 0x7ff) - 1023) / 2;  // half the exponent of the squared norm
+      }
     }
     __syncthreads();
     if (s_done) break;
+    const int off = s_off;
     for (int round = 0; round < r - 1; ++round) {
       double x[2][4], ev[4][2];
       int bx[2][4], ei[4][2];
@@ -634,15 +641,15 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(double *A0, double *A1, 
         }
       auto put_rotation = [&](int at, double apq, double app, double aqq) {
         double c = 1.0, sv = 0.0;
-        const float fp = seed_f32(apq), fd = seed_f32(aqq - app);
-        if (fp != 0.f) {  // an entry below FP32's range is left as it is
+        const float fp = seed_f32(apq, off), fd = seed_f32(aqq - app, off);
+        if (fp != 0.f) {
           const float tau = __fdividef(0.5f * fd, fp), f = fabsf(tau);
           const float t = __frcp_rn(f + __fsqrt_rn(fmaf(f, f, 1.f)));
           const float h1 = __fdividef(t, 1.f + __fsqrt_rn(fmaf(t, t, 1.f)));  // tan of half the angle, at most 0.42
           double hh = widen_f32(tau < 0.f ? -h1 : h1);
           // Newton from the rest that this angle would leave (times (1 + h^2)^2)
           const double u = fma(-hh, hh, 1.0), v = 2.0 * hh, uv = u * v, uu = fma(u, u, -v * v);
-          const float rest = seed_f32(fma(uu, apq, -uv * (aqq - app)));
+          const float rest = seed_f32(fma(uu, apq, -uv * (aqq - app)), off);
           const float slope = fmaf(seed_f32(uu), fd, 4.f * seed_f32(uv) * fp);
           hh += widen_f32(__fdividef(0.5f * fmaf(h1, h1, 1.f) * rest, slope));
           const double w = fma(hh, hh, 1.0);
