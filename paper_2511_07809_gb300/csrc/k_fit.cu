@@ -1765,9 +1765,10 @@ tlda_status online_rewhiten(tlda_ctx *ctx) {
   if (tlda_status st = cholqr_pass(w.Y, w.Q1, w.L1)) return st;
   if (tlda_status st = cholqr_pass(w.Q1, w.Q2, w.L2)) return st;
   gemm_tn64(w.Q2, r, ctx->on_Om, r, w.C2, r, r, r, V, ex, V, sms, s);  // Q^T Omega
-  // Q^T Y = R = (L1 L2)^T = L2^T L1^T
+  // Q^T Y = R = (L1 L2)^T = L2^T L1^T, in plain FP64 (its rows fall with the spectrum)
   k_transpose_rr<<<(r * r + 255) / 256, 256, 0, s>>>(w.L1, r, w.L1T);
-  gemm_tn64(w.L2, r, w.L1T, r, w.C1, r, r, r, r, ex, V, sms, s);
+  k_transpose_rr<<<(r * r + 255) / 256, 256, 0, s>>>(w.L2, r, w.Ms);
+  k_small_nn<<<r, 256, 0, s>>>(w.Ms, w.L1T, r, r, nullptr, w.C1);
   // B = (Q^T Y)(Q^T Omega)^-1, symmetrised by the eigensolver
   if (tlda_status st = run_solve_right(ctx, w.C1, w.C2, r, w.Ms, w.Rs, w.Bm, status + 1, s)) return st;
   CKF(cudaGetLastError());
