@@ -474,9 +474,9 @@ tlda_status tlda_selftest_barrier(void *cuda_stream, int32_t *blocks_out, int32_
  *   0 scan_whiten  1 qy  2 rz  3 zh  4 g_reduce  5 reduce_update
  *   6 phi_gram  7 phi_terms (6 and 7 run on the context's side stream)
  * A step may launch several kernels under one id: 0 the whitening or the batch
- * statistics, and the touched words; 1 the rows of Q and those of Y, the former
- * on the side stream; 2 in the FP32 form without the loss the documents' Y, Z
- * and scatter; 3 the same-token rows and the clearing of H and c.
+ * statistics, and the touched words (BF16: on a side stream); 2 in the FP32 form
+ * without the loss the documents' Y, Z and scatter; 3 the same-token rows and the
+ * clearing of H and c (BF16: on a side stream).
  *   8 fused (BF16 form with D, K in (64, 128]: replaces kernels 0-4)
  *   9 pass (the persistent kernel of tlda_cp_pass in that form: one launch
  *     runs every step of the pass, kernels 0-8 do not run).

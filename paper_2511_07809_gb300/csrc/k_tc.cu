@@ -32,10 +32,10 @@ __host__ __device__ constexpr int tc_stages(int kp) { return kp <= 256 ? 4 : kp 
 __host__ __device__ constexpr int tc_stage_bytes(int kp) { return 128 * 128 + kp * 128; }
 
 // ------------------------------------------------------------------ Q and Y
-// Rows of [U; X] from `first` on, up to V (part 0: Q, which needs no document) or
-// up to V + n_docs (part 1: Y).
+// Rows of [U; X] up to V + n_docs; without the same-token correction, which alone
+// reads Q, from V on.
 template <int KP>
-__global__ void __launch_bounds__(128) k_qy_tc(StepArgs a, int part, const __grid_constant__ CUtensorMap tmA) {
+__global__ void __launch_bounds__(128) k_qy_tc(StepArgs a, const __grid_constant__ CUtensorMap tmA) {
   constexpr int NST = tc_stages(KP), NH = KP > 256 ? 2 : 1, NN = KP / NH;
   constexpr int A_BYTES = 128 * 128, B_BYTES = KP * 128, STAGE = A_BYTES + B_BYTES;
   extern __shared__ unsigned char smem_raw[];
@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(128) k_qy_tc(StepArgs a, int part, const __gri
   uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nd = a.st->cur.n_docs;
-  const int rows = part ? a.V + nd : a.V;
-  const int r0 = (part ? a.V : 0) + blockIdx.x * 128;
+  const int rows = a.V + nd;
+  const int r0 = (a.same_token ? 0 : a.V) + blockIdx.x * 128;
   if (r0 >= rows) return;
   const int KA = a.Dp / 64;
   if (tid == 0) {
@@ -383,13 +383,13 @@ int tc_smem() {
 }
 
 template <int KP>
-void qy_launch(const StepArgs &a, const TcMaps &m, cudaStream_t s, int part) {
+void qy_launch(const StepArgs &a, const TcMaps &m, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_qy_tc<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<KP>());
     attr = true;
   }
-  k_qy_tc<KP><<<((part ? a.Bmax : a.V) + 127) / 128, 128, tc_smem<KP>(), s>>>(a, part, m.ux);
+  k_qy_tc<KP><<<((a.same_token ? a.V : 0) + a.Bmax + 127) / 128, 128, tc_smem<KP>(), s>>>(a, m.ux);
 }
 
 template <int KP>
@@ -424,21 +424,21 @@ void *tc_make_maps(const __nv_bfloat16 *UX16, const __nv_bfloat16 *ZU16, const _
 
 void tc_free_maps(void *p) { delete static_cast<TcMaps *>(p); }
 
-#define TLDA_KP_DISPATCH(F, ...)                                  \
+#define TLDA_KP_DISPATCH(F)                                       \
   switch (a.Kp) {                                                 \
-    case 64: return F<64>(a, m, s, ##__VA_ARGS__);                \
-    case 128: return F<128>(a, m, s, ##__VA_ARGS__);              \
-    case 192: return F<192>(a, m, s, ##__VA_ARGS__);              \
-    case 256: return F<256>(a, m, s, ##__VA_ARGS__);              \
-    case 320: return F<320>(a, m, s, ##__VA_ARGS__);              \
-    case 384: return F<384>(a, m, s, ##__VA_ARGS__);              \
-    case 448: return F<448>(a, m, s, ##__VA_ARGS__);              \
-    default: return F<512>(a, m, s, ##__VA_ARGS__);               \
+    case 64: return F<64>(a, m, s);                               \
+    case 128: return F<128>(a, m, s);                             \
+    case 192: return F<192>(a, m, s);                             \
+    case 256: return F<256>(a, m, s);                             \
+    case 320: return F<320>(a, m, s);                             \
+    case 384: return F<384>(a, m, s);                             \
+    case 448: return F<448>(a, m, s);                             \
+    default: return F<512>(a, m, s);                              \
   }
 
-void launch_qy_tc(const StepArgs &a, cudaStream_t s, int part) {
+void launch_qy_tc(const StepArgs &a, cudaStream_t s) {
   const TcMaps &m = *static_cast<const TcMaps *>(a.tc_maps);
-  TLDA_KP_DISPATCH(qy_launch, part)
+  TLDA_KP_DISPATCH(qy_launch)
 }
 
 void launch_g_tc(const StepArgs &a, cudaStream_t s) {

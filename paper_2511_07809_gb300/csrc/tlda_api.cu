@@ -162,9 +162,8 @@ bool wants_touch(const tlda_ctx *ctx, const StepArgs &a) {
 // terms on the side stream, the data-term chain on the main stream, then the
 // reduction and update once both are done.
 // With `touched`, the batch's touched words are there already (an earlier step's
-// reduction kernel or the caller found them); with `host`, the batch was copied
-// from the host just before.
-tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false, bool host = false) {
+// reduction kernel or the caller found them; FP32 only).
+tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false) {
   const bool tc = a.precision == TLDA_BF16;
   auto fork_phi = [&]() -> tlda_status {
     CK(cudaEventRecord(ctx->ev_fork, main));
@@ -175,33 +174,26 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
     CK(cudaEventRecord(ctx->ev_join, ctx->side));
     return TLDA_OK;
   };
-  const bool tc_chain = tc && !ctx->fused;
-  // beside k_doc in the FP32 form by word (its warps wait for memory), not beside
-  // the product before it; behind Q in the BF16 chain
-  if (!tc_chain && !by_word(a))
-    if (tlda_status s = fork_phi()) return s;
-  // Q = U Phi needs no document: on the side stream beside the whitening (57 of the
-  // 95 us of [Q; Y] at V = 100,000 and K = 300), but for wide steps on copied input,
-  // which it slows (us a pass, beside the whitening against before Y: 4 batches of
-  // 33781 documents at V = 98359, K = 250 from the host 2873 against 2612, from the
-  // device 1610 against 1621; 103 batches of 1936 to 3873 at V = 1341, K = 26 from
-  // the host 6272 against 6375, from the device 3998 against 4243)
-  const bool q_side = tc_chain && a.same_token && !(host && a.Kp > 64);
-  if (tc_chain && a.same_token) {
+  // The BF16 chain finds the touched words, which zc reads first, and clears H and
+  // c beside its other work.  On the side stream with the Phi-only terms: a branch
+  // more costs a narrow step more than it hides (us a pass, one against two side
+  // streams: 146 batches of 2000 documents at K = 9 6860 against 7200, 100 batches
+  // of 2048 at K = 50 3880 against 4120).  Where those terms are long (wide, with
+  // the loss) they would hold the clearing up: on a stream of its own (32 batches of
+  // 2500 documents at K = 266 from the host 8960 against 8350, 4 of 33781 at K = 250
+  // 2520 against 2430).  Q on a stream of its own too, apart from Y, was slower in
+  // narrow steps (7130 and 4070) and no faster in wide ones.
+  const bool beside = tc && !ctx->fused && a.same_token;
+  const cudaStream_t aux = a.want_loss && a.Kp > 64 ? ctx->side2 : ctx->side;
+  if (beside) {
     CK(cudaEventRecord(ctx->ev_fork, main));
-    CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
-    if (q_side) {
-      Prof p(ctx, kQY, ctx->side);
-      launch_qy_tc(a, ctx->side, 0);
-      CK(cudaEventRecord(ctx->ev_q, ctx->side));
-    }
-    if (!touched) {  // the touched words are read by zh only
-      Prof p(ctx, kWhiten, ctx->side);
-      launch_touch(a, ctx->side);
-    }
-    CK(cudaEventRecord(ctx->ev_touch, ctx->side));
+    CK(cudaStreamWaitEvent(aux, ctx->ev_fork, 0));
+    { Prof p(ctx, kWhiten, aux); launch_touch(a, aux); }
+    CK(cudaEventRecord(ctx->ev_touch, aux));
   }
-  if (tc_chain)
+  // beside k_doc in the FP32 form by word (its warps wait for memory), not beside
+  // the product before it
+  if (!by_word(a))
     if (tlda_status s = fork_phi()) return s;
   if (tc && ctx->fused) {
     // the fused kernel fills its SMs' shared memory: it leaves kPhiSMs SMs
@@ -218,26 +210,21 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
   } else {
     if (!tc && a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
     { Prof p(ctx, kWhiten, main); launch_whiten(a, main); }
-    {
-      Prof p(ctx, kQY, main);
-      if (tc && a.same_token && !q_side) launch_qy_tc(a, main, 0);
-      if (tc) launch_qy_tc(a, main, 1);
-      else launch_qy_f32(a, main);
-    }
-    if (q_side) CK(cudaStreamWaitEvent(main, ctx->ev_q, 0));
+    { Prof p(ctx, kQY, main); if (tc) launch_qy_tc(a, main); else launch_qy_f32(a, main); }
     { Prof p(ctx, kRZ, main); launch_rz(a, main); }
-    if (tc && a.same_token) CK(cudaStreamWaitEvent(main, ctx->ev_touch, 0));
+    if (beside) CK(cudaStreamWaitEvent(main, ctx->ev_touch, 0));
     if (a.same_token) { Prof p(ctx, kZH, main); if (tc) launch_zh_tc(a, main); else launch_zh_f32(a, main); }
-    if (tc && a.same_token) {  // H and c are cleared beside the last product
+    if (beside) {  // H and c are cleared beside the last product
       CK(cudaEventRecord(ctx->ev_zc, main));
-      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_zc, 0));
-      { Prof p(ctx, kZH, ctx->side); launch_h_clear(a, ctx->side); }
-      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+      CK(cudaStreamWaitEvent(aux, ctx->ev_zc, 0));
+      { Prof p(ctx, kZH, aux); launch_h_clear(a, aux); }
+      CK(cudaEventRecord(aux == ctx->side ? ctx->ev_join : ctx->ev_clear, aux));
     }
     { Prof p(ctx, kG, main); if (tc) launch_g_tc(a, main); else launch_g_f32(a, main); }
   }
   CKL();
   CK(cudaStreamWaitEvent(main, ctx->ev_join, 0));
+  if (beside && aux != ctx->side) CK(cudaStreamWaitEvent(main, ctx->ev_clear, 0));
   { Prof p(ctx, kReduceUpdate, main); launch_reduce_update(a, main); }
   CKL();
   return TLDA_OK;
@@ -671,9 +658,10 @@ tlda_status tlda_create(tlda_ctx **out, int32_t vocab, const tlda_params *p, voi
   CA(cudaGetDevice(&ctx->device));
   CA(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
   CA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
+  CA(cudaStreamCreateWithFlags(&ctx->side2, cudaStreamNonBlocking));
   CA(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   CA(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
-  CA(cudaEventCreateWithFlags(&ctx->ev_q, cudaEventDisableTiming));
+  CA(cudaEventCreateWithFlags(&ctx->ev_clear, cudaEventDisableTiming));
   CA(cudaEventCreateWithFlags(&ctx->ev_zc, cudaEventDisableTiming));
   CA(cudaEventCreateWithFlags(&ctx->ev_touch, cudaEventDisableTiming));
   CA(cudaStreamCreateWithFlags(&ctx->pstream, cudaStreamNonBlocking));
@@ -767,10 +755,11 @@ tlda_status tlda_destroy(tlda_ctx *ctx) {
   for (cudaEvent_t e : ctx->prof_pool) cudaEventDestroy(e);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  if (ctx->ev_q) cudaEventDestroy(ctx->ev_q);
+  if (ctx->ev_clear) cudaEventDestroy(ctx->ev_clear);
   if (ctx->ev_zc) cudaEventDestroy(ctx->ev_zc);
   if (ctx->ev_touch) cudaEventDestroy(ctx->ev_touch);
   if (ctx->side) cudaStreamDestroy(ctx->side);
+  if (ctx->side2) cudaStreamDestroy(ctx->side2);
   if (ctx->step_exec) cudaGraphExecDestroy(ctx->step_exec);
   if (ctx->pstream) cudaStreamDestroy(ctx->pstream);
   if (ctx->ev_pass0) cudaEventDestroy(ctx->ev_pass0);
@@ -959,14 +948,14 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
   // one captured step, replayed per batch (not while the event profiler is on)
   const bool use_graph = ctx->prof_mask == 0;
   if (use_graph && !(ctx->step_exec && ctx->g_lr == lr && ctx->g_phi == Phi && ctx->g_loss == a.want_loss &&
-                     ctx->g_touch == a.touch_next && ctx->g_host == host)) {
+                     ctx->g_touch == a.touch_next)) {
     if (ctx->step_exec) {
       cudaGraphExecDestroy(ctx->step_exec);
       ctx->step_exec = nullptr;
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(ps, cudaStreamCaptureModeThreadLocal));
-    tlda_status cs = enqueue_step(ctx, a, ps, ahead, host);
+    tlda_status cs = enqueue_step(ctx, a, ps, ahead);
     cudaError_t ce = cudaStreamEndCapture(ps, &g);
     if (cs) {
       if (g) cudaGraphDestroy(g);
@@ -980,7 +969,6 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
     ctx->g_phi = Phi;
     ctx->g_loss = a.want_loss;
     ctx->g_touch = a.touch_next;
-    ctx->g_host = host;
   }
   for (int b = 0; b < n_batches && s == TLDA_OK; ++b) {
     if (host) {
@@ -998,7 +986,7 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
       }
     }
     if (use_graph) CK(cudaGraphLaunch(ctx->step_exec, ps));
-    else s = enqueue_step(ctx, a, ps, ahead, host);
+    else s = enqueue_step(ctx, a, ps, ahead);
     if (loss_out && s == TLDA_OK)
       CK(cudaMemcpyAsync(no_wait ? loss_out + b : losses + b, &ctx->st->loss, sizeof(double),
                          no_wait ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ps));

@@ -189,8 +189,8 @@ struct NvtxRange {
 struct tlda_ctx {
   int V = 0, D = 0, K = 0, Dp = 0, Kp = 0, Bmax = 0;
   tlda_params p{};
-  cudaStream_t stream = nullptr, side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_q = nullptr, ev_touch = nullptr, ev_zc = nullptr;
+  cudaStream_t stream = nullptr, side = nullptr, side2 = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_touch = nullptr, ev_clear = nullptr, ev_zc = nullptr;
   int device = 0, num_sms = 0;
   std::string err;
   bool whitened = false;
@@ -264,7 +264,6 @@ struct tlda_ctx {
   float g_lr = 0.f;
   const float *g_phi = nullptr;
   int g_loss = -1, g_touch = -1;
-  bool g_host = false;                 // captured for host input
   // event profiler: kernels whose bit is set in prof_mask are bracketed by events
   uint32_t prof_mask = 0;
   struct ProfRec { int id; cudaEvent_t a, b; };
@@ -341,7 +340,7 @@ bool tc_supported(int Dp, int Kp);
 void *tc_make_maps(const __nv_bfloat16 *UX16, const __nv_bfloat16 *ZU16, const __nv_bfloat16 *Z16, int V, int Bmax,
                    int Dp, int Kp);
 void tc_free_maps(void *maps);
-void launch_qy_tc(const StepArgs &a, cudaStream_t s, int part);  // 0: Q rows, 1: Y rows
+void launch_qy_tc(const StepArgs &a, cudaStream_t s);  // without the same-token correction: Y alone
 void launch_zh_tc(const StepArgs &a, cudaStream_t s);
 void launch_h_clear(const StepArgs &a, cudaStream_t s);
 void launch_g_tc(const StepArgs &a, cudaStream_t s);
