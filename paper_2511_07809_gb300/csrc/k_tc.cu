@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(128) k_g_tc(StepArgs a, const __grid_constant_
 // k_zc_tc: one warp per compact slot t (8 per block): row t of ZU16 takes
 // [Zc_t | U_m] in BF16, Zc_t = q (2 c_m q - 2 H_m) with m = widx[t].  Slots
 // in [n_touched, round_up(n_touched, 64)) get zero rows (chunk padding);
-// k_g_tc reads the rows directly.  k_h_clear then clears H_m and c_m for the
-// next batch: a warp that loads an H row and then stores to it (an L2 miss
+// k_g_tc reads the rows directly.  k_h_clear then clears H_m, c_m and the flag
+// for the next batch: a warp that loads an H row and then stores to it (an L2 miss
 // followed by a write to the pending line) ran about six times slower than
 // the load or the store alone.
 template <int NK, bool REP>
@@ -314,7 +314,6 @@ __global__ void __launch_bounds__(256) k_zc_tc(StepArgs a) {
     for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
     if (lane == 0) atomicAdd(&a.st->loss_data, 2.0 * (double)c * (double)ls);
   }
-  if (lane == 0 && m >= 0) a.flag[m] = 0;  // the next batch's words may be looked for
 }
 
 template <int NK>
