@@ -116,29 +116,30 @@ __device__ __forceinline__ bool row_in_batch(const BatchDesc &b, int lo, int hi,
 // Touched words of the batch into widx (compact, no fixed order) with flag set.
 // A word's first meeting in a block goes to its flag, the others end at the
 // block's bitmap (a word that most documents hold would else queue thousands of
-// exchanges at one address: 11.7 us a batch of 4096 tweets).  Flat over the nonzeros, 1024 a
-// block and turn; a word already flagged costs one load, not an atomic; one add
+// exchanges at one address: 11.7 us a batch of 4096 tweets).  Flat over the nonzeros, four
+// a thread of the NT and turn; a word already flagged costs one load, not an atomic; one add
 // to n_touched a block and turn.
 constexpr int kTouchBits = 1 << 17;  // words a block's bitmap holds (16 KB); larger vocabularies do without
+template <int NT>
 __device__ void touch_words(const StepArgs &a, const BatchDesc &b, int *n_touched, int block, int blocks) {
   if (b.n_docs <= 0) return;
   const int lo = b.indptr[0], hi = b.indptr[b.n_docs];
   if (lo < b.nz_base || hi < lo) return;  // corrupt: k_doc / k_scan_whiten report it
-  __shared__ int wsum[8], base;
+  __shared__ int wsum[NT / 32], base;
   __shared__ unsigned seen[kTouchBits / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool small = a.V <= kTouchBits;
-  if ((long long)lo + (long long)block * 1024 >= hi) return;
+  if ((long long)lo + (long long)block * (4 * NT) >= hi) return;
   if (small) {
-    for (int i = tid; i < (a.V + 31) / 32; i += 256) seen[i] = 0;
+    for (int i = tid; i < (a.V + 31) / 32; i += NT) seen[i] = 0;
     __syncthreads();
   }
-  for (long long j0 = (long long)lo + (long long)block * 1024; j0 < hi; j0 += (long long)blocks * 1024) {
+  for (long long j0 = (long long)lo + (long long)block * (4 * NT); j0 < hi; j0 += (long long)blocks * (4 * NT)) {
     int m[4];
     unsigned fresh = 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const long long j = j0 + u * 256 + tid;
+      const long long j = j0 + u * NT + tid;
       m[u] = j < hi ? __ldg(b.indices + (j - b.nz_base)) : -1;
     }
 #pragma unroll
@@ -162,7 +163,7 @@ __device__ void touch_words(const StepArgs &a, const BatchDesc &b, int *n_touche
     if (tid == 0) {
       int t = 0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < NT / 32; ++q) {
         const int x = wsum[q];
         wsum[q] = t;
         t += x;
@@ -179,14 +180,17 @@ __device__ void touch_words(const StepArgs &a, const BatchDesc &b, int *n_touche
 }
 
 __global__ void __launch_bounds__(256) k_touch(StepArgs a) {
-  touch_words(a, a.st->cur, &a.st->n_touched, blockIdx.x, gridDim.x);
+  touch_words<256>(a, a.st->cur, &a.st->n_touched, blockIdx.x, gridDim.x);
 }
 
 // The same for a batch given by value, which becomes the step's batch.
 __global__ void __launch_bounds__(256) k_touch_batch(StepArgs a, BatchDesc b) {
   if (blockIdx.x == 0 && threadIdx.x == 0) a.st->cur = b;
-  touch_words(a, b, &a.st->n_touched, blockIdx.x, gridDim.x);
+  touch_words<256>(a, b, &a.st->n_touched, blockIdx.x, gridDim.x);
 }
+
+// Blocks of 256 threads that find the touched words beside other work (one turn each at 32 nonzeros a document).
+int touch_blocks(const StepArgs &a) { return std::max(64, std::min(2 * a.sms, a.Bmax / 32)); }
 
 void launch_touch(const StepArgs &a, cudaStream_t s) { k_touch<<<2 * a.sms, 256, 0, s>>>(a); }
 void launch_touch_batch(const StepArgs &a, const BatchDesc &b, cudaStream_t s) {
@@ -221,18 +225,21 @@ __device__ __forceinline__ void add_rows(const NzChunk &c, int q, const float *U
 // One warp per document: validates the row, accumulates L_d and
 // x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, adds c_m to this
 // block's copy and the block's share of S3.  TC=true writes X in BF16 row-major
-// (X16), whole rows, else in FP32.
+// (X16), whole rows, else in FP32.  The first `touch` blocks (FP32 only) find the
+// batch's touched words meanwhile: the product after this kernel reads them.
 template <int NV, bool TC>
-__global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a) {
+__global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a, int touch) {
   const BatchDesc b = a.st->cur;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int d0 = blockIdx.x * kDocsPerBlock;
+  if constexpr (!TC)
+    if ((int)blockIdx.x < touch) return touch_words<32 * kDocsPerBlock>(a, b, &a.st->n_touched, blockIdx.x, touch);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, block = blockIdx.x - touch;
+  const int d0 = block * kDocsPerBlock;
   if (d0 >= (TC ? round_up(b.n_docs, 64) : b.n_docs)) return;
   const int d = d0 + warp;
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
   __syncthreads();
-  int *cnt = a.cnt + (long long)(blockIdx.x % a.nrep) * a.V;
+  int *cnt = a.cnt + (long long)(block % a.nrep) * a.V;
   float4 acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
@@ -283,12 +290,13 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a) 
 
 void launch_whiten(const StepArgs &a, cudaStream_t s) {
   const bool tc = a.precision == TLDA_BF16;
-  const int grid = round_up(a.Bmax, 64) / kDocsPerBlock;
+  const int touch = !tc && a.same_token ? touch_blocks(a) * 256 / (32 * kDocsPerBlock) : 0;
+  const int grid = touch + round_up(a.Bmax, 64) / kDocsPerBlock;
   const int nv = (a.Dp + 127) / 128;
 #define TLDA_WHITEN(NVv)                                                              \
   if (nv == NVv) {                                                                    \
-    if (tc) k_scan_whiten<NVv, true><<<grid, 32 * kDocsPerBlock, 0, s>>>(a);          \
-    else k_scan_whiten<NVv, false><<<grid, 32 * kDocsPerBlock, 0, s>>>(a);            \
+    if (tc) k_scan_whiten<NVv, true><<<grid, 32 * kDocsPerBlock, 0, s>>>(a, touch);   \
+    else k_scan_whiten<NVv, false><<<grid, 32 * kDocsPerBlock, 0, s>>>(a, touch);     \
     return;                                                                           \
   }
   TLDA_WHITEN(1) TLDA_WHITEN(2) TLDA_WHITEN(3) TLDA_WHITEN(4)
@@ -1249,7 +1257,7 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
   DevState *st = a.st;
   const int entry_blocks = (a.D * a.K + 31) / 32;
   if ((int)blockIdx.x >= entry_blocks && st->descs && st->pass_pos < st->n_descs)
-    touch_words(a, st->descs[st->pass_pos], &st->n_touched_next, blockIdx.x - entry_blocks, a.touch_next);
+    touch_words<256>(a, st->descs[st->pass_pos], &st->n_touched_next, blockIdx.x - entry_blocks, a.touch_next);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
   const unsigned long long S3 = st->S3;

@@ -153,16 +153,11 @@ struct Prof {
 // The FP32 form without the loss takes its data term regrouped by word.
 bool by_word(const StepArgs &a) { return a.precision == TLDA_FP32 && !a.want_loss; }
 
-// Whether a step needs the touched words.
-bool wants_touch(const tlda_ctx *ctx, const StepArgs &a) {
-  return !(a.precision == TLDA_BF16 && ctx->fused) && (by_word(a) || a.same_token);
-}
-
 // Enqueues one CP step on ctx->stream for the batch in st->cur: the Phi-only
 // terms on the side stream, the data-term chain on the main stream, then the
 // reduction and update once both are done.
 // With `touched`, the batch's touched words are there already (an earlier step's
-// reduction kernel or the caller found them; FP32 only).
+// reduction kernel or the caller found them; by_word only).
 tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touched = false) {
   const bool tc = a.precision == TLDA_BF16;
   auto fork_phi = [&]() -> tlda_status {
@@ -208,7 +203,6 @@ tlda_status enqueue_step(tlda_ctx *ctx, StepArgs a, cudaStream_t main, bool touc
     { Prof p(ctx, kRZ, main); launch_doc(a, main); }
     { Prof p(ctx, kG, main); launch_gw_f32(a, main); }
   } else {
-    if (!tc && a.same_token && !touched) { Prof p(ctx, kWhiten, main); launch_touch(a, main); }
     { Prof p(ctx, kWhiten, main); launch_whiten(a, main); }
     { Prof p(ctx, kQY, main); if (tc) launch_qy_tc(a, main); else launch_qy_f32(a, main); }
     { Prof p(ctx, kRZ, main); launch_rz(a, main); }
@@ -829,7 +823,7 @@ static tlda_status step_common(tlda_ctx *ctx, const tlda_csr *batch, float *Phi,
   a.gdata_out = gdata_out;
   a.mode = mode;
   a.want_loss = loss_out ? 1 : 0;
-  const bool touch = a.precision == TLDA_FP32 && wants_touch(ctx, a);  // the BF16 chain finds them beside its other work
+  const bool touch = by_word(a);  // the other forms find the touched words beside their other work
   if (touch) launch_touch_batch(a, desc_of(batch), ctx->stream);
   else launch_set_desc(ctx->st, desc_of(batch), ctx->stream);
   if (a.PhiImg) launch_phi_img(a, ctx->stream);
@@ -934,15 +928,32 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
   if (loss_out && !no_wait) CK(cudaMallocHost(reinterpret_cast<void **>(&losses), sizeof(double) * n_batches));
   launch_begin_pass(ctx->st, ctx->descs, n_batches, ps);
   if (a.PhiImg) launch_phi_img(a, ps);
-  // FP32, device input: each step's reduction kernel finds the next batch's
-  // touched words beside its own work, the first batch's are found here (with host
-  // input the next batch is copied only after the step; the BF16 chain has a side
-  // stream to find them on, where the reduction would wait for them: 4.26 against
-  // 3.98 ms a pass of 103 batches of 1936 to 3873 documents at K = 26)
-  const bool ahead = !host && by_word(a);
+  // Host input: a batch's copy on the pass's stream, into the slot that the step
+  // two batches before read last, earlier on that stream.
+  auto copy_batch = [&](int b) -> tlda_status {
+    const int64_t d0 = batch_offsets[b], d1 = batch_offsets[b + 1];
+    const long long lo = corpus->indptr[d0], hi = corpus->indptr[d1];
+    const BatchDesc &d = hd[b];
+    CK(cudaMemcpyAsync(const_cast<int32_t *>(d.indptr), corpus->indptr + d0, sizeof(int32_t) * (d1 - d0 + 1),
+                       cudaMemcpyHostToDevice, ps));
+    if (hi > lo) {
+      CK(cudaMemcpyAsync(const_cast<int32_t *>(d.indices), corpus->indices + lo, sizeof(int32_t) * (hi - lo),
+                         cudaMemcpyHostToDevice, ps));
+      CK(cudaMemcpyAsync(const_cast<int32_t *>(d.counts), corpus->counts + lo, sizeof(int32_t) * (hi - lo),
+                         cudaMemcpyHostToDevice, ps));
+    }
+    return TLDA_OK;
+  };
+  // FP32 by word: each step's reduction kernel finds the next batch's touched words
+  // beside its own work, the first batch's are found here; host input is copied one
+  // batch ahead of the step for this.  With the loss the whitening kernel finds them,
+  // and the BF16 chain has a side stream, where the reduction would wait for them:
+  // 4.26 against 3.98 ms a pass of 103 batches of 1936 to 3873 documents at K = 26.
+  const bool ahead = by_word(a);
   if (ahead) {
-    a.touch_next = std::max(64, std::min(2 * ctx->num_sms, ctx->Bmax / 32));  // 32 nonzeros a document: one turn each
-    launch_touch(a, ps);
+    if (host) s = copy_batch(0);
+    a.touch_next = touch_blocks(a);
+    if (s == TLDA_OK) launch_touch(a, ps);
   }
   CKL();
   // one captured step, replayed per batch (not while the event profiler is on)
@@ -972,18 +983,9 @@ tlda_status tlda_cp_pass(tlda_ctx *ctx, const tlda_csr *corpus, const int64_t *b
   }
   for (int b = 0; b < n_batches && s == TLDA_OK; ++b) {
     if (host) {
-      // the slot was last read by step b-2, earlier on the same stream
-      const int64_t d0 = batch_offsets[b], d1 = batch_offsets[b + 1];
-      const long long lo = corpus->indptr[d0], hi = corpus->indptr[d1];
-      const BatchDesc &d = hd[b];
-      CK(cudaMemcpyAsync(const_cast<int32_t *>(d.indptr), corpus->indptr + d0, sizeof(int32_t) * (d1 - d0 + 1),
-                         cudaMemcpyHostToDevice, ps));
-      if (hi > lo) {
-        CK(cudaMemcpyAsync(const_cast<int32_t *>(d.indices), corpus->indices + lo, sizeof(int32_t) * (hi - lo),
-                           cudaMemcpyHostToDevice, ps));
-        CK(cudaMemcpyAsync(const_cast<int32_t *>(d.counts), corpus->counts + lo, sizeof(int32_t) * (hi - lo),
-                           cudaMemcpyHostToDevice, ps));
-      }
+      const int next = ahead ? b + 1 : b;
+      if (next < n_batches) s = copy_batch(next);
+      if (s) break;
     }
     if (use_graph) CK(cudaGraphLaunch(ctx->step_exec, ps));
     else s = enqueue_step(ctx, a, ps, ahead);

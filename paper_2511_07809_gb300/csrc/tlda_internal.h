@@ -285,6 +285,7 @@ void launch_set_desc(DevState *st, const BatchDesc &b, cudaStream_t s);
 void launch_begin_pass(DevState *st, const BatchDesc *descs, int n, cudaStream_t s);
 void launch_whiten(const StepArgs &a, cudaStream_t s);
 void launch_whiten_out(const StepArgs &a, const BatchDesc &b, cudaStream_t s, float *X);
+int touch_blocks(const StepArgs &a);
 void launch_touch(const StepArgs &a, cudaStream_t s);
 void launch_touch_batch(const StepArgs &a, const BatchDesc &b, cudaStream_t s);
 void launch_q_f32(const StepArgs &a, cudaStream_t s);
