@@ -1262,7 +1262,15 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
   const int e = blockIdx.x * 32 + lane;
   const unsigned long long S3 = st->S3;
   const int err = st->err;
-  const double scale = S3 ? a.c3 / (double)S3 : 0.0;
+  // what the end of the step needs besides, requested now by the thread that may do it
+  const bool ends = threadIdx.x == 32;
+  const BatchDesc *descs = nullptr;
+  int pos = 0, n_descs = 0, step = 0;
+  double loss_phi = 0.0, loss_data = 0.0;
+  if (ends) {
+    descs = st->descs, pos = st->pass_pos, n_descs = st->n_descs, step = st->step;
+    loss_phi = st->loss_phi, loss_data = st->loss_data;
+  }
   const bool live = (int)blockIdx.x < entry_blocks && e < a.D * a.K;
   const int i = live ? e / a.K : 0, n = live ? e % a.K : 0;
   const long long off = (long long)i * a.Kp + n, stride = (long long)a.Dp * a.Kp;
@@ -1278,6 +1286,10 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) part += acc[u];
   }
+  const double scale = S3 ? a.c3 / (double)S3 : 0.0;
+  const bool more = descs && pos < n_descs;
+  BatchDesc next{};
+  if (more) next = descs[pos];
   __shared__ float red[8][32];
   red[w][lane] = part;
   __syncthreads();
@@ -1299,21 +1311,24 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
     }
   }
   // the last block to get here (every block has read the step's sums) ends the
-  // step: its loss, the sums cleared for the next batch, the step counter, and
-  // the next batch descriptor of a pass
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(&st->done, 1u) == gridDim.x - 1) {
-      __threadfence();
+  // step, beside its update: its loss, the sums cleared for the next batch, the step
+  // counter, and the next batch descriptor of a pass
+  if (ends) {
+    unsigned before;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(&st->done) : "memory");
+    if (before == gridDim.x - 1) {
+      st->n_touched = __ldcg(&st->n_touched_next);
+      st->n_touched_next = 0;
       st->done = 0;
-      st->loss = S3 ? st->loss_phi - scale * st->loss_data : 0.0;
+      st->loss = S3 ? loss_phi - scale * loss_data : 0.0;
       st->last_S3 = S3;
       st->S3 = 0;
       st->loss_data = 0.0;
-      st->n_touched = st->n_touched_next;
-      st->n_touched_next = 0;
-      st->step += 1;
-      if (st->descs && st->pass_pos < st->n_descs) st->cur = st->descs[st->pass_pos++];
+      st->step = step + 1;
+      if (more) {
+        st->cur = next;
+        st->pass_pos = pos + 1;
+      }
     }
   }
 }
