@@ -29,7 +29,7 @@
 // H (or B) and c take one add per nonzero.  A word that most documents hold
 // (the head of a Zipf vocabulary) would queue every document's add at one
 // address, so small tables are kept nrep times (StepArgs::nrep): a block adds
-// to one copy, and the reader sums them.
+// to one copy, and the reader sums them (batches of few documents use one).
 #include <algorithm>
 #include <cstdio>
 
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a, 
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
   __syncthreads();
-  int *cnt = a.cnt + (long long)(block % a.nrep) * a.V;
+  int *cnt = a.cnt + (long long)(block % copies(a, b.n_docs)) * a.V;
   float4 acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
                                          : f4(0.f);
     r[v] = f4(0.f);
   }
-  float *H = a.H32 + (long long)(blockIdx.x % a.nrep) * a.V * a.Kp;
+  float *H = a.H32 + (long long)(blockIdx.x % copies(a, b.n_docs)) * a.V * a.Kp;
   if (a.same_token && d < b.n_docs) {
     const int lo = b.indptr[d], hi = b.indptr[d + 1];
     if (row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs])) {
@@ -637,17 +637,16 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
   }
 }
 
-// c_m and four columns of H_m (or B_m), summed over the copies.
-__device__ __forceinline__ int word_count(const StepArgs &a, int m) {
+// c_m and four columns of H_m (or B_m), summed over the nrep copies in use.
+__device__ __forceinline__ int word_count(const StepArgs &a, int nrep, int m) {
   int c = a.cnt[m];
-  if (a.nrep > 1)
-    for (int r = 1; r < a.nrep; ++r) c += a.cnt[(long long)r * a.V + m];
+  for (int r = 1; r < nrep; ++r) c += a.cnt[(long long)r * a.V + m];
   return c;
 }
-__device__ __forceinline__ float4 word_sum(const StepArgs &a, int m, int col) {
+__device__ __forceinline__ float4 word_sum(const StepArgs &a, int nrep, int m, int col) {
   const float4 *p = reinterpret_cast<const float4 *>(a.H32 + (long long)m * a.Kp + col);
   float4 h = *p;
-  for (int r = 1; r < a.nrep; ++r) {
+  for (int r = 1; r < nrep; ++r) {
     const float4 x = p[(long long)r * a.V * (a.Kp / 4)];
     h = make_float4(h.x + x.x, h.y + x.y, h.z + x.z, h.w + x.w);
   }
@@ -663,8 +662,8 @@ __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + warp;
   if (t >= a.st->n_touched) return;
-  const int m = a.widx[t];
-  const float c = (float)word_count(a, m);
+  const int m = a.widx[t], nrep = copies(a, a.st->cur.n_docs);
+  const float c = (float)word_count(a, nrep, m);
   float ls = 0.f;
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
@@ -672,11 +671,11 @@ __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
     if (col < a.Kp) {
       float4 *hp = reinterpret_cast<float4 *>(a.H32 + (long long)m * a.Kp + col);
       const float4 q = *reinterpret_cast<const float4 *>(a.Q32 + (long long)m * a.Kp + col);
-      const float4 h = word_sum(a, m, col);
+      const float4 h = word_sum(a, nrep, m, col);
       const float4 z = make_float4(q.x * (2.f * c * q.x - 2.f * h.x), q.y * (2.f * c * q.y - 2.f * h.y),
                                    q.z * (2.f * c * q.z - 2.f * h.z), q.w * (2.f * c * q.w - 2.f * h.w));
       *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = z;
-      for (int r = 0; r < a.nrep; ++r) hp[(long long)r * a.V * (a.Kp / 4)] = f4(0.f);
+      for (int r = 0; r < nrep; ++r) hp[(long long)r * a.V * (a.Kp / 4)] = f4(0.f);
       ls += q.x * q.x * q.x + q.y * q.y * q.y + q.z * q.z * q.z + q.w * q.w * q.w;
     }
   }
@@ -686,7 +685,7 @@ __global__ void __launch_bounds__(256) k_zh_f32(StepArgs a) {
   }
   __syncwarp();
   if (lane == 0) {
-    for (int r = 0; r < a.nrep; ++r) a.cnt[(long long)r * a.V + m] = 0;
+    for (int r = 0; r < nrep; ++r) a.cnt[(long long)r * a.V + m] = 0;
     a.flag[m] = 0;
   }
 }
@@ -938,7 +937,7 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LW, sl = lane % LW;
   const int K4 = (a.K + 3) & ~3;  // the padding columns are zero and stay so
   float *rows = doc_rows + (long long)warp * R * K4;
-  float *B = a.H32 + (long long)(blockIdx.x % a.nrep) * a.V * a.Kp;
+  float *B = a.H32 + (long long)(blockIdx.x % copies(a, b.n_docs)) * a.V * a.Kp;
   const int first = b.indptr[0], last = b.indptr[b.n_docs];
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
@@ -1088,7 +1087,7 @@ __global__ void __launch_bounds__(256) k_b_fold(StepArgs a) {
   for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
     const int m = a.widx[t];
     for (int col = lane * 4; col < a.Kp; col += 128)
-      *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = word_sum(a, m, col);
+      *reinterpret_cast<float4 *>(a.Zc32 + (long long)t * a.Kp + col) = word_sum(a, copies(a, a.st->cur.n_docs), m, col);
   }
 }
 
@@ -1099,7 +1098,7 @@ __global__ void __launch_bounds__(256) k_b_clear(StepArgs a) {
   const int lane = threadIdx.x & 31;
   for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
     const int m = a.widx[t];
-    for (int r = 0; r < a.nrep; ++r)
+    for (int r = 0; r < copies(a, a.st->cur.n_docs); ++r)
       for (int col = lane * 4; col < a.Kp; col += 128)
         *reinterpret_cast<float4 *>(a.H32 + ((long long)r * a.V + m) * a.Kp + col) = f4(0.f);
     if (lane == 0) a.flag[m] = 0;
@@ -1119,7 +1118,7 @@ template <int BI, int BN, int TM, bool FOLD>
 __global__ void __launch_bounds__(BI / TM * (BN / 4)) k_gw_f32(StepArgs a, int stages) {
   constexpr int TN = 4, TX = BN / TN, NT = BI / TM * TX, BR = kGwRows;
   extern __shared__ __align__(16) float gw_sm[];
-  const int reps = FOLD ? a.nrep : 1, stage = BR * (BI + reps * BN);
+  const int reps = FOLD ? copies(a, a.st->cur.n_docs) : 1, stage = BR * (BI + reps * BN);  // at most the host's
   const int nt = a.st->n_touched, tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int s = blockIdx.x, i0 = blockIdx.y * BI, n0 = blockIdx.z * BN;
   const int rb = (int)((long long)nt * s / a.nsplit), re = (int)((long long)nt * (s + 1) / a.nsplit);

@@ -276,9 +276,10 @@ __global__ void __launch_bounds__(256) k_zc_tc(StepArgs a) {
   const int t = blockIdx.x * 8 + warp, nt = a.st->n_touched;
   if (t >= round_up(nt, 64)) return;  // per warp: no block barrier follows
   const int m = t < nt ? a.widx[t] : -1;
+  const int nrep = REP ? copies(a, a.st->cur.n_docs) : 1;
   int cs = m >= 0 ? a.cnt[m] : 0;
   if (REP && m >= 0)
-    for (int r = 1; r < a.nrep; ++r) cs += a.cnt[(long long)r * a.V + m];
+    for (int r = 1; r < nrep; ++r) cs += a.cnt[(long long)r * a.V + m];
   const float c = (float)cs;
   __nv_bfloat16 *row = a.ZU16 + (long long)t * (a.Kp + a.Dp);
   float ls = 0.f;
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(256) k_zc_tc(StepArgs a) {
         const float4 *hp = reinterpret_cast<const float4 *>(a.H32 + (long long)m * a.Kp + col);
         const float4 q = *reinterpret_cast<const float4 *>(a.Q32 + (long long)m * a.Kp + col);
         float4 h = *hp;
-        if constexpr (REP) for (int r = 1; r < a.nrep; ++r) {
+        if constexpr (REP) for (int r = 1; r < nrep; ++r) {
           const float4 x = hp[(long long)r * a.V * (a.Kp / 4)];
           h = make_float4(h.x + x.x, h.y + x.y, h.z + x.z, h.w + x.w);
         }
@@ -321,16 +322,16 @@ __global__ void __launch_bounds__(256) k_h_clear(StepArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + warp;
   if (t >= a.st->n_touched) return;
-  const int m = a.widx[t];
+  const int m = a.widx[t], nrep = copies(a, a.st->cur.n_docs);
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
     const int col = v * 128 + lane * 4;
     if (col < a.Kp)
-      for (int r = 0; r < a.nrep; ++r)
+      for (int r = 0; r < nrep; ++r)
         *reinterpret_cast<float4 *>(a.H32 + ((long long)r * a.V + m) * a.Kp + col) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   if (lane == 0) {
-    for (int r = 0; r < a.nrep; ++r) a.cnt[(long long)r * a.V + m] = 0;
+    for (int r = 0; r < nrep; ++r) a.cnt[(long long)r * a.V + m] = 0;
     a.flag[m] = 0;
   }
 }
