@@ -35,6 +35,8 @@
 
 #include <cstdint>
 
+#include "smem_limit.h"
+
 namespace {
 
 constexpr int kG64Tile = 64;     // rows and columns of C per block
@@ -313,9 +315,8 @@ __global__ void __launch_bounds__(256, 1) k_gemm64(const TA *A, int lda, const T
 template <bool AKROWS, bool ADD, bool SYM, class TA, class TB>
 void g64_launch(const TA *A, int lda, const TB *B, int ldb, double *C, int ldc, int M, int N, int Kd, int splits,
                 const int *eA, const int *eB, const int *ck, cudaStream_t s) {
-  static const cudaError_t attr = cudaFuncSetAttribute(k_gemm64<AKROWS, ADD, SYM, TA, TB>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, g64_smem<TA, TB>());
-  (void)attr;
+  static tlda::SmemLimit lim;
+  lim.raise((const void *)k_gemm64<AKROWS, ADD, SYM, TA, TB>, g64_smem<TA, TB>());
   const int folds = (Kd + kG64Fold - 1) / kG64Fold, per = (folds + splits - 1) / splits;
   const dim3 g((N + kG64Tile - 1) / kG64Tile, (M + kG64Tile - 1) / kG64Tile, (folds + per - 1) / per);
   k_gemm64<AKROWS, ADD, SYM, TA, TB><<<g, 256, g64_smem<TA, TB>(), s>>>(A, lda, B, ldb, C, ldc, M, N, Kd, per * kG64Fold, eA, eB, ck);

@@ -197,10 +197,9 @@ int sgemm_splits(int M, int N, int Kd, int sms) {
 template <int TM, int TN>
 void sgemm_launch(const float *A, int lda, const float *B, int ldb, float *out, int M, int N, int Kd, int chunk, int splits,
                   cudaStream_t s) {
-  static const cudaError_t attr[2] = {
-      cudaFuncSetAttribute(k_sgemm<TM, TN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sgemm_smem<TM, TN>()),
-      cudaFuncSetAttribute(k_sgemm<TM, TN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sgemm_smem<TM, TN>())};
-  (void)attr;
+  static SmemLimit lim[2];
+  lim[0].raise((const void *)k_sgemm<TM, TN, true>, sgemm_smem<TM, TN>());
+  lim[1].raise((const void *)k_sgemm<TM, TN, false>, sgemm_smem<TM, TN>());
   const dim3 g((N + 16 * TN - 1) / (16 * TN), (M + 16 * TM - 1) / (16 * TM), splits);
   const bool wide = lda % 4 == 0 && Kd % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;  // chunk is a multiple of 32
   if (wide) k_sgemm<TM, TN, true><<<g, 256, sgemm_smem<TM, TN>(), s>>>(A, lda, B, ldb, out, N, M, N, Kd, chunk, (long long)M * N);

@@ -1216,11 +1216,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_pass(StepArgs a, PassArgs 
 bool fused_supported(int Dp, int Kp) { return Dp == 128 && Kp == 128; }
 
 void launch_fused(const StepArgs &a, cudaStream_t s, int grid) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem);
-    attr = true;
-  }
+  static SmemLimit lim;
+  lim.raise((const void *)k_fused, kFusedSmem);
   k_fused<<<grid, kFusedThreads, kFusedSmem, s>>>(a);
 }
 

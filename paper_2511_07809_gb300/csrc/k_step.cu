@@ -910,9 +910,8 @@ void launch_q_f32(const StepArgs &a, cudaStream_t s) {
 #define TLDA_Q(TNv, blocks)                                                                               \
   {                                                                                                       \
     const int smem = (kQRows * (kQDeep + 4) + deep * 16 * TNv) * (int)sizeof(float);                          \
-    static const cudaError_t attr = cudaFuncSetAttribute(                                                 \
-        k_q_f32<TNv>, cudaFuncAttributeMaxDynamicSharedMemorySize, (kQRows * (kQDeep + 4) + kQDeep * 16 * TNv) * 4); \
-    (void)attr;                                                                                           \
+    static SmemLimit lim;                                                                                 \
+    lim.raise((const void *)k_q_f32<TNv>, (kQRows * (kQDeep + 4) + kQDeep * 16 * TNv) * 4);               \
     k_q_f32<TNv><<<std::min(blocks * a.sms, rt * ((a.Kp + 16 * TNv - 1) / (16 * TNv))), kQThreads, smem, s>>>(a); \
   }
   if (a.Kp <= 64) TLDA_Q(4, 3)
@@ -1066,9 +1065,8 @@ void launch_doc(const StepArgs &a, cudaStream_t s) {
   const int grid = std::max(1, std::min((a.Bmax + 7) / 8, 4 * a.sms));
 #define TLDA_DOC(NKv, LWv)                                                                                     \
   {                                                                                                            \
-    static const cudaError_t attr =                                                                            \
-        cudaFuncSetAttribute(k_doc<NKv, LWv>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kDocBytes);     \
-    (void)attr;                                                                                                \
+    static SmemLimit lim;                                                                                      \
+    lim.raise((const void *)k_doc<NKv, LWv>, 8 * kDocBytes);                                                   \
     k_doc<NKv, LWv><<<grid, 256, smem, s>>>(a, R);                                                             \
   }
   if (K4 <= 32) TLDA_DOC(1, 8)
@@ -1225,9 +1223,8 @@ template <int BI, int BN, int TM, bool FOLD>
 void gw_launch(const StepArgs &a, dim3 grid, cudaStream_t s) {
   const int stage = kGwRows * (BI + (FOLD ? a.nrep : 1) * BN) * (int)sizeof(float);
   const int stages = std::max(2, std::min(6, 98304 / stage));
-  static const cudaError_t attr = cudaFuncSetAttribute(k_gw_f32<BI, BN, TM, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       147456);
-  (void)attr;
+  static SmemLimit lim;
+  lim.raise((const void *)k_gw_f32<BI, BN, TM, FOLD>, 147456);
   k_gw_f32<BI, BN, TM, FOLD><<<grid, BI / TM * (BN / 4), stages * stage, s>>>(a, stages);
 }
 

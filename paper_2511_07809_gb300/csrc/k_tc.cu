@@ -384,21 +384,15 @@ int tc_smem() {
 
 template <int KP>
 void qy_launch(const StepArgs &a, const TcMaps &m, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_qy_tc<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<KP>());
-    attr = true;
-  }
+  static SmemLimit lim;
+  lim.raise((const void *)k_qy_tc<KP>, tc_smem<KP>());
   k_qy_tc<KP><<<((a.same_token ? a.V : 0) + a.Bmax + 127) / 128, 128, tc_smem<KP>(), s>>>(a, m.ux);
 }
 
 template <int KP>
 void g_launch(const StepArgs &a, const TcMaps &m, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_g_tc<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<KP>());
-    attr = true;
-  }
+  static SmemLimit lim;
+  lim.raise((const void *)k_g_tc<KP>, tc_smem<KP>());
   k_g_tc<KP><<<dim3(a.nsplit, (a.Dp + 127) / 128), 128, tc_smem<KP>(), s>>>(a, m.gx, m.gu, m.gz, m.gc);
 }
 

@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "smem_limit.h"
 #include "tlda.h"
 
 #include <nvtx3/nvToolsExt.h>
