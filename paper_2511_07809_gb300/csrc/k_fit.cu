@@ -207,16 +207,21 @@ void sgemm_launch(const float *A, int lda, const float *B, int ldb, float *out, 
 }
 
 // part: splits x M x N floats when there is more than one split (C then is M x N).
-// Unsplit products (few terms) take tiles of 32 rows, for more blocks.
+// Products of few terms (Q L^-T, at most kMaxRitz) take tiles of 32 rows, for more
+// blocks; with many terms 128 rows are ahead also where they are not split (the
+// fit's milliseconds in 32-row tiles and these: V = 30,000 and D = 100 310 -> 241,
+// V = 20,000 and D = 40 89.2 -> 85.8, V = 12,000 and D = 150 86.0 -> 84.8; V =
+// 20,000 and D = 100, five tiles more than SMs, 155.0 -> 155.5).
 void sgemm(const float *A, int lda, const float *B, int ldb, float *C, int M, int N, int Kd, float *part, int splits,
            cudaStream_t s) {
   const int nt = (N + 127) / 128, tn = (N + 16 * nt - 1) / (16 * nt);
   const int chunk = ((Kd + splits - 1) / splits + kSgBk - 1) / kSgBk * kSgBk;
   splits = (Kd + chunk - 1) / chunk;
   float *out = splits > 1 ? part : C;
+  const bool tall = Kd >= 2 * kMaxDim || splits > 1;
 #define TLDA_SGEMM(TNv)                                                                         \
   case TNv:                                                                                     \
-    if (splits > 1) sgemm_launch<8, TNv>(A, lda, B, ldb, out, M, N, Kd, chunk, splits, s);      \
+    if (tall) sgemm_launch<8, TNv>(A, lda, B, ldb, out, M, N, Kd, chunk, splits, s);            \
     else sgemm_launch<2, TNv>(A, lda, B, ldb, out, M, N, Kd, chunk, splits, s);                 \
     break;
   switch (tn) {
