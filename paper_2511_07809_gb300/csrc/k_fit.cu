@@ -31,6 +31,7 @@ using namespace tlda;
 namespace {
 
 constexpr int kMaxFitV = 65536;
+constexpr size_t kKeepTopics = size_t(32) << 20;   // bytes of topics that a context keeps room for
 constexpr int kOversample = 16;                    // columns of the fit's subspace beyond D
 constexpr int kMaxRitz = kMaxDim + kOversample;    // largest order of the dense FP64 kernels
 
@@ -1981,7 +1982,8 @@ tlda_status tlda_unwhiten_topics(tlda_ctx *ctx, const float *Phi, double *mu_out
   double *G = nullptr, *Linv = nullptr, *LinvT = nullptr, *T1 = nullptr, *T = nullptr, *sum = nullptr, *n2 = nullptr;
   double *Lf = nullptr, *Zs = nullptr, *mu = nullptr, *al = nullptr;
   int *status = nullptr;
-  const size_t DD = (size_t)D * D;
+  const size_t DD = (size_t)D * D, topics = sizeof(double) * V * K;
+  const bool keep = topics <= kKeepTopics;
   auto lay = [&](Carver &c) {
     c.take(G, DD);
     c.take(Linv, DD);
@@ -1994,10 +1996,10 @@ tlda_status tlda_unwhiten_topics(tlda_ctx *ctx, const float *Phi, double *mu_out
     c.take(n2, K);
     c.take(status, 1);
     c.take(al, K);
-    c.take(mu, host ? (size_t)V * K : 1);
+    if (host && keep) c.take(mu, (size_t)V * K);
   };
-  // the context keeps this workspace (V K doubles with host output): an
-  // allocation and its release took 150 us of each call
+  // the context keeps this workspace, with the topics of a host output up to
+  // kKeepTopics: an allocation and its release took 150 us of each call
   Carver need{nullptr};
   lay(need);
   if (ctx->uw_bytes < need.off) {
@@ -2008,6 +2010,8 @@ tlda_status tlda_unwhiten_topics(tlda_ctx *ctx, const float *Phi, double *mu_out
   }
   Carver real{ctx->uw_ws};
   lay(real);
+  Scratch large;  // larger topics go with the call, which copies them for longer than that
+  if (host && !keep) CKF(large.carve([&](Carver &c) { c.take(mu, (size_t)V * K); }));
   if (!host) {
     mu = mu_out;
     al = alpha_out;

@@ -248,7 +248,7 @@ struct tlda_ctx {
   float *on_Om32 = nullptr;            // V x r: FP32 copy of Omega for the sketch's products
   int *on_status = nullptr;            // its device status words
   int jacobi_sweeps = 0;               // sweeps of the last symmetric eigensolve
-  char *uw_ws = nullptr;               // workspace of tlda_unwhiten_topics
+  char *uw_ws = nullptr;               // workspace of tlda_unwhiten_topics (bounded, see there)
   size_t uw_bytes = 0;
   int *g64_exp = nullptr;              // operand exponents of the FP64 products (V rows, two sets of columns)
   void *coop_ctl = nullptr;            // control block of the grid-wide FP64 kernels (k_fit.cu)
