@@ -11,11 +11,13 @@
 // each exact in BF16.  A product of digits is at most 2^14 in magnitude; the
 // digit products of equal order s = i + j are added in one FP32 accumulator,
 // at most 7 of them over 128 terms, below 2^24: every sum is exact, whatever
-// the order in which the tensor core adds.  After each 128 terms the seven
-// accumulators of an entry are folded into two 64-bit integers, and at the end
-// into one FP64 value.  Orders s > 6 are dropped: per term they are at most
-// 2^-53 of 2^(eA+eB) and of either sign, no more than the rounding of an FP64
-// sum of such terms.
+// the order in which the tensor core adds.  After each 128 terms the eight
+// accumulators of an entry are folded into two 64-bit integers (order 7 rounded
+// to order 6's unit), and at the end into one FP64 value.  Orders s > 7 are
+// dropped: per term they are at most 2^-61 of 2^(eA+eB).  Order 7 counts: in
+// W^T W of a Zipf vocabulary, whose columns have few large entries, its sum was
+// 5e-15 of the result (plain FP64 4e-16, with it 2e-16; 28 digit products a term
+// without it, 34 with it).
 //
 // C = A B sums over columns of A that may differ in scale by many powers of two
 // with rows of B the other way round (a whitening and its pseudo-inverse: an
@@ -24,8 +26,8 @@
 // column's largest magnitude, so that the slices are relative to the terms.
 //
 // What bounds it, and why: GB300 issues 2 FP64 FMAs a clock per SM (1.2
-// TFLOP/s), where the tensor cores take the 28 digit products of a term far
-// faster.  Tiles of 64 x 64 by 8 warps (16 x 32 each: 112 accumulators and 32
+// TFLOP/s), where the tensor cores take the 34 digit products of a term far
+// faster.  Tiles of 64 x 64 by 8 warps (16 x 32 each: 128 accumulators and 32
 // 64-bit sums a thread); the raw operands come by cp.async one 32-term slab
 // ahead of the products, and are cut into digits in shared memory.
 #pragma once
@@ -43,6 +45,7 @@ constexpr int kG64Tile = 64;     // rows and columns of C per block
 constexpr int kG64Slab = 32;     // terms per shared-memory slab
 constexpr int kG64Fold = 128;    // terms per exact FP32 sum
 constexpr int kG64Dig = 7;
+constexpr int kG64Ord = 8;       // orders of digit products that are summed
 constexpr int kG64Ld = kG64Slab + 8;                       // digit row, in BF16 (80 bytes: conflict-free ldmatrix)
 constexpr int kG64DigBytes = kG64Dig * kG64Tile * kG64Ld * 2;  // one operand's digits of a slab
 constexpr int kG64RawLd = kG64Tile + 1;                    // raw slab row (terms x tile), in elements
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm64(const TA *A, int lda, const T
   if (tid < 64) ea[tid] = m0 + tid < M ? eA[m0 + tid] : 0;
   else if (tid < 128) eb[tid - 64] = n0 + tid - 64 < N ? eB[n0 + tid - 64] : 0;
   const bool live = m0 + wm < M && n0 + wn < N;
-  float acc[kG64Dig][4][4];
+  float acc[kG64Ord][4][4];
   long long hi[4][4], lo[4][4];
 #pragma unroll
   for (int j = 0; j < 4; ++j)
@@ -226,7 +229,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm64(const TA *A, int lda, const T
     for (int q = 0; q < 4; ++q) {
       hi[j][q] = lo[j][q] = 0;
 #pragma unroll
-      for (int s = 0; s < kG64Dig; ++s) acc[s][j][q] = 0.f;
+      for (int s = 0; s < kG64Ord; ++s) acc[s][j][q] = 0.f;
     }
   g64_load<AKROWS>(rawA, A, lda, m0, M, kb, ke);
   g64_load<true>(rawB, B, ldb, n0, N, kb, ke);
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm64(const TA *A, int lda, const T
         g64_ldsm4(b0, bj);
         g64_ldsm4(b1, bj + 16 * kG64Ld * 2);
 #pragma unroll
-        for (int i = 0; i + j < kG64Dig; ++i) {
+        for (int i = 0; i < kG64Dig && i + j < kG64Ord; ++i) {
           uint32_t a[4];
           g64_ldsm4(a, sA + aoff + (uint32_t)(i * kG64Tile * kG64Ld + kk) * 2);
           g64_mma(acc[i + j][0], a, b0[0], b0[1]);
@@ -282,9 +285,10 @@ __global__ void __launch_bounds__(256, 1) k_gemm64(const TA *A, int lda, const T
           hi[j][q] += ((long long)__float2int_rn(acc[0][j][q]) << 16) + ((long long)__float2int_rn(acc[1][j][q]) << 8) +
                       __float2int_rn(acc[2][j][q]);
           lo[j][q] += ((long long)__float2int_rn(acc[3][j][q]) << 24) + ((long long)__float2int_rn(acc[4][j][q]) << 16) +
-                      ((long long)__float2int_rn(acc[5][j][q]) << 8) + __float2int_rn(acc[6][j][q]);
+                      ((long long)__float2int_rn(acc[5][j][q]) << 8) + __float2int_rn(acc[6][j][q]) +
+                      ((__float2int_rn(acc[7][j][q]) + 128) >> 8);
 #pragma unroll
-          for (int s = 0; s < kG64Dig; ++s) acc[s][j][q] = 0.f;
+          for (int s = 0; s < kG64Ord; ++s) acc[s][j][q] = 0.f;
         }
     }
   }
