@@ -872,7 +872,7 @@ def billion_main(args):
         some kinds), and the roofline of the two dense contractions: BF16
         [Q; Y] = [U; X] Phi, algorithmic 2 (n_t + B) D K flop (Q is needed for
         the n_t touched words only), and [X; U_t]^T [Z; Zc], 2 (B + n_t) D K;
-        FP32, by word, Q = U_t Phi and G = U_t^T (B + Zc), 2 n_t D K each."""
+        FP32, by word, Q = U_t Phi and G = U_t^T B, 2 n_t D K each."""
         n = min(chunk, args.billion_docs)
         c = gen.generate(0, n, out=buf)
         offs = list(range(0, n, B)) + [n]
