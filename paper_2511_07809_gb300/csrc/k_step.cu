@@ -226,9 +226,11 @@ __device__ __forceinline__ void add_rows(const NzChunk &c, int q, const float *U
 // x_d = sum_m f_dm u_m (FP32) four U rows in flight at a time, adds c_m to this
 // block's copy and the block's share of S3.  TC=true writes X in BF16 row-major
 // (X16), whole rows, else in FP32.  The first `touch` blocks (FP32 only) find the
-// batch's touched words meanwhile: the product after this kernel reads them.
+// batch's touched words meanwhile: the product after this kernel reads them.  Up
+// to 128 features two blocks an SM are asked for: without that the compiler takes
+// 40 registers and spills, 2 to 3 us a step.
 template <int NV, bool TC>
-__global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a, int touch) {
+__global__ void __launch_bounds__(32 * kDocsPerBlock, NV == 1 ? 2 : 0) k_scan_whiten(StepArgs a, int touch) {
   const BatchDesc b = a.st->cur;
   if constexpr (!TC)
     if ((int)blockIdx.x < touch) return touch_words<32 * kDocsPerBlock>(a, b, &a.st->n_touched, blockIdx.x, touch);
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a, 
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
   __syncthreads();
-  int *cnt = a.cnt + (long long)(block % copies(a, b.n_docs)) * a.V;
+  const int copy = (block & (copies(a, b.n_docs) - 1)) * a.V;  // this block's counts start there
   float4 acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = f4(0.f);
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(32 * kDocsPerBlock) k_scan_whiten(StepArgs a, 
         if (__any_sync(0xffffffffu, c.bad)) bad = true;
         prev = __shfl_sync(0xffffffffu, c.in ? c.m : -1, c.n - 1);
         lsum += c.f;
-        if (a.same_token && c.f > 0) atomicAdd(cnt + c.m, c.f);
+        if (a.same_token && c.f > 0) atomicAdd(a.cnt + (copy + c.m), c.f);
         for (int q = 0; q < c.n; q += 4) add_rows<NV>(c, q, a.U32, a.Dp, a.Dp, lane, acc);
       }
     }
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(256) k_rz(StepArgs a) {
                                          : f4(0.f);
     r[v] = f4(0.f);
   }
-  float *H = a.H32 + (long long)(blockIdx.x % copies(a, b.n_docs)) * a.V * a.Kp;
+  float *H = a.H32 + (long long)(blockIdx.x & (copies(a, b.n_docs) - 1)) * a.V * a.Kp;
   if (a.same_token && d < b.n_docs) {
     const int lo = b.indptr[d], hi = b.indptr[d + 1];
     if (row_in_batch(b, lo, hi, b.indptr[0], b.indptr[b.n_docs])) {
@@ -936,7 +938,7 @@ __global__ void __launch_bounds__(256, NK == 1 ? 4 : 3) k_doc(StepArgs a, int R)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LW, sl = lane % LW;
   const int K4 = (a.K + 3) & ~3;  // the padding columns are zero and stay so
   float *rows = doc_rows + (long long)warp * R * K4;
-  float *B = a.H32 + (long long)(blockIdx.x % copies(a, b.n_docs)) * a.V * a.Kp;
+  float *B = a.H32 + (long long)(blockIdx.x & (copies(a, b.n_docs) - 1)) * a.V * a.Kp;
   const int first = b.indptr[0], last = b.indptr[b.n_docs];
   __shared__ unsigned long long s3;
   if (threadIdx.x == 0) s3 = 0;
@@ -1313,8 +1315,8 @@ __global__ void __launch_bounds__(256) k_reduce_update(StepArgs a) {
     unsigned before;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(&st->done) : "memory");
     if (before == gridDim.x - 1) {
-      st->n_touched = __ldcg(&st->n_touched_next);
-      st->n_touched_next = 0;
+      st->n_touched = a.touch_next ? __ldcg(&st->n_touched_next) : 0;
+      if (a.touch_next) st->n_touched_next = 0;
       st->done = 0;
       st->loss = S3 ? loss_phi - scale * loss_data : 0.0;
       st->last_S3 = S3;

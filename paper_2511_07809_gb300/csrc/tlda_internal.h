@@ -121,7 +121,7 @@ struct StepArgs {
   float *Y32;                    // Bmax x Kp
   float *Z32;                    // Bmax x Kp: Y*Y - R
   float *Zc32;                   // V x Kp: compact rows Q*(2cQ - 2H) of the touched words
-  int nrep, sms;                 // copies of H32 and cnt (a block adds to one, the reader sums them); SMs
+  int nrep, sms;                 // copies of H32 and cnt (1, 2 or 4; a block adds to one, the reader sums them); SMs
   float *H32;                    // nrep x V x Kp, zero between steps (H, or B of the FP32 form without loss)
   int *cnt;                      // nrep x V, zero between steps (c_m = sum_d f_dm)
   int *flag;                     // V, zero between steps: the word is in widx
@@ -153,6 +153,8 @@ struct StepArgs {
 // V = 1000 and K = 10: 768 uniform documents (FP32, loss) 4910 against 4980, BF16 3420
 // against 3584; 768 Zipf documents 4083 against 4093, 3160 against 3361; 2048 Zipf
 // documents 5010 against 4700, 4029 against 3500.
+// A block's copy is its index masked (they are 1, 2 or 4; a remainder by a value
+// that the compiler does not know is some 40 instructions before the first add).
 constexpr int kCopyDocs = 1024;
 __device__ inline int copies(const StepArgs &a, int n_docs) { return n_docs < kCopyDocs ? 1 : a.nrep; }
 
