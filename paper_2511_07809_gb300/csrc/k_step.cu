@@ -1081,7 +1081,8 @@ void launch_doc(const StepArgs &a, cudaStream_t s) {
 }
 
 // Rows t of B summed over the copies into the compact Zc32 (D or K above 128:
-// several blocks of k_gw_f32 read a row); k_b_clear clears them afterwards.
+// several blocks of k_gw_f32 read a row; a single copy is read where it is);
+// k_b_clear clears them afterwards.
 __global__ void __launch_bounds__(256) k_b_fold(StepArgs a) {
   const int lane = threadIdx.x & 31;
   for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < a.st->n_touched; t += gridDim.x * 8) {
@@ -1144,7 +1145,9 @@ __global__ void __launch_bounds__(BI / TM * (BN / 4)) k_gw_f32(StepArgs a, int s
           const int e = tid + i * NT, r = r0 + e / (BN / 4), c = e % (BN / 4) * 4;
           const bool in = r < re && n0 + c < a.Kp;
           const float *src = a.Zc32;
-          if (in) src = FOLD ? a.H32 + ((long long)p * a.V + a.widx[r]) * a.Kp + n0 + c : a.Zc32 + (long long)r * a.Kp + n0 + c;
+          if (in)
+            src = FOLD || a.nrep == 1 ? a.H32 + ((long long)p * a.V + a.widx[r]) * a.Kp + n0 + c
+                                      : a.Zc32 + (long long)r * a.Kp + n0 + c;
           cp16(B + p * BR * BN + e * 4, src, in);
         }
     }
@@ -1238,7 +1241,7 @@ void launch_gw_f32(const StepArgs &a, cudaStream_t s) {
   } else if (a.Dp <= 128) {
     gw_launch<128, 128, 8, true>(a, dim3(a.nsplit), s);
   } else {
-    k_b_fold<<<4 * a.sms, 256, 0, s>>>(a);
+    if (a.nrep > 1) k_b_fold<<<4 * a.sms, 256, 0, s>>>(a);
     gw_launch<128, 128, 8, false>(a, dim3(a.nsplit, (a.Dp + 127) / 128, (a.Kp + 127) / 128), s);
     k_b_clear<<<4 * a.sms, 256, 0, s>>>(a);
   }
